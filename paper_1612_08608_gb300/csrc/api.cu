@@ -1327,8 +1327,8 @@ asap_status asap_local_step(asap_ctx* c) {
       // the host, or an earlier local step of the round changed them): gather.
       time_begin(c, ASAP_KERNEL_GATHER);
       CU(launch_gather_wv(c->W[r & 1], c->ld, reinterpret_cast<const uint32_t*>(block + c->list_off[tk]),
-                          reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->wv[r & 1],
-                          c->sm_count, c->stream),
+                          reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->max_region,
+                          c->wv[r & 1], c->sm_count, c->stream),
          "launching the gather kernel");
       time_end(c);
       c->launches += 1;
@@ -1371,8 +1371,8 @@ asap_status asap_local_step(asap_ctx* c) {
       // whose owned rows must hold x - eta g before they are sent.
       time_begin(c, ASAP_KERNEL_APPLY);
       CU(launch_apply_update(c->W[r & 1], c->ld, reinterpret_cast<const uint32_t*>(block + c->list_off[tk]),
-                             reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->gsum, upd,
-                             c->sm_count, c->stream),
+                             reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->max_region,
+                             c->gsum, upd, c->sm_count, c->stream),
          "launching the local update kernel");
       time_end(c);
       c->launches += 1;

@@ -186,9 +186,9 @@ cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cud
 size_t local_step_smem_bytes(int B, int stages);
 cudaError_t local_step_configure(size_t smem);
 cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
-                                int S, const float* gsum, float scale, int sm_count, cudaStream_t s);
+                                int S, int max_region, const float* gsum, float scale, int sm_count, cudaStream_t s);
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
-                             int S, float* wv, int sm_count, cudaStream_t s);
+                             int S, int max_region, float* wv, int sm_count, cudaStream_t s);
 constexpr int kMixComputeWarps = 16;
 constexpr int kMixUpdaterWarps = 2;
 // compute warps + one TMA producer warp + the warps that apply the fused update

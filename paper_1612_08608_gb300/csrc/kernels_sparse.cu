@@ -684,32 +684,40 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
   }
 }
 
+// The two kernels below walk a step's slab-major column list with a group of
+// TPS threads per slab (a warp, or a whole CTA), four entries per thread in
+// flight.  Both are latency chains over a slab's region: list entry, then the
+// parameter it names.  A warp suffices while regions are short (hashed
+// columns: ~400 entries, and 8,192 slabs fill the chip); with skewed columns
+// the hottest slab's region paces the launch, and a CTA walks it eight times
+// faster (RCV1-shaped, N = 16, d = 47,236, a region of 8,192 entries:
+// 23.8 -> 8.4 us for the update, 22.7 -> 8.2 us for the gather).
+
 // wv[e] = W[i][s*S + cl] for every entry e of a step's column list
 // (parameters written from the host, or changed by an earlier local step of
-// the round, have no exported copy).  One warp per slab, four entries per
-// lane in flight.
+// the round, have no exported copy).
+template <int TPS>
 __global__ void __launch_bounds__(kThreads) k_gather_wv(const float* __restrict__ W, int64_t ld,
                                                        const uint32_t* __restrict__ list,
                                                        const int* __restrict__ slab_off, long long n_slabs, int S,
                                                        float* __restrict__ wv) {
   constexpr int kU = 4;
-  const int lane = threadIdx.x & 31;
-  const long long nw = static_cast<long long>(gridDim.x) * (kThreads / 32);
-  for (long long s = static_cast<long long>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5); s < n_slabs;
-       s += nw) {
+  const int t = threadIdx.x % TPS;
+  const long long ng = static_cast<long long>(gridDim.x) * (kThreads / TPS);
+  for (long long s = static_cast<long long>(blockIdx.x) * (kThreads / TPS) + threadIdx.x / TPS; s < n_slabs; s += ng) {
     const int a0 = slab_off[s], a1 = slab_off[s + 1];
     const float* Ws = W + s * S;
-    for (int e0 = a0 + lane; e0 < a1; e0 += kU * 32) {
+    for (int e0 = a0 + t; e0 < a1; e0 += kU * TPS) {
       uint32_t code[kU];
       float v[kU];
 #pragma unroll
-      for (int u = 0; u < kU; ++u) code[u] = e0 + 32 * u < a1 ? list[e0 + 32 * u] : kListPad;
+      for (int u = 0; u < kU; ++u) code[u] = e0 + TPS * u < a1 ? list[e0 + TPS * u] : kListPad;
 #pragma unroll
       for (int u = 0; u < kU; ++u)
         v[u] = code[u] != kListPad ? Ws[static_cast<int64_t>(code[u] >> 16) * ld + (code[u] & 0xffffu)] : 0.f;
 #pragma unroll
       for (int u = 0; u < kU; ++u)
-        if (code[u] != kListPad) wv[e0 + 32 * u] = v[u];
+        if (code[u] != kListPad) wv[e0 + TPS * u] = v[u];
     }
   }
 }
@@ -717,27 +725,26 @@ __global__ void __launch_bounds__(kThreads) k_gather_wv(const float* __restrict_
 // W[i][s*S + cl] -= scale * g[e] for every entry {i << 16 | cl} of a slab-major
 // column list: the update of a local step that is not the round's last (the
 // last one is applied inside the stochastic reduce).  The entries of a list
-// are distinct, so every parameter is written by one thread.  One warp per
-// slab, four entries per lane in flight.
+// are distinct, so every parameter is written by one thread.
+template <int TPS>
 __global__ void __launch_bounds__(kThreads) k_apply_update(float* __restrict__ W, int64_t ld,
                                                           const uint32_t* __restrict__ list,
                                                           const int* __restrict__ slab_off, long long n_slabs, int S,
                                                           const float* __restrict__ g, float scale) {
   constexpr int kU = 4;
-  const int lane = threadIdx.x & 31;
-  const long long nw = static_cast<long long>(gridDim.x) * (kThreads / 32);
-  for (long long s = static_cast<long long>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5); s < n_slabs;
-       s += nw) {
+  const int t = threadIdx.x % TPS;
+  const long long ng = static_cast<long long>(gridDim.x) * (kThreads / TPS);
+  for (long long s = static_cast<long long>(blockIdx.x) * (kThreads / TPS) + threadIdx.x / TPS; s < n_slabs; s += ng) {
     const int a0 = slab_off[s], a1 = slab_off[s + 1];
     float* Ws = W + s * S;
-    for (int e0 = a0 + lane; e0 < a1; e0 += kU * 32) {
+    for (int e0 = a0 + t; e0 < a1; e0 += kU * TPS) {
       uint32_t code[kU];
       float gv[kU], wv[kU];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        const bool in = e0 + 32 * u < a1;
-        code[u] = in ? list[e0 + 32 * u] : kListPad;
-        gv[u] = in ? g[e0 + 32 * u] : 0.f;
+        const bool in = e0 + TPS * u < a1;
+        code[u] = in ? list[e0 + TPS * u] : kListPad;
+        gv[u] = in ? g[e0 + TPS * u] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < kU; ++u)
@@ -752,18 +759,31 @@ __global__ void __launch_bounds__(kThreads) k_apply_update(float* __restrict__ W
 
 }  // namespace
 
-// One warp per slab; at most one wave of 8-warp CTAs.
-static int slab_warp_grid(long long n_slabs, int sm_count) {
-  const long long ctas = (n_slabs + kThreads / 32 - 1) / (kThreads / 32);
+// One CTA per slab while the CTAs of one wave cover all slabs (nothing is
+// gained by packing slabs then) or where a region is longer than a CTA's
+// four entries a thread; else one warp per slab, whose walk is a few
+// latencies long and which needs an eighth of the CTAs.
+constexpr int kWarpRegion = 4 * kThreads;
+
+static bool slab_per_cta(long long n_slabs, int max_region, int sm_count) {
+  return n_slabs <= 8LL * sm_count || max_region > kWarpRegion;
+}
+
+static int slab_grid(long long n_slabs, int sm_count, int slabs_per_cta) {
+  const long long ctas = (n_slabs + slabs_per_cta - 1) / slabs_per_cta;
   const long long cap = 8LL * sm_count;
   const long long g = ctas < cap ? ctas : cap;
   return static_cast<int>(g > 0 ? g : 1);
 }
 
 cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
-                                int S, const float* gsum, float scale, int sm_count, cudaStream_t s) {
-  k_apply_update<<<slab_warp_grid(n_slabs, sm_count), kThreads, 0, s>>>(W, ld, list, slab_off, n_slabs, S, gsum,
-                                                                        scale);
+                                int S, int max_region, const float* gsum, float scale, int sm_count, cudaStream_t s) {
+  if (slab_per_cta(n_slabs, max_region, sm_count))
+    k_apply_update<kThreads><<<slab_grid(n_slabs, sm_count, 1), kThreads, 0, s>>>(W, ld, list, slab_off, n_slabs, S,
+                                                                                  gsum, scale);
+  else
+    k_apply_update<32><<<slab_grid(n_slabs, sm_count, kThreads / 32), kThreads, 0, s>>>(W, ld, list, slab_off,
+                                                                                        n_slabs, S, gsum, scale);
   return cudaGetLastError();
 }
 
@@ -803,8 +823,12 @@ cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cud
 }
 
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
-                             int S, float* wv, int sm_count, cudaStream_t s) {
-  k_gather_wv<<<slab_warp_grid(n_slabs, sm_count), kThreads, 0, s>>>(W, ld, list, slab_off, n_slabs, S, wv);
+                             int S, int max_region, float* wv, int sm_count, cudaStream_t s) {
+  if (slab_per_cta(n_slabs, max_region, sm_count))
+    k_gather_wv<kThreads><<<slab_grid(n_slabs, sm_count, 1), kThreads, 0, s>>>(W, ld, list, slab_off, n_slabs, S, wv);
+  else
+    k_gather_wv<32><<<slab_grid(n_slabs, sm_count, kThreads / 32), kThreads, 0, s>>>(W, ld, list, slab_off, n_slabs,
+                                                                                     S, wv);
   return cudaGetLastError();
 }
 
