@@ -349,7 +349,7 @@ asap_status configure_mix_launch(asap_ctx* c, bool fused) {
     }
   c->mix_smem = mix_smem_bytes(c->N, c->tab_kp1, c->S, c->rows_pad, c->stages, region);
   if (c->mix_smem > (227u << 10)) return fail(c, ASAP_ERR_ARG, "reduce stages do not fit in shared memory");
-  CU(mix_configure(complete, fused, c->tab_kp1, shadow, c->mix_smem), "configuring the reduce kernel");
+  CU(mix_configure(complete, fused, c->tab_kp1, shadow), "configuring the reduce kernel");
   int blocks = 0;
   CU(mix_occupancy(complete, fused, c->tab_kp1, shadow, c->mix_smem, &blocks), "occupancy of the reduce kernel");
   if (blocks < 1) return fail(c, ASAP_ERR_ARG, "reduce kernel does not fit on an SM for this N");
@@ -969,7 +969,7 @@ asap_status asap_set_model(asap_ctx* c, asap_loss loss, int num_classes, int bat
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(5, smem_sm / static_cast<int64_t>(c->step_smem + 1024)));
     c->step_q = kMaxStepCluster;
     while (c->step_q > 1 && static_cast<int64_t>(c->N) * c->step_q > per_sm * c->sm_count) c->step_q >>= 1;
-    CU(local_step_configure(c->step_smem), "configuring the local-step kernel");
+    CU(local_step_configure(), "configuring the local-step kernel");
     c->permuted = false;
   } else if (loss == ASAP_LOSS_SOFTMAX) {
     c->Cq = (num_classes + 255) / 256;

@@ -184,7 +184,7 @@ asap_status build_graph_host(asap_graph_kind kind, int N, int k, uint64_t seed, 
 // Launchers (kernels_*.cu).  Each returns the cudaError_t of the launch.
 cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cudaStream_t s);
 size_t local_step_smem_bytes(int B, int stages);
-cudaError_t local_step_configure(size_t smem);
+cudaError_t local_step_configure();
 cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
                                 int S, int max_region, const float* gsum, float scale, int sm_count, cudaStream_t s);
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
@@ -197,7 +197,7 @@ cudaError_t launch_mix(const CUtensorMap& tmap, const MixArgs& a, bool complete,
                        cudaStream_t s);
 ASAP_HD size_t mix_stage_bytes(int S, int rows_pad, int max_region);
 size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_region);
-cudaError_t mix_configure(bool complete, bool fused, int kp1, bool shadow, size_t smem);
+cudaError_t mix_configure(bool complete, bool fused, int kp1, bool shadow);
 cudaError_t mix_occupancy(bool complete, bool fused, int kp1, bool shadow, size_t smem, int* blocks);
 size_t dense_smem_bytes();
 cudaError_t dense_configure();

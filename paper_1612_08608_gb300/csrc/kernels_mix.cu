@@ -829,9 +829,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
 
 template <int KP1, bool SHADOW, bool FUSED>
 struct MixKernel {
-  static cudaError_t attr(size_t smem) {
-    return cudaFuncSetAttribute(k_mix<KP1, SHADOW, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem));
+  // The limit is the function's, not a launch's: contexts of other sizes
+  // share it, so it is always the device's (227 KB).
+  static cudaError_t attr() {
+    return cudaFuncSetAttribute(k_mix<KP1, SHADOW, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
   }
   static cudaError_t occ(size_t smem, int* blocks) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_mix<KP1, SHADOW, FUSED>, kMixThreads, smem);
@@ -907,8 +908,8 @@ size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_r
   return b + 4 * static_cast<size_t>(N) * kp1;                            // weights
 }
 
-cudaError_t mix_configure(bool complete, bool fused, int kp1, bool shadow, size_t smem) {
-  return dispatch(complete, fused, kp1, shadow, [&](auto k) { return decltype(k)::attr(smem); });
+cudaError_t mix_configure(bool complete, bool fused, int kp1, bool shadow) {
+  return dispatch(complete, fused, kp1, shadow, [&](auto k) { return decltype(k)::attr(); });
 }
 
 cudaError_t mix_occupancy(bool complete, bool fused, int kp1, bool shadow, size_t smem, int* blocks) {

@@ -793,12 +793,14 @@ size_t local_step_smem_bytes(int B, int stages) {
          4 * (kWarps + 1) * b_smem + 16 + 8 * kFragRing * kWarps * 2 + 4 * kWarps + 4;
 }
 
-cudaError_t local_step_configure(size_t smem) {
+// The limit is the functions', shared by contexts of other minibatch sizes:
+// always the device's (227 KB).
+cudaError_t local_step_configure() {
   cudaError_t e = cudaFuncSetAttribute(k_local_step<ASAP_LOSS_HINGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+                                       227 << 10);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_local_step<ASAP_LOSS_LOGISTIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem));
+                              227 << 10);
 }
 
 cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cudaStream_t s) {
