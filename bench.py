@@ -59,7 +59,7 @@ SCHED = {"tau": 1, "kind": "constant", "gamma": 0.0}   # local steps per round, 
 TRAFFIC = {
     ("sparse_logistic_hashed", "reduce"): ("stochastic_reduce_sparse_logistic_hashed.txt", "kernels_mix.cu"),
     ("dense_softmax", "dense_grad"): ("dense_gemms_dense_softmax.txt", "kernels_dense.cu"),
-    ("sparse_logistic_hashed", "local_step"): ("local_step_sparse_logistic_hashed.txt", "kernels_sparse.cu"),
+    ("sparse_logistic_hashed", "local_step"): ("local_step_sparse_logistic_hashed.txt", "kernels_entry.cu"),
 }
 
 
@@ -227,9 +227,19 @@ def kernel_work(sh):
         nnz += rp[-1] - rp[0]
         touched += np.unique(sh.col[i][rp[0]:rp[-1]]).shape[0]
     nnz, touched = nnz * N / samples, touched * N / samples
-    # the fused local step reads every entry once (list position, value,
-    # row, segment slot: 12 B), the w value and writes the column sum of
-    # every distinct (worker, column) (8 B), and the labels
+    if w["name"] == "sparse_logistic_hashed":
+        # entry layout: the local step adds up one product per entry and reads
+        # a label and a length and writes r per row
+        out["local_step"] = ("GB/s", 4.0 * nnz + 10.0 * N * B, "hbm")
+        out["reduce"] = ("GB/s", 8.0 * N * ld, "hbm")
+        # local steps before the round's last: code, value and r per entry, w read and written per column; then
+        # code, value, place and w per entry, a product written
+        out["apply"] = ("GB/s", 12.0 * nnz + 8.0 * touched, "hbm")
+        out["gather"] = ("GB/s", 18.0 * nnz, "hbm")
+        return out
+    # list layout: the fused local step reads every entry once (list position,
+    # value, row, segment slot: 12 B), the w value and writes the column sum
+    # of every distinct (worker, column) (8 B), and the labels
     out["local_step"] = ("GB/s", 12.0 * nnz + 8.0 * touched + 4.0 * N * B, "hbm")
     out["reduce"] = ("GB/s", 8.0 * N * ld, "hbm")
     # local steps before the round's last: the update scatter and the next gather

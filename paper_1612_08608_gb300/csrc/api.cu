@@ -123,10 +123,19 @@ struct asap_ctx {
   std::vector<int64_t> list_len;
   int max_region = 0;               // entries of the largest slab region of any list
   int64_t max_list = 0;
-  float* wv[2] = {nullptr, nullptr};  // w at the list positions of round t's steps: wv[t & 1] (the
-                                    // reduce of round t writes wv[(t+1) & 1] while round t's step may run)
+  // entry layout (kernels_entry.cu) instead of column lists: where a block's arrays begin
+  struct EntryOffsets {
+    size_t y, len, soff, code, val, place;
+  };
+  bool entries = false;
+  std::vector<EntryOffsets> entry_off;
+  int64_t row_stride = 0;           // floats per row of the table of products
+  int row_q = 0, row_rows = 0;      // local-step CTAs per worker, rows per CTA
+  float* r_ent = nullptr;           // [N][B] r of the last local step's rows
+  float* wv[2] = {nullptr, nullptr};  // w at the list positions (entries: the products) of round t's steps: wv[t & 1]
+                                    // (the reduce of round t writes wv[(t+1) & 1] while round t's step may run)
   float* gsum = nullptr;            // column sums at the current round's list positions
-  int64_t wv_step = -1;             // global local step whose column list wv holds (-1: none)
+  int64_t wv_step = -1;             // global local step whose values wv holds (-1: none)
   // host residency: a round reads its own block and the next one
   static constexpr int kStaging = 3;
   unsigned char* staging[kStaging] = {nullptr, nullptr, nullptr};
@@ -158,9 +167,8 @@ struct asap_ctx {
   cudaStream_t read_stream = nullptr;
 
   CUtensorMap tmap[2];
-  int S = 0, rows_pad = 0, box_rows = 0, n_boxes = 0, stages = 0;
+  int S = 0, rows_pad = 0, box_rows = 0, n_boxes = 0, stages = 0, list_slots = 0;
   int s_cap = 1024;                 // upper bound on the slab width (lowered for skewed column lists)
-  bool fused_cfg = false;
   long long n_slabs = 0;
   int mix_grid = 0;
   size_t mix_smem = 0;
@@ -228,6 +236,9 @@ void free_shards(asap_ctx* c) {
   dfree(c->gsum);
   dfree(c->mpart_big);
   dfree(c->r_big);
+  dfree(c->r_ent);
+  c->entries = false;
+  c->entry_off.clear();
   for (int b = 0; b < asap_ctx::kStaging; ++b) {
     dfree(c->staging[b]);
     c->staged_round[b] = -1;
@@ -328,34 +339,40 @@ asap_status setup_dense_param_maps(asap_ctx* c) {
   return ASAP_OK;
 }
 
-asap_status configure_mix_launch(asap_ctx* c, bool fused) {
+asap_status configure_mix_launch(asap_ctx* c, int mode) {
   const bool complete = is_complete_kernel(c);
   const bool shadow = c->Wbf[0] != nullptr;
+  const bool fused = mode != kMixPlain;
   const int region = fused ? c->max_region : 0;
-  const long long key = (complete ? 1 : 0) | (shadow ? 2 : 0) | (fused ? 4 : 0) |
-                        (static_cast<long long>(c->tab_kp1) << 3) | (static_cast<long long>(region) << 12);
+  const long long key = (complete ? 1 : 0) | (shadow ? 2 : 0) | (mode << 2) |
+                        (static_cast<long long>(c->tab_kp1) << 4) | (static_cast<long long>(region) << 12);
   if (key == c->configured_key) return ASAP_OK;
   // Stages of ~32 KB slabs: three keep enough bytes in flight per SM to
   // stream at full rate; more only queue in the memory system (on GB300 the
   // reduce alone and the dense reduce run 3-10 % faster with 3 than with 5).
   // The fused reduce holds each slab longer (the update precedes the mix)
   // and wants one more.  Fewer when the footprint does not fit.
+  // On the entry layout the entries run kEntryAhead slabs ahead of the slabs.
   const int want = fused ? 4 : 3;
+  const int ahead = mode == kMixEntries ? kEntryAhead : 0;
+  auto smem_of = [&](int st) {
+    return mix_smem_bytes(c->N, c->tab_kp1, c->S, c->rows_pad, st, region, mode, ahead ? st + ahead : 0);
+  };
   c->stages = 2;
   for (int st = want; st > 2; --st)
-    if (mix_smem_bytes(c->N, c->tab_kp1, c->S, c->rows_pad, st, region) <= (220u << 10)) {
+    if (smem_of(st) <= (224u << 10)) {
       c->stages = st;
       break;
     }
-  c->mix_smem = mix_smem_bytes(c->N, c->tab_kp1, c->S, c->rows_pad, c->stages, region);
+  c->list_slots = ahead ? c->stages + ahead : 0;
+  c->mix_smem = smem_of(c->stages);
   if (c->mix_smem > (227u << 10)) return fail(c, ASAP_ERR_ARG, "reduce stages do not fit in shared memory");
-  CU(mix_configure(complete, fused, c->tab_kp1, shadow), "configuring the reduce kernel");
+  CU(mix_configure(complete, mode, c->tab_kp1, shadow), "configuring the reduce kernel");
   int blocks = 0;
-  CU(mix_occupancy(complete, fused, c->tab_kp1, shadow, c->mix_smem, &blocks), "occupancy of the reduce kernel");
+  CU(mix_occupancy(complete, mode, c->tab_kp1, shadow, c->mix_smem, &blocks), "occupancy of the reduce kernel");
   if (blocks < 1) return fail(c, ASAP_ERR_ARG, "reduce kernel does not fit on an SM for this N");
   c->mix_grid = static_cast<int>(std::min<long long>(c->n_slabs, static_cast<long long>(c->sm_count) * blocks));
   if (c->mix_grid > c->cons_cap) return fail(c, ASAP_ERR_ARG, "internal: reduce grid exceeds its scratch");
-  c->fused_cfg = fused;
   c->configured_key = key;
   return ASAP_OK;
 }
@@ -663,6 +680,268 @@ void build_batch_image(int N, int B, int64_t d, int S, long long n_slabs, int Q,
   }
 }
 
+// The entry layout of minibatch t (host only): labels and entry counts of
+// every row, the slab offsets, and per slab the entries by (worker, column,
+// row) -- code, value, place in the row.
+struct EntryImage {
+  std::vector<unsigned char> img;
+  asap_ctx::EntryOffsets off{};
+  int max_region = 0, max_run = 0;
+  const char* err = nullptr;
+};
+
+// Entries per slab and worker of minibatch t, counted into cnt[slab * N + i];
+// false with *err set for a column id outside [0, d).
+bool count_entries(int N, int B, int64_t d, int lS, int t, const int64_t* const* rowptr, const int32_t* const* col,
+                   std::vector<int32_t>& cnt, const char** err) {
+  for (int i = 0; i < N; ++i) {
+    const int64_t* rp = rowptr[i];
+    if (!rp) continue;   // a worker this context does not step (worker-sharded): no entries
+    const int64_t r0 = static_cast<int64_t>(t) * B;
+    const int32_t* c = col[i];
+    for (int64_t e = rp[r0]; e < rp[r0 + B]; ++e) {
+      if (c[e] < 0 || c[e] >= d) {
+        *err = "column id out of range [0, d)";
+        return false;
+      }
+      cnt[static_cast<size_t>(c[e] >> lS) * N + i]++;
+    }
+  }
+  return true;
+}
+
+void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int t, const int64_t* const* rowptr,
+                       const int32_t* const* col, const float* const* val, const float* const* y, EntryImage& im) {
+  const int lS = __builtin_ctz(static_cast<unsigned>(S));
+  std::vector<int32_t> at(static_cast<size_t>(n_slabs) * N, 0);
+  if (!count_entries(N, B, d, lS, t, rowptr, col, at, &im.err)) return;
+  int64_t tot = 0;
+  for (int32_t& n : at) {
+    const int32_t c = n;
+    n = static_cast<int32_t>(tot);
+    tot += c;
+  }
+  // Entries by (slab, worker), in row order so far.
+  struct Item {
+    uint32_t code;
+    float val;
+    uint16_t place;
+  };
+  std::vector<Item> items(tot);
+  for (int i = 0; i < N; ++i) {
+    const int64_t* rp = rowptr[i];
+    if (!rp) continue;
+    const int64_t r0 = static_cast<int64_t>(t) * B;
+    for (int b = 0; b < B; ++b)
+      for (int64_t e0 = rp[r0 + b], e = e0; e < rp[r0 + b + 1]; ++e) {
+        const int32_t cc = col[i][e];
+        items[at[static_cast<size_t>(cc >> lS) * N + i]++] =
+            Item{(static_cast<uint32_t>(b) << 16) | static_cast<uint32_t>(i * S + (cc & (S - 1))), val[i][e],
+                 static_cast<uint16_t>(e - e0)};
+      }
+  }
+  // Then by column, keeping that order within a column, and into regions of
+  // whole 16-byte rows of uint16.  A column's run does not cross a multiple of
+  // 32 entries of its region (the reduce adds it up within a warp): padding
+  // goes before a run that would.
+  std::vector<int32_t> soff(n_slabs + 1, 0);
+  std::vector<uint32_t> code;
+  std::vector<float> vals;
+  std::vector<uint16_t> place;
+  const size_t expect = static_cast<size_t>(tot) + tot / 32 + 8 * static_cast<size_t>(std::min<int64_t>(n_slabs, tot));
+  code.reserve(expect);
+  vals.reserve(expect);
+  place.reserve(expect);
+  auto pad_to = [&](size_t n) {
+    code.resize(n, kListPad);
+    vals.resize(n, 0.f);
+    place.resize(n, 0);
+  };
+  int32_t p0 = 0;
+  for (long long s = 0; s < n_slabs; ++s) {
+    const size_t start = code.size();
+    soff[s] = static_cast<int32_t>(start);
+    for (int i = 0; i < N; ++i) {
+      const int32_t p1 = at[static_cast<size_t>(s) * N + i];
+      std::stable_sort(items.begin() + p0, items.begin() + p1,
+                       [](const Item& u, const Item& v) { return (u.code & kEntryOff) < (v.code & kEntryOff); });
+      for (int32_t p = p0, q; p < p1; p = q) {
+        for (q = p + 1; q < p1 && ((items[q].code ^ items[p].code) & kEntryOff) == 0u;) ++q;
+        im.max_run = std::max(im.max_run, q - p);
+        if (q - p > kEntryRun) return;
+        const size_t at32 = (code.size() - start) & 31u;
+        if (at32 + static_cast<size_t>(q - p) > 32) pad_to(code.size() + 32 - at32);
+        for (int32_t j = p; j < q; ++j) {
+          code.push_back(items[j].code | (j > p ? kEntryNext : 0u) | (j + 1 < q ? kEntryMore : 0u));
+          vals.push_back(items[j].val);
+          place.push_back(items[j].place);
+        }
+      }
+      p0 = p1;
+    }
+    pad_to(start + (code.size() - start + 7) / 8 * 8);
+    im.max_region = std::max(im.max_region, static_cast<int>(code.size() - start));
+    if (code.size() >= (1ull << 31)) {
+      im.err = "column list of a minibatch too long";
+      return;
+    }
+  }
+  soff[n_slabs] = static_cast<int32_t>(code.size());
+  const size_t rows = static_cast<size_t>(N) * B;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at0 = off;
+    off = align_up(off + bytes, 16);
+    return at0;
+  };
+  im.off.y = take(4 * rows);
+  im.off.len = take(2 * rows);
+  im.off.soff = take(4 * soff.size());
+  im.off.code = take(4 * code.size());
+  im.off.val = take(4 * code.size());
+  im.off.place = take(2 * code.size());
+  im.img.assign(align_up(off, 256), 0);
+  unsigned char* base = im.img.data();
+  float* y_o = reinterpret_cast<float*>(base + im.off.y);
+  uint16_t* len_o = reinterpret_cast<uint16_t*>(base + im.off.len);
+  std::memcpy(base + im.off.soff, soff.data(), 4 * soff.size());
+  if (!code.empty()) {
+    std::memcpy(base + im.off.code, code.data(), 4 * code.size());
+    std::memcpy(base + im.off.val, vals.data(), 4 * code.size());
+    std::memcpy(base + im.off.place, place.data(), 2 * code.size());
+  }
+  for (int i = 0; i < N; ++i) {
+    const int64_t* rp = rowptr[i];
+    if (!rp) continue;   // labels and counts stay zero
+    const int64_t r0 = static_cast<int64_t>(t) * B;
+    for (int b = 0; b < B; ++b) {
+      y_o[static_cast<size_t>(i) * B + b] = y[i][r0 + b];
+      len_o[static_cast<size_t>(i) * B + b] = static_cast<uint16_t>(rp[r0 + b + 1] - rp[r0 + b]);
+    }
+  }
+}
+
+// fn(t) for every minibatch t, on up to 32 host threads.
+template <typename F>
+void for_batches(int nb, F&& fn) {
+  const unsigned nthr = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
+  std::vector<std::thread> pool;
+  for (unsigned w = 0; w < nthr && w < static_cast<unsigned>(nb); ++w)
+    pool.emplace_back([&, w]() {
+      for (int t = static_cast<int>(w); t < nb; t += static_cast<int>(nthr)) fn(t);
+    });
+  for (auto& th : pool) th.join();
+}
+
+// Copies built minibatch images into the shard pool (device or pinned host)
+// and fills block_off / block_bytes; img(t) is released as it is copied.
+template <typename Img>
+asap_status upload_blocks(asap_ctx* c, int nb, Img&& img) {
+  size_t total = 0, mb = 0;
+  c->block_off.assign(nb, 0);
+  c->block_bytes.assign(nb, 0);
+  for (int t = 0; t < nb; ++t) {
+    c->block_off[t] = total;
+    c->block_bytes[t] = img(t).size();
+    total += img(t).size();
+    mb = std::max(mb, img(t).size());
+  }
+  const bool host = c->residency == ASAP_SHARDS_HOST;
+  if (host) {
+    CU(cudaHostAlloc(&c->pool, total, cudaHostAllocDefault), "allocating pinned shard memory");
+  } else {
+    CU(cudaMalloc(&c->pool, total), "allocating device shard memory");
+  }
+  c->pool_pinned = host;
+  c->pool_bytes = total;
+  for (int t = 0; t < nb; ++t) {
+    if (host)
+      std::memcpy(c->pool + c->block_off[t], img(t).data(), img(t).size());
+    else
+      CU(cudaMemcpy(c->pool + c->block_off[t], img(t).data(), img(t).size(), cudaMemcpyHostToDevice),
+         "copying shards to the device");
+    std::vector<unsigned char>().swap(img(t));
+  }
+  if (host) {
+    c->staging_bytes = mb;
+    for (int b = 0; b < asap_ctx::kStaging; ++b) CU(cudaMalloc(&c->staging[b], mb), "allocating staging buffers");
+  }
+  return ASAP_OK;
+}
+
+// Builds and uploads the entry layout if the shards allow it (kEntryRegion,
+// kEntryRun, kEntryWaste); c->entries says whether it did.  c->nb is left to
+// the caller.
+asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, const int32_t* const* col,
+                         const float* const* val, const float* const* y) {
+  const int N = c->N, B = c->B;
+  const int lS = __builtin_ctz(static_cast<unsigned>(c->S));
+  // Longest row, most entries of a minibatch, and the longest slab region of
+  // the first one, before anything is built.
+  int64_t max_len = 0, max_nnz = 0;
+  for (int t = 0; t < nb; ++t) {
+    int64_t nnz = 0;
+    for (int i = 0; i < N; ++i) {
+      if (!rowptr[i]) continue;
+      const int64_t* rp = rowptr[i] + static_cast<int64_t>(t) * B;
+      nnz += rp[B] - rp[0];
+      for (int b = 0; b < B; ++b) max_len = std::max(max_len, rp[b + 1] - rp[b]);
+    }
+    max_nnz = std::max(max_nnz, nnz);
+  }
+  const int64_t stride = std::max<int64_t>(4, (max_len + 3) / 4 * 4);
+  const int64_t table = static_cast<int64_t>(N) * B * stride;
+  if (max_len > 65535 || table > kEntryWaste * max_nnz + 65536 || table >= (1ll << 31)) return ASAP_OK;
+  if (max_nnz > static_cast<int64_t>(kEntryRegion) * c->n_slabs) return ASAP_OK;
+  {
+    std::vector<int32_t> cnt(static_cast<size_t>(c->n_slabs) * N, 0);
+    const char* err = nullptr;
+    if (!count_entries(N, B, c->d, lS, 0, rowptr, col, cnt, &err)) return fail(c, ASAP_ERR_ARG, err);
+    for (long long s = 0; s < c->n_slabs; ++s) {
+      int64_t n = 0;
+      for (int i = 0; i < N; ++i) n += cnt[static_cast<size_t>(s) * N + i];
+      if (n > kEntryRegion) return ASAP_OK;
+    }
+  }
+  std::vector<EntryImage> built(nb);
+  for_batches(nb, [&](int t) { build_entry_image(N, B, c->d, c->S, c->n_slabs, t, rowptr, col, val, y, built[t]); });
+  int max_region = 0;
+  for (const EntryImage& im : built) {
+    if (im.err) return fail(c, ASAP_ERR_ARG, im.err);
+    if (im.max_region > kEntryRegion || im.max_run > kEntryRun) return ASAP_OK;
+    max_region = std::max(max_region, im.max_region);
+  }
+  if (mix_smem_bytes(N, std::min(c->k + 1, kMaxKp1Sparse), c->S, c->rows_pad, 2, max_region, kMixEntries,
+                     2 + kEntryAhead) >
+      (220u << 10))
+    return ASAP_OK;
+  asap_status s = upload_blocks(c, nb, [&](int t) -> std::vector<unsigned char>& { return built[t].img; });
+  if (s != ASAP_OK) return s;
+  for (const EntryImage& im : built) c->entry_off.push_back(im.off);
+  const size_t pb = 4 * static_cast<size_t>(table);
+  for (int b = 0; b < 2; ++b) {
+    CU(cudaMalloc(&c->wv[b], pb), "allocating the table of products");
+    CU(cudaMemset(c->wv[b], 0, pb), "zeroing the table of products");
+  }
+  CU(cudaMalloc(&c->r_ent, 4 * static_cast<size_t>(N) * B), "allocating the step scratch");
+  CU(cudaMemset(c->r_ent, 0, 4 * static_cast<size_t>(N) * B), "zeroing the step scratch");
+  c->row_stride = stride;
+  c->max_region = max_region;
+  c->entries = true;
+  return ASAP_OK;
+}
+
+// The entries of minibatch t in its block.
+EntryList entry_list(const asap_ctx* c, const unsigned char* block, int t) {
+  const asap_ctx::EntryOffsets& o = c->entry_off[t];
+  EntryList x;
+  x.code = reinterpret_cast<const uint32_t*>(block + o.code);
+  x.val = reinterpret_cast<const float*>(block + o.val);
+  x.place = reinterpret_cast<const uint16_t*>(block + o.place);
+  x.off = reinterpret_cast<const int*>(block + o.soff);
+  return x;
+}
+
 // eta_k of global local step k.
 float lr_at(const asap_ctx* c, int64_t k) {
   if (c->lr_kind == ASAP_LR_INVERSE) return static_cast<float>(c->lr / (1.0 + c->lr_gamma * static_cast<double>(k)));
@@ -956,7 +1235,13 @@ asap_status asap_set_model(asap_ctx* c, asap_loss loss, int num_classes, int bat
   dfree(c->RT);
   c->n_loss_part = 0;
   if (loss == ASAP_LOSS_HINGE || loss == ASAP_LOSS_LOGISTIC) {
-    c->n_loss_part = c->N;
+    // Entry layout: CTAs of kRowStepRows rows, more rows per CTA once one
+    // wave (eight CTAs per SM) is full.
+    const int64_t per_wave = 8LL * c->sm_count * kRowStepRows;
+    c->row_rows = kRowStepRows * static_cast<int>(std::max<int64_t>(
+        1, (static_cast<int64_t>(c->N) * batch + per_wave - 1) / per_wave));
+    c->row_q = (batch + c->row_rows - 1) / c->row_rows;
+    c->n_loss_part = c->N * c->row_q;
     // The local step: one cluster of Q CTAs per worker, Q as large as keeps
     // all clusters resident (at most 8, the portable size).  Two ring stages
     // keep a CTA small enough for five per SM at the usual minibatch sizes
@@ -1091,27 +1376,23 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
   c->s_cap = 1024;
   s0 = setup_mix(c);
   if (s0 != ASAP_OK) return s0;
+  s0 = load_entries(c, nb, rp_use.data(), col, val, y);
+  if (s0 != ASAP_OK) return s0;
+  c->wv_step = -1;
+  c->configured_key = -1;
+  if (c->entries) {
+    c->nb = nb;
+    return ASAP_OK;
+  }
   const int Q = c->step_q;
   // Build every minibatch's image; narrow the slabs and rebuild while a
   // slab's column list is too long for the fused reduce's shared memory.
   for (;;) {
     const int S = c->S;
-    const long long n_slabs = c->n_slabs;
-
     std::vector<BatchImage> built(nb);
-    auto build_batch = [&](int t) {
-      build_batch_image(N, B, c->d, S, n_slabs, Q, t, rp_use.data(), col, val, y, built[t]);
-    };
-    {
-      const unsigned nthr = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
-      std::vector<std::thread> pool;
-      for (unsigned w = 0; w < nthr; ++w)
-        pool.emplace_back([&, w]() {
-          for (int t = static_cast<int>(w); t < nb; t += static_cast<int>(nthr)) build_batch(t);
-        });
-      for (auto& th : pool) th.join();
-    }
-    size_t total = 0;
+    for_batches(nb, [&](int t) {
+      build_batch_image(N, B, c->d, S, c->n_slabs, Q, t, rp_use.data(), col, val, y, built[t]);
+    });
     int max_nnz = 0, max_region = 0;
     int64_t max_list = 0;
     for (int t = 0; t < nb; ++t)
@@ -1119,54 +1400,28 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
     for (int t = 0; t < nb; ++t) max_region = std::max(max_region, built[t].max_region);
     // Two stages of the fused reduce (slab + three list regions each) must fit
     // in shared memory; skewed column popularity calls for narrower slabs.
-    if (mix_smem_bytes(N, std::min(c->k + 1, kMaxKp1Sparse), S, c->rows_pad, 2, max_region) > (220u << 10)) {
+    if (mix_smem_bytes(N, std::min(c->k + 1, kMaxKp1Sparse), S, c->rows_pad, 2, max_region, kMixLists, 0) >
+        (220u << 10)) {
       if (S <= 8) return fail(c, ASAP_ERR_ARG, "a column slab's list does not fit in shared memory");
       c->s_cap = S / 2;
       asap_status sm = setup_mix(c);
       if (sm != ASAP_OK) return sm;
       continue;
     }
-    max_region = 0;
-    c->block_off.assign(nb, 0);
-    c->block_bytes.assign(nb, 0);
     c->list_off.assign(nb, 0);
     c->soff_off.assign(nb, 0);
     c->list_len.assign(nb, 0);
     std::vector<BatchDesc> desc(static_cast<size_t>(nb) * N);
     for (int t = 0; t < nb; ++t) {
-      if (built[t].err) return fail(c, ASAP_ERR_ARG, built[t].err);
-      c->block_off[t] = total;
-      c->block_bytes[t] = built[t].img.size();
       c->list_off[t] = built[t].list_off;
       c->soff_off[t] = built[t].soff_off;
       c->list_len[t] = built[t].list_len;
-      total += built[t].img.size();
       max_nnz = std::max(max_nnz, built[t].max_nnz);
-      max_region = std::max(max_region, built[t].max_region);
       max_list = std::max(max_list, built[t].list_len);
       std::copy(built[t].desc.begin(), built[t].desc.end(), desc.begin() + static_cast<size_t>(t) * N);
     }
-    if (c->residency == ASAP_SHARDS_HOST) {
-      CU(cudaHostAlloc(&c->pool, total, cudaHostAllocDefault), "allocating pinned shard memory");
-      c->pool_pinned = true;
-      size_t mb = 0;
-      for (int t = 0; t < nb; ++t) {
-        std::memcpy(c->pool + c->block_off[t], built[t].img.data(), built[t].img.size());
-        mb = std::max(mb, built[t].img.size());
-        std::vector<unsigned char>().swap(built[t].img);
-      }
-      c->staging_bytes = mb;
-      for (int b = 0; b < asap_ctx::kStaging; ++b) CU(cudaMalloc(&c->staging[b], mb), "allocating staging buffers");
-    } else {
-      CU(cudaMalloc(&c->pool, total), "allocating device shard memory");
-      c->pool_pinned = false;
-      for (int t = 0; t < nb; ++t) {
-        CU(cudaMemcpy(c->pool + c->block_off[t], built[t].img.data(), built[t].img.size(), cudaMemcpyHostToDevice),
-           "copying shards to the device");
-        std::vector<unsigned char>().swap(built[t].img);
-      }
-    }
-    c->pool_bytes = total;
+    s0 = upload_blocks(c, nb, [&](int t) -> std::vector<unsigned char>& { return built[t].img; });
+    if (s0 != ASAP_OK) return s0;
     CU(cudaMalloc(&c->d_desc, desc.size() * sizeof(BatchDesc)), "allocating batch descriptors");
     CU(cudaMemcpy(c->d_desc, desc.data(), desc.size() * sizeof(BatchDesc), cudaMemcpyHostToDevice),
        "copying batch descriptors");
@@ -1185,8 +1440,6 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
     c->max_nnz = max_nnz;
     c->max_region = max_region;
     c->max_list = max_list;
-    c->wv_step = -1;
-    c->configured_key = -1;
     return ASAP_OK;
   }
 }
@@ -1322,45 +1575,78 @@ asap_status asap_local_step(asap_ctx* c) {
     const unsigned char* block = nullptr;
     asap_status sb = block_of(c, k, &block);
     if (sb != ASAP_OK) return sb;
+    const float* wv = c->wv[r & 1];
     if (c->wv_step != k) {
       // No exported w values for this step's columns (parameters came from
       // the host, or an earlier local step of the round changed them): gather.
       time_begin(c, ASAP_KERNEL_GATHER);
-      CU(launch_gather_wv(c->W[r & 1], c->ld, reinterpret_cast<const uint32_t*>(block + c->list_off[tk]),
-                          reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->max_region,
-                          c->wv[r & 1], c->sm_count, c->stream),
-         "launching the gather kernel");
+      if (c->entries)
+        CU(launch_entry_products(c->W[r & 1], c->ld, entry_list(c, block, tk), c->n_slabs, c->S, c->max_region,
+                                 c->wv[r & 1], c->B, c->row_stride, c->sm_count, c->stream),
+           "launching the gather kernel");
+      else
+        CU(launch_gather_wv(c->W[r & 1], c->ld, reinterpret_cast<const uint32_t*>(block + c->list_off[tk]),
+                            reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->max_region,
+                            c->wv[r & 1], c->sm_count, c->stream),
+           "launching the gather kernel");
       time_end(c);
       c->launches += 1;
       c->wv_step = k;
     }
-    LocalStepArgs a;
-    a.block = block;
-    a.desc = c->d_desc + static_cast<size_t>(tk) * c->N;
-    a.wv = c->wv[r & 1];
-    a.gsum = c->gsum;
-    a.mpart_big = c->mpart_big;
-    a.r_big = c->r_big;
-    a.loss_part = c->loss_part;
-    a.ready = c->ready;
-    a.st = c->st;
-    a.worker_of = (c->permuted || c->sharded) ? c->d_worker_of : nullptr;
-    a.N = c->sharded ? c->own_n : c->N;
-    a.B = c->B;
-    a.Q = c->step_q;
-    a.stages = c->step_stages;
-    a.round = static_cast<unsigned>(r);
-    a.mscale = s_scale;
-    a.notify = last ? 1 : 0;
-    a.skip_worker = last ? c->skip_notify : -1;
+    const int* worker_of = (c->permuted || c->sharded) ? c->d_worker_of : nullptr;
+    const int n_step = c->sharded ? c->own_n : c->N;   // workers stepped
+    const int skip = last ? c->skip_notify : -1;
     if (last) {
       c->skip_notify = -1;
       asap_status sg = prepare_graph(c, r);   // upload a regenerated graph ahead of the reduce
       if (sg != ASAP_OK) return sg;
     }
-    time_begin(c, ASAP_KERNEL_LOCAL_STEP);
-    CU(launch_local_step(a, c->loss, c->step_smem, c->stream), "launching the local-step kernel");
-    time_end(c);
+    if (c->entries) {
+      const asap_ctx::EntryOffsets& o = c->entry_off[tk];
+      RowStepArgs a;
+      a.y = reinterpret_cast<const float*>(block + o.y);
+      a.len = reinterpret_cast<const uint16_t*>(block + o.len);
+      a.prod = wv;
+      a.row_stride = c->row_stride;
+      a.r = c->r_ent;
+      a.loss_part = c->loss_part;
+      a.ticket = c->ticket;
+      a.ready = c->ready;
+      a.worker_of = worker_of;
+      a.B = c->B;
+      a.Q = c->row_q;
+      a.rows = c->row_rows;
+      a.round = static_cast<unsigned>(r);
+      a.skip_worker = skip;
+      a.mscale = s_scale;
+      a.notify = last ? 1 : 0;
+      time_begin(c, ASAP_KERNEL_LOCAL_STEP);
+      CU(launch_row_step(a, c->loss, n_step, c->stream), "launching the local-step kernel");
+      time_end(c);
+    } else {
+      LocalStepArgs a;
+      a.block = block;
+      a.desc = c->d_desc + static_cast<size_t>(tk) * c->N;
+      a.wv = wv;
+      a.gsum = c->gsum;
+      a.mpart_big = c->mpart_big;
+      a.r_big = c->r_big;
+      a.loss_part = c->loss_part;
+      a.ready = c->ready;
+      a.st = c->st;
+      a.worker_of = worker_of;
+      a.N = n_step;
+      a.B = c->B;
+      a.Q = c->step_q;
+      a.stages = c->step_stages;
+      a.round = static_cast<unsigned>(r);
+      a.mscale = s_scale;
+      a.notify = last ? 1 : 0;
+      a.skip_worker = skip;
+      time_begin(c, ASAP_KERNEL_LOCAL_STEP);
+      CU(launch_local_step(a, c->loss, c->step_smem, c->stream), "launching the local-step kernel");
+      time_end(c);
+    }
     c->launches += 1;
     const float eta = lr_at(c, k);
     const float s_next = s_scale * (1.0f - eta * c->l2);
@@ -1370,10 +1656,15 @@ asap_status asap_local_step(asap_ctx* c) {
       // the round's last update itself, except in a worker-sharded context,
       // whose owned rows must hold x - eta g before they are sent.
       time_begin(c, ASAP_KERNEL_APPLY);
-      CU(launch_apply_update(c->W[r & 1], c->ld, reinterpret_cast<const uint32_t*>(block + c->list_off[tk]),
-                             reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S, c->max_region,
-                             c->gsum, upd, c->sm_count, c->stream),
-         "launching the local update kernel");
+      if (c->entries)
+        CU(launch_entry_update(c->W[r & 1], c->ld, entry_list(c, block, tk), c->n_slabs, c->S, c->max_region,
+                               c->r_ent, c->B, upd, c->sm_count, c->stream),
+           "launching the local update kernel");
+      else
+        CU(launch_apply_update(c->W[r & 1], c->ld, reinterpret_cast<const uint32_t*>(block + c->list_off[tk]),
+                               reinterpret_cast<const int*>(block + c->soff_off[tk]), c->n_slabs, c->S,
+                               c->max_region, c->gsum, upd, c->sm_count, c->stream),
+           "launching the local update kernel");
       time_end(c);
       c->launches += 1;
       if (c->residency == ASAP_SHARDS_HOST) {
@@ -1416,7 +1707,8 @@ asap_status asap_stochastic_reduce(asap_ctx* c) {
           return fail(c, ASAP_ERR_ARG, "an in-neighbour's row was not delivered this round (asap_write_rows)");
       }
   }
-  asap_status s = configure_mix_launch(c, fused);
+  const int mode = !fused ? kMixPlain : c->entries ? kMixEntries : kMixLists;
+  asap_status s = configure_mix_launch(c, mode);
   if (s != ASAP_OK) return s;
   s = prepare_graph(c, r);
   if (s != ASAP_OK) return s;
@@ -1439,6 +1731,7 @@ asap_status asap_stochastic_reduce(asap_ctx* c) {
   a.box_rows = c->box_rows;
   a.n_boxes = c->n_boxes;
   a.stages = c->stages;
+  a.list_slots = c->list_slots;
   a.n_slabs = c->n_slabs;
   if (fused) {
     const unsigned char* bt = nullptr;
@@ -1449,18 +1742,27 @@ asap_status asap_stochastic_reduce(asap_ctx* c) {
     s = block_of(c, kl + 1, &bn);
     if (s != ASAP_OK) return s;
     const int t = static_cast<int>(kl % c->nb), tn = static_cast<int>((kl + 1) % c->nb);
-    a.upd_list = reinterpret_cast<const uint32_t*>(bt + c->list_off[t]);
-    a.upd_off = reinterpret_cast<const int*>(bt + c->soff_off[t]);
-    a.gsum = c->gsum;
     a.upd_scale = c->pend_upd;
-    a.exp_list = reinterpret_cast<const uint32_t*>(bn + c->list_off[tn]);
-    a.exp_off = reinterpret_cast<const int*>(bn + c->soff_off[tn]);
-    a.wv_out = c->wv[(r + 1) & 1];
     a.max_region = c->max_region;
+    if (c->entries) {
+      a.upd = entry_list(c, bt, t);
+      a.exp = entry_list(c, bn, tn);
+      a.r = c->r_ent;
+      a.prod_out = c->wv[(r + 1) & 1];
+      a.row_stride = c->row_stride;
+      a.B = c->B;
+    } else {
+      a.upd_list = reinterpret_cast<const uint32_t*>(bt + c->list_off[t]);
+      a.upd_off = reinterpret_cast<const int*>(bt + c->soff_off[t]);
+      a.gsum = c->gsum;
+      a.exp_list = reinterpret_cast<const uint32_t*>(bn + c->list_off[tn]);
+      a.exp_off = reinterpret_cast<const int*>(bn + c->soff_off[tn]);
+      a.wv_out = c->wv[(r + 1) & 1];
+    }
   }
   a.cons_part = c->cons_part;
   a.loss_part = c->loss_part;
-  a.n_loss_part = c->step_pending ? c->n_loss_part : 0;
+  a.n_loss_part = !c->step_pending ? 0 : sparse && !c->entries ? c->N : c->n_loss_part;
   a.loss_norm = c->B > 0 ? 1.0f / (static_cast<float>(c->N) * static_cast<float>(c->B)) : 0.f;
   a.have_loss = c->step_pending ? 1 : 0;
   a.metrics_loss = c->m_loss;
@@ -1476,7 +1778,7 @@ asap_status asap_stochastic_reduce(asap_ctx* c) {
   a.own_lo = c->sharded ? c->own_lo : 0;
   a.own_n = c->sharded ? c->own_n : c->N;
   time_begin(c, ASAP_KERNEL_REDUCE);
-  CU(launch_mix(c->tmap[r & 1], a, is_complete_kernel(c), fused, c->mix_grid, c->mix_smem, c->stream),
+  CU(launch_mix(c->tmap[r & 1], a, is_complete_kernel(c), mode, c->mix_grid, c->mix_smem, c->stream),
      "launching the stochastic reduce");
   time_end(c);
   c->launches += 1;

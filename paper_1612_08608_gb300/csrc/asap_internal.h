@@ -105,6 +105,54 @@ struct LocalStepArgs {
   int notify;                  // publish NOTIFY (last local step of the round)
 };
 
+// The entry layout of a minibatch (kernels_entry.cu).  All workers' entries,
+// by column slab of the reduce, then worker, column and row; a slab's region
+// starts at a multiple of 8 entries and is padded with kListPad codes, at its
+// end and before a run of one column that would cross a multiple of 32 entries.
+struct EntryList {
+  const uint32_t* code;        // row << 16 | flags | worker * S + column in the slab
+  const float* val;
+  const uint16_t* place;       // place in the row's products
+  const int* off;              // [n_slabs + 1] slab regions
+};
+
+constexpr uint32_t kEntryOff = 0x3fffu;       // worker * S + column (a slab holds at most 16,384 parameters)
+constexpr uint32_t kEntryMore = 0x4000u;      // the next entry has the same worker and column
+constexpr uint32_t kEntryNext = 0x8000u;      // so has the entry before (set in padding too)
+
+// It is used when every slab region of every minibatch holds at most
+// kEntryRegion entries and no column of a worker's minibatch more than
+// kEntryRun: both bound the chain of the reduce's updater warps, which look
+// up an r per entry (480 entries in one pass), and a region's 10 bytes an
+// entry in every stage and 12 in the entry ring must leave the reduce its
+// shared-memory stages; a run must fit the 32 entries a warp holds.  Above, the list layout's column sums, formed
+// outside the reduce, are the better split.  The table of products is
+// rectangular, kEntryWaste bounds what padding to the longest row may cost.
+constexpr int kEntryRegion = 1024;
+constexpr int kEntryRun = 32;
+constexpr int kEntryWaste = 8;
+constexpr int kEntryAhead = 2;           // slabs by which the reduce's entry ring runs ahead of its slabs
+constexpr int kRowStepRows = 32;         // rows a local-step CTA works on at once
+
+// Arguments of the local step on the entry layout: Q CTAs per worker, `rows`
+// rows (a multiple of kRowStepRows) each.
+struct RowStepArgs {
+  const float* y;              // [N][B] labels
+  const uint16_t* len;         // [N][B] entries of each row
+  const float* prod;           // [N][B][row_stride] val * w of each entry
+  int64_t row_stride;
+  float* r;                    // [N][B]
+  float* loss_part;            // [N][Q]
+  unsigned int* ticket;        // [N] CTAs of the worker that have finished
+  unsigned int* ready;
+  const int* worker_of;        // as in LocalStepArgs
+  int B, Q, rows;
+  unsigned int round;
+  int skip_worker;
+  float mscale;
+  int notify;
+};
+
 // Arguments of the stochastic reduce.
 struct MixArgs {
   float* out;                  // next parameter buffer
@@ -131,6 +179,13 @@ struct MixArgs {
   const int* exp_off;          // [n_slabs + 1]
   float* wv_out;               // w_{t+1} at exp_list positions
   int max_region;              // entries: the largest slab region of any list
+  // entry layout (kMixEntries kernels): upd / exp replace the lists above
+  EntryList upd, exp;          // this round's minibatch, the next step's
+  int list_slots;              // ring slots of upd's regions (0 without entries)
+  const float* r;              // [N][B] r of this round's rows
+  float* prod_out;             // [N][B][row_stride] products of the next step's entries
+  int64_t row_stride;
+  int B;
   // metrics and protocol
   double* cons_part;           // scratch [gridDim.x]
   const float* loss_part;      // [n_loss_part] from the local step
@@ -190,15 +245,42 @@ cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, cons
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
                              int S, int max_region, float* wv, int sm_count, cudaStream_t s);
 constexpr int kMixComputeWarps = 16;
-constexpr int kMixUpdaterWarps = 2;
+constexpr int kMixUpdaterWarps = 3;
 // compute warps + one TMA producer warp + the warps that apply the fused update
 constexpr int kMixThreads = (kMixComputeWarps + 1 + kMixUpdaterWarps) * 32;
-cudaError_t launch_mix(const CUtensorMap& tmap, const MixArgs& a, bool complete, bool fused, int grid, size_t smem,
+// What a reduce does to a slab beside mixing it: nothing; a sparse model's
+// update and export through the column list; or through its entries.
+constexpr int kMixPlain = 0;
+constexpr int kMixLists = 1;
+constexpr int kMixEntries = 2;
+cudaError_t launch_mix(const CUtensorMap& tmap, const MixArgs& a, bool complete, int mode, int grid, size_t smem,
                        cudaStream_t s);
-ASAP_HD size_t mix_stage_bytes(int S, int rows_pad, int max_region);
-size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_region);
-cudaError_t mix_configure(bool complete, bool fused, int kp1, bool shadow);
-cudaError_t mix_occupancy(bool complete, bool fused, int kp1, bool shadow, size_t smem, int* blocks);
+ASAP_HD size_t mix_stage_bytes(int S, int rows_pad, int max_region, int mode);
+size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_region, int mode, int list_slots);
+cudaError_t mix_configure(bool complete, int mode, int kp1, bool shadow);
+cudaError_t mix_occupancy(bool complete, int mode, int kp1, bool shadow, size_t smem, int* blocks);
+cudaError_t launch_row_step(const RowStepArgs& a, int loss, int workers, cudaStream_t s);
+cudaError_t launch_entry_products(const float* W, int64_t ld, const EntryList& x, long long n_slabs, int S,
+                                  int max_region, float* prod, int B, int64_t stride, int sm_count, cudaStream_t s);
+cudaError_t launch_entry_update(float* W, int64_t ld, const EntryList& x, long long n_slabs, int S, int max_region,
+                                const float* r, int B, float scale, int sm_count, cudaStream_t s);
+
+// How the kernels that walk a step's slab regions are laid out: one CTA per
+// slab while the CTAs of one wave cover all slabs (nothing is gained by
+// packing slabs then) or where a region is longer than a CTA's four entries a
+// thread; else one warp per slab, whose walk is a few latencies long and which
+// needs an eighth of the CTAs.
+inline bool slab_per_cta(long long n_slabs, int max_region, int sm_count) {
+  return n_slabs <= 8LL * sm_count || max_region > 4 * kThreads;
+}
+
+// CTAs of such a kernel, at most one wave.
+inline int slab_grid(long long n_slabs, int sm_count, int slabs_per_cta) {
+  const long long ctas = (n_slabs + slabs_per_cta - 1) / slabs_per_cta;
+  const long long cap = 8LL * sm_count;
+  const long long g = ctas < cap ? ctas : cap;
+  return static_cast<int>(g > 0 ? g : 1);
+}
 size_t dense_smem_bytes();
 cudaError_t dense_configure();
 cudaError_t launch_dense_fwd(const CUtensorMap& tmX, const CUtensorMap& tmW, const DenseFwdArgs& f, int N,

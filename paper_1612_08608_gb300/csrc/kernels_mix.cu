@@ -15,13 +15,16 @@
 // Sparse models (FUSED): the local step left, per distinct (worker, column)
 // of the minibatch, the column sum g of r_b x_b (kernels_sparse.cu).  The
 // producer also copies the slab's part of that list (and of the next
-// round's list) into the stage; once a slab has landed two updater warps
+// round's list) into the stage; once a slab has landed the updater warps
 // apply the round's last local update to it, w -= eta / (B s) g, and release
 // it to the compute warps through a "ready" mbarrier -- so w_{t+1/2} exists
 // only in shared memory.  s is the round's L2 shrink, prod_j (1 - eta_j l2)
 // over its local steps, which also scales the mixing weights (true w =
 // s * stored w).  After mixing the compute warps export w_{t+1} at the next
-// round's columns, which is all the next margin kernel reads.
+// round's columns, which is all the next margin kernel reads.  On the entry
+// layout (kMixEntries, kernels_entry.cu) the updaters form each column's sum
+// of r * value themselves (update_entries), and the export is value * w_{t+1}
+// of every entry of the next step.
 //
 // Consensus error per column: with K the column's value in row 0 (a shift
 // against cancellation), sum_i (w_i - wbar)^2 = sum_i (w_i - K)^2 -
@@ -75,6 +78,22 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
 
 __device__ __forceinline__ void st_release_u32(unsigned int* p, unsigned int v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
+}
+
+// 4-byte asynchronous copy global -> shared.
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(src))
+               : "memory");
+}
+
+__device__ __forceinline__ int ld_acquire_cta(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_release_cta(int* p, int v) {
+  asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" :: "r"(smem_u32(p)), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -271,10 +290,16 @@ struct MixSmem {
   uint64_t* ready;   // FUSED: the producer has applied the slab's update
   float4* part;      // [stages][warps][nq]: per-warp column sums (consensus / complete-graph mean)
   int* info;         // [stages][4]: n_upd, n_exp, exp_base
+  // entry layout: ring of a.list_slots slots of code, value and r [max_region]
+  unsigned char* lists;
+  size_t list_bytes;
+  uint64_t* lfull;
+  int* linfo;        // [list_slots]: entries of the slab
   int* nbr;
   float* wgt;
   double* dscratch;
-  int* flags;        // [0]: fail, [1]: last, [2]: failed CTAs of the launch (last CTA)
+  int* flags;        // [0]: fail, [1]: last, [2]: failed CTAs of the launch (last CTA), [3]: slabs whose NOTIFY
+                     // the producer has seen (gated reduces on the entry layout)
   unsigned* seen;    // [32]: bitmap of workers whose NOTIFY this CTA has seen (gated reduces)
 };
 
@@ -283,19 +308,26 @@ struct MixSmem {
 // Regions are formed from `raw` by pointer arithmetic (offsets only), so that
 // the compiler keeps the pointers in the shared address space and emits
 // plain shared-memory accesses.
-__device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, int kp1) {
+__device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, int kp1, int mode) {
   MixSmem m;
   auto a16 = [](size_t v) { return (v + 15) & ~static_cast<size_t>(15); };
   size_t off = (1024u - (smem_u32(raw) & 1023u)) & 1023u;   // 1024-byte aligned stages
-  m.stage_bytes = mix_stage_bytes(a.S, a.rows_pad, a.max_region);
+  m.stage_bytes = mix_stage_bytes(a.S, a.rows_pad, a.max_region, mode);
   m.stage0 = raw + off;
   off += m.stage_bytes * a.stages;
+  m.lists = raw + off;
+  m.list_bytes = 12 * static_cast<size_t>(a.max_region);
+  off = (off + m.list_bytes * a.list_slots + 15) & ~static_cast<size_t>(15);
   m.full = reinterpret_cast<uint64_t*>(raw + off);
   off += 8 * a.stages;
   m.empty = reinterpret_cast<uint64_t*>(raw + off);
   off += 8 * a.stages;
   m.ready = reinterpret_cast<uint64_t*>(raw + off);
-  off = a16(off + 8 * a.stages);
+  off += 8 * a.stages;
+  m.lfull = reinterpret_cast<uint64_t*>(raw + off);
+  off += 8 * a.list_slots;
+  m.linfo = reinterpret_cast<int*>(raw + off);
+  off = a16(off + 4 * a.list_slots);
   m.dscratch = reinterpret_cast<double*>(raw + off);
   off = a16(off + 16 * (kMixThreads / 32));
   m.flags = reinterpret_cast<int*>(raw + off);
@@ -312,17 +344,143 @@ __device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, i
   return m;
 }
 
+// The updater warps' walk on the entry layout: once a slab has landed, w -=
+// upd_scale * sum of r * value at every column of this round's entries.  Its
+// pace is a chain of shared-memory accesses, a few hundred cycles each while
+// the compute warps keep that pipe two thirds busy, so the chain is kept short:
+// the entries run ahead of the slabs in a ring of their own; a thread keeps
+// its entries' codes in registers and fetches the r they name (4-byte
+// cp.async from L2) kAhead slabs early; a landed slab costs it one round of
+// loads (w, value, r) and one of stores.  A column's entries lie in one
+// 32-entry group, so its run is added up by shuffles, in row order, into the
+// lane of its first entry, the column's only writer.  Hashed workload (N =
+// 64, d = 2^20, ~400 entries a slab, 1.6 us a slab streamed): codes and r looked
+// up in the landed slab 167 us a reduce; r early, runs read in a loop 144; so,
+// 140 us (129 us with the update left out).  In a gated reduce r is read only after the NOTIFY of its worker:
+// early for slabs the producer has passed (sm.flags[3]), else in the landed
+// slab.
+__device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs& a, int n_slabs, bool gated, int lS,
+                                               int lqb, int box_col, bool& failed) {
+  constexpr int kUpd = kMixUpdaterWarps * 32, kU = 5, kAhead = 2;
+  const int ut = threadIdx.x - kUpdater0 * 32, lane = threadIdx.x & 31;
+  const int S = 1 << lS, QB = 1 << lqb;
+  auto r_at = [&](uint32_t c) { return a.r + static_cast<int64_t>((c & kEntryOff) >> lS) * a.B + (c >> 16); };
+  int fsl = 0, sl = 0, st = 0;         // ring positions: entries being fetched, entries and stage being used
+  uint32_t fph = 0, ph = 0;            // and phases
+  uint32_t early = 0;                  // bit d: r of the slab d ahead is on its way
+  uint32_t code[kAhead + 1][kU];       // this thread's first kU entries of the slab d ahead
+  // Entries of slab it into code[d], their r on the way; false if they never came.
+  auto fetch = [&](int it, int d) {
+    uint32_t (&c)[kU] = code[d];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) c[u] = kListPad;
+    if (it >= n_slabs) return true;
+    if (!__all_sync(kFull, mbar_wait_bounded(sm.lfull + fsl, fph))) return false;
+    const uint32_t* list = reinterpret_cast<const uint32_t*>(sm.lists + fsl * sm.list_bytes);
+    float* r = reinterpret_cast<float*>(sm.lists + fsl * sm.list_bytes) + 2 * a.max_region;
+    const int n = sm.linfo[fsl];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (ut + u * kUpd < n) c[u] = list[ut + u * kUpd];
+    if (!gated || __all_sync(kFull, ld_acquire_cta(sm.flags + 3) > it)) {
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (c[u] != kListPad) cp_async4(r + ut + u * kUpd, r_at(c[u]));
+      for (int e = ut + kU * kUpd; e < n; e += kUpd)
+        if (list[e] != kListPad) cp_async4(r + e, r_at(list[e]));
+      early |= 1u << d;
+    }
+    if (++fsl == a.list_slots) {
+      fsl = 0;
+      fph ^= 1u;
+    }
+    return true;
+  };
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < kAhead; ++d) {
+    ok = ok && fetch(d, d);
+    asm volatile("cp.async.commit_group;" ::: "memory");   // one group per slab, empty ones included
+  }
+  for (int it = 0; it < n_slabs && ok; ++it) {
+    ok = __all_sync(kFull, mbar_wait_bounded(sm.full + st, ph));
+    if (!ok) break;
+    asm volatile("cp.async.wait_group %0;" :: "n"(kAhead - 1) : "memory");   // all but the slabs after this one
+    float* x = reinterpret_cast<float*>(sm.stage0 + st * sm.stage_bytes);
+    const uint32_t* list = reinterpret_cast<const uint32_t*>(sm.lists + sl * sm.list_bytes);
+    const float* val = reinterpret_cast<const float*>(list) + a.max_region;
+    const float* r = val + a.max_region;
+    const bool have_r = early & 1u;
+    const int n = sm.linfo[sl];
+    for (int e0 = ut; e0 - lane < n; e0 += kU * kUpd) {    // one turn unless the region is longer than kU * kUpd
+      uint32_t c[kU];
+      float g[kU], w[kU];
+      int off[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int e = e0 + u * kUpd;
+        c[u] = e0 == ut ? code[0][u] : e < n ? list[e] : kListPad;
+        const int i = static_cast<int>((c[u] & kEntryOff) >> lS), cl = static_cast<int>(c[u]) & (S - 1), q = cl >> 2;
+        off[u] = 4 * ((i << lqb) + (q >> lqb) * box_col + (q & (QB - 1))) + (cl & 3);
+        g[u] = 0.f;
+        w[u] = 0.f;
+        if (c[u] != kListPad) g[u] = (have_r ? r[e] : __ldcg(r_at(c[u]))) * val[e];
+        if ((c[u] & kEntryNext) == 0u) w[u] = x[off[u]];
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        // add the run's later products: step d brings that of the entry d on
+        // while the run (kEntryMore up to there) reaches it
+        float sum = g[u];
+        uint32_t more = c[u] == kListPad ? 0u : c[u] & kEntryMore;
+        for (int d = 1; __any_sync(kFull, more != 0u); ++d) {
+          const float gd = __shfl_down_sync(kFull, g[u], d);
+          const uint32_t cd = __shfl_down_sync(kFull, c[u], d);
+          if (more) {
+            sum += gd;
+            more = cd & kEntryMore;
+          }
+        }
+        if ((c[u] & kEntryNext) == 0u) x[off[u]] = fmaf(-a.upd_scale, sum, w[u]);
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before this stage's next TMA
+    __syncwarp();
+    if (lane == 0) mbar_arrive(sm.ready + st);
+    if (++sl == a.list_slots) sl = 0;
+    if (++st == a.stages) {
+      st = 0;
+      ph ^= 1u;
+    }
+    ok = fetch(it + kAhead, kAhead);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    early >>= 1;
+#pragma unroll
+    for (int d = 0; d < kAhead; ++d)
+#pragma unroll
+      for (int u = 0; u < kU; ++u) code[d][u] = code[d + 1][u];
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (!ok) {
+    if (lane == 0) record_error(a.st, ASAP_ERR_CUDA, 0xfffffffdu, a.round);
+    failed = true;
+  }
+}
+
 // KP1 > 0: sparse graph with KP1 neighbours per row (compile-time);
 // KP1 == 0: sparse graph, runtime a.kp1 (<= kMaxKp1Sparse);
 // KP1 < 0: complete graph with equal weights.
-template <int KP1, bool SHADOW, bool FUSED>
+template <int KP1, bool SHADOW, int MODE>
 __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ CUtensorMap tmap, const MixArgs a) {
   extern __shared__ unsigned char smem_raw[];
+  constexpr bool FUSED = MODE != kMixPlain;
+  constexpr bool ENTRIES = MODE == kMixEntries;
   const int kp1 = KP1 > 0 ? KP1 : (KP1 == 0 ? a.kp1 : 0);
-  MixSmem sm = carve(smem_raw, a, kp1);
+  MixSmem sm = carve(smem_raw, a, kp1, MODE);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int S = a.S, nq = S >> 2;            // column quads per slab, a power of two <= 256
   const int lq = __ffs(nq) - 1;
+  const int lS = lq + 2;
   const int QB = nq < 64 ? nq : 64;           // quads per TMA box row (a box spans <= 256 columns)
   const int lqb = __ffs(QB) - 1;
   const int box_col = a.rows_pad << lqb;      // float4s per column box of a slab
@@ -331,7 +489,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   const size_t list_off = (slab_floats * 4 + 15) & ~static_cast<size_t>(15);
   const size_t list_bytes = (static_cast<size_t>(a.max_region) * 4 + 15) & ~static_cast<size_t>(15);
 
-  if (tid == 0) { sm.flags[0] = 0; sm.flags[1] = 0; }
+  if (tid == 0) { sm.flags[0] = 0; sm.flags[1] = 0; sm.flags[3] = 0; }
   if (tid < 32) sm.seen[tid] = 0u;
   __syncthreads();
   // A gated reduce (NOTIFY_ACK or ASYNC, sparse models) runs while the local
@@ -377,6 +535,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         mbar_init(sm.empty + s, kMixComputeWarps);
         mbar_init(sm.ready + s, kMixUpdaterWarps);
       }
+      for (int s = 0; s < a.list_slots; ++s) mbar_init(sm.lfull + s, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -395,12 +554,15 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // List offsets of the next 32 slabs, one slab per lane, loaded ahead so
       // that issuing a stage never waits on a global load.
       int4 offs = make_int4(0, 0, 0, 0);
+      int2 loffs = make_int2(0, 0);                   // entry ring: the same, list_slots - stages slabs ahead
       for (long long it = 0; it < n_my + a.stages; ++it) {
         if (FUSED && (it & 31) == 0 && it < n_my) {
           const long long sl = blockIdx.x + (it + lane) * stride;
           if (it + lane < n_my)
-            offs = make_int4(__ldg(a.upd_off + sl), __ldg(a.upd_off + sl + 1), __ldg(a.exp_off + sl),
-                             __ldg(a.exp_off + sl + 1));
+            offs = ENTRIES ? make_int4(__ldg(a.upd.off + sl), __ldg(a.upd.off + sl + 1), __ldg(a.exp.off + sl),
+                                       __ldg(a.exp.off + sl + 1))
+                           : make_int4(__ldg(a.upd_off + sl), __ldg(a.upd_off + sl + 1), __ldg(a.exp_off + sl),
+                                       __ldg(a.exp_off + sl + 1));
         }
         int4 o = make_int4(0, 0, 0, 0);
         if (FUSED) {
@@ -443,11 +605,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             n_read += static_cast<unsigned long long>(a.N);
             n_current += static_cast<unsigned long long>(a.N);
           } else if (nu > 0) {
-            const unsigned w0 = __ldg(a.upd_list + o.x) >> 16;
+            const uint32_t* codes = ENTRIES ? a.upd.code : a.upd_list;
+            auto worker_of = [&](uint32_t c) { return ENTRIES ? (c & kEntryOff) >> lS : c >> 16; };
+            const unsigned w0 = worker_of(__ldg(codes + o.x));
             unsigned w1 = w0;
-            for (int e = nu - 1; e >= 0 && e >= nu - 4; --e) {
-              const uint32_t c = __ldg(a.upd_list + o.x + e);
-              if (c != kListPad) { w1 = c >> 16; break; }
+            for (int e = nu - 1; e >= 0 && e >= nu - 8; --e) {   // past the region's padding
+              const uint32_t c = __ldg(codes + o.x + e);
+              if (c != kListPad) { w1 = worker_of(c); break; }
             }
             bool acquired = false;
             for (unsigned j0 = w0; j0 <= w1 && j0 < static_cast<unsigned>(a.N); j0 += 32) {
@@ -483,6 +647,31 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             if (acquired && lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
           }
         }
+        if (ENTRIES) {
+          // The entries of the slab list_slots - stages ahead: their slot is
+          // that of the slab whose stage has just come back.  (At first, also
+          // those of the slabs before.)
+          const int ahead = a.list_slots - a.stages;
+          for (long long j = it > 0 ? it + ahead : 0; j <= it + ahead && j < n_my; ++j) {
+            if ((j & 31) == 0) {
+              const long long sl = blockIdx.x + (j + lane) * stride;
+              if (j + lane < n_my) loffs = make_int2(__ldg(a.upd.off + sl), __ldg(a.upd.off + sl + 1));
+            }
+            const int u0 = __shfl_sync(kFull, loffs.x, static_cast<int>(j & 31));
+            const int n = __shfl_sync(kFull, loffs.y, static_cast<int>(j & 31)) - u0;
+            if (lane != 0) continue;
+            const int slot = static_cast<int>(j % a.list_slots);
+            unsigned char* dst = sm.lists + slot * sm.list_bytes;
+            sm.linfo[slot] = n;
+            mbar_expect_tx(sm.lfull + slot, 8u * n);
+            if (n > 0) {
+              bulk_load(dst, a.upd.code + u0, 4u * n, sm.lfull + slot);
+              bulk_load(dst + 4 * static_cast<size_t>(a.max_region), a.upd.val + u0, 4u * n, sm.lfull + slot);
+            }
+          }
+          __syncwarp();
+        }
+        if (ENTRIES && gated && it < n_my && lane == 0) st_release_cta(sm.flags + 3, static_cast<int>(it + 1));
         if (it < n_my && lane == 0) {
           const long long slab = blockIdx.x + it * stride;
           const int st = static_cast<int>(it % a.stages);
@@ -494,7 +683,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             n_upd = o.y - o.x;
             x0 = o.z;
             n_exp = o.w - o.z;
-            bytes += 8u * n_upd + 4u * n_exp;
+            bytes += ENTRIES ? 10u * n_exp : 8u * n_upd + 4u * n_exp;
           }
           int* info = sm.info + 4 * st;
           info[0] = n_upd;
@@ -507,7 +696,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             for (int b = 0; b < a.n_boxes; ++b)
               tma_load_2d(base + (static_cast<size_t>(xb) * a.rows_pad + static_cast<size_t>(b) * a.box_rows) * QB * 16,
                           &tmap, sm.full + st, static_cast<int>(slab * S + xb * QB * 4), b * a.box_rows, policy);
-          if (FUSED) {
+          if (ENTRIES) {
+            if (n_exp > 0) {
+              bulk_load(base + list_off, a.exp.code + x0, 4u * n_exp, sm.full + st);
+              bulk_load(base + list_off + list_bytes, a.exp.val + x0, 4u * n_exp, sm.full + st);
+              bulk_load(base + list_off + 2 * list_bytes, a.exp.place + x0, 2u * n_exp, sm.full + st);
+            }
+          } else if (FUSED) {
             if (n_upd > 0) {
               bulk_load(base + list_off, a.upd_list + u0, 4u * n_upd, sm.full + st);
               bulk_load(base + list_off + list_bytes, a.gsum + u0, 4u * n_upd, sm.full + st);
@@ -526,7 +721,9 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // ================= updater warps (FUSED) =================
       // Once a slab has landed, apply w -= eta/B (1 - eta l2)^-1 g to it and
       // release it to the compute warps.
-      if (FUSED) {
+      if constexpr (ENTRIES) {
+        update_entries(sm, a, static_cast<int>(n_my), gated, lS, lqb, box_col, failed);
+      } else if (FUSED) {
         const int ut = tid - kUpdater0 * 32;
         for (long long it = 0; it < n_my; ++it) {
           const int st = static_cast<int>(it % a.stages);
@@ -579,6 +776,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       const int qoff = (q_t >> lqb) * box_col + (q_t & (QB - 1));   // float4 offset of (row 0, quad q_t)
       const int rows_t = (a.N - g_t + G - 1) / G;
       auto xq = [&](int q) { return (q >> lqb) * box_col + (q & (QB - 1)); };
+      // Entry layout: value * w of the stage's export entry e, to its row.
+      auto export_product = [&](uint32_t code, int e, const unsigned char* base, float w) {
+        const float val = reinterpret_cast<const float*>(base + list_off + list_bytes)[e];
+        const int place = reinterpret_cast<const uint16_t*>(base + list_off + 2 * list_bytes)[e];
+        const int64_t row = static_cast<int64_t>((code & kEntryOff) >> lS) * a.B + (code >> 16);
+        st_f32_hint(a.prod_out + row * a.row_stride + place, val * w, keep);
+      };
       // With a compile-time neighbour count and at most kCacheRows rows per
       // thread, the neighbour offsets of the thread's rows (its quad folded
       // in) stay in registers as 16-bit pairs, and an equal weight in one
@@ -651,12 +855,16 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             }
           }
           if (FUSED) {
-            const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off + 2 * list_bytes);
+            const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off + (ENTRIES ? 0 : 2 * list_bytes));
             const int n_exp = info[1], xbase = info[2];
             const float* means = reinterpret_cast<const float*>(part);
             for (int e = tid; e < n_exp; e += kCompute) {
               const uint32_t code = xl[e];
-              if (code != kListPad) a.wv_out[xbase + e] = means[code & 0xffffu];
+              if (code == kListPad) continue;
+              if constexpr (ENTRIES)
+                export_product(code, e, base, means[code & static_cast<uint32_t>(S - 1)]);
+              else
+                a.wv_out[xbase + e] = means[code & 0xffffu];
             }
           }
           compute_bar();   // the means are read before the next slab's sums overwrite them
@@ -735,12 +943,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
           if (FUSED) {
             // w_{t+1} at the next round's columns, recomputed with the same
             // operations in the same order as the stored outputs.
-            const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off + 2 * list_bytes);
+            const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off + (ENTRIES ? 0 : 2 * list_bytes));
             const int n_exp = info[1], xbase = info[2];
             for (int e = tid; e < n_exp; e += kCompute) {
               const uint32_t code = xl[e];
               if (code == kListPad) continue;
-              const int i = static_cast<int>(code >> 16), cl = static_cast<int>(code & 0xffffu);
+              const int i = static_cast<int>(ENTRIES ? (code & kEntryOff) >> lS : code >> 16);
+              const int cl = static_cast<int>(ENTRIES ? code & static_cast<uint32_t>(S - 1) : code & 0xffffu);
               const int* nb = sm.nbr + i * kp1;
               const float* wt = sm.wgt + i * kp1;
               const int xo = xq(cl >> 2), comp = cl & 3;
@@ -750,7 +959,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
                 if (KP1 == 0 && m >= kp1) break;
                 v = fmaf(uni ? wu : wt[m], x[4 * (nb[m] + xo) + comp], v);
               }
-              st_f32_hint(a.wv_out + xbase + e, v, keep);
+              if constexpr (ENTRIES) export_product(code, e, base, v);
+              else st_f32_hint(a.wv_out + xbase + e, v, keep);
             }
           }
         }
@@ -827,15 +1037,15 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   }
 }
 
-template <int KP1, bool SHADOW, bool FUSED>
+template <int KP1, bool SHADOW, int MODE>
 struct MixKernel {
   // The limit is the function's, not a launch's: contexts of other sizes
   // share it, so it is always the device's (227 KB).
   static cudaError_t attr() {
-    return cudaFuncSetAttribute(k_mix<KP1, SHADOW, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
+    return cudaFuncSetAttribute(k_mix<KP1, SHADOW, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
   }
   static cudaError_t occ(size_t smem, int* blocks) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_mix<KP1, SHADOW, FUSED>, kMixThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_mix<KP1, SHADOW, MODE>, kMixThreads, smem);
   }
   static cudaError_t launch(const CUtensorMap& tmap, const MixArgs& a, int grid, size_t smem, cudaStream_t s) {
     // A programmatic dependent of the local step's last kernel.
@@ -849,34 +1059,37 @@ struct MixKernel {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_mix<KP1, SHADOW, FUSED>, tmap, a);
+    return cudaLaunchKernelEx(&cfg, k_mix<KP1, SHADOW, MODE>, tmap, a);
   }
 };
 
-// Dispatch over (complete / k+1, shadow, fused); Op is a functor template.
-template <template <int, bool, bool> class K, bool SHADOW, bool FUSED>
+// Dispatch over (complete / k+1, shadow, mode); K is a functor template.
+template <template <int, bool, int> class K, bool SHADOW, int MODE>
 struct ByKp1 {
   template <typename F>
   static cudaError_t go(bool complete, int kp1, F&& f) {
-    if (complete) return f(K<-1, SHADOW, FUSED>());
+    if (complete) return f(K<-1, SHADOW, MODE>());
     switch (kp1) {
-      case 1: return f(K<1, SHADOW, FUSED>());
-      case 2: return f(K<2, SHADOW, FUSED>());
-      case 3: return f(K<3, SHADOW, FUSED>());
-      case 5: return f(K<5, SHADOW, FUSED>());
-      default: return f(K<0, SHADOW, FUSED>());
+      case 1: return f(K<1, SHADOW, MODE>());
+      case 2: return f(K<2, SHADOW, MODE>());
+      case 3: return f(K<3, SHADOW, MODE>());
+      case 5: return f(K<5, SHADOW, MODE>());
+      default: return f(K<0, SHADOW, MODE>());
     }
   }
 };
 
 template <typename F>
-cudaError_t dispatch(bool complete, bool fused, int kp1, bool shadow, F&& f) {
+cudaError_t dispatch(bool complete, int mode, int kp1, bool shadow, F&& f) {
   if (shadow) {
-    if (fused) return cudaErrorInvalidValue;   // dense models never fuse a sparse update
-    return ByKp1<MixKernel, true, false>::go(complete, kp1, f);
+    if (mode != kMixPlain) return cudaErrorInvalidValue;   // dense models never fuse a sparse update
+    return ByKp1<MixKernel, true, kMixPlain>::go(complete, kp1, f);
   }
-  return fused ? ByKp1<MixKernel, false, true>::go(complete, kp1, f)
-               : ByKp1<MixKernel, false, false>::go(complete, kp1, f);
+  switch (mode) {
+    case kMixLists: return ByKp1<MixKernel, false, kMixLists>::go(complete, kp1, f);
+    case kMixEntries: return ByKp1<MixKernel, false, kMixEntries>::go(complete, kp1, f);
+    default: return ByKp1<MixKernel, false, kMixPlain>::go(complete, kp1, f);
+  }
 }
 
 __global__ void k_cast_bf16(const float* __restrict__ src, uint16_t* __restrict__ dst, int64_t n) {
@@ -889,16 +1102,20 @@ __global__ void k_cast_bf16(const float* __restrict__ src, uint16_t* __restrict_
 
 }  // namespace
 
-ASAP_HD size_t mix_stage_bytes(int S, int rows_pad, int max_region) {
+ASAP_HD size_t mix_stage_bytes(int S, int rows_pad, int max_region, int mode) {
   const size_t slab = (static_cast<size_t>(rows_pad) * S * 4 + 15) & ~static_cast<size_t>(15);
   const size_t list = (static_cast<size_t>(max_region) * 4 + 15) & ~static_cast<size_t>(15);
-  return (slab + 3 * list + 1023) & ~static_cast<size_t>(1023);
+  // lists: update codes and sums, export codes; entries: the export's codes,
+  // values and places
+  const size_t lists = mode == kMixEntries ? 2 * list + ((list / 2 + 15) & ~static_cast<size_t>(15)) : 3 * list;
+  return (slab + lists + 1023) & ~static_cast<size_t>(1023);
 }
 
-size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_region) {
+size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_region, int mode, int list_slots) {
   auto a16 = [](size_t v) { return (v + 15) & ~static_cast<size_t>(15); };
-  size_t b = 1024 + mix_stage_bytes(S, rows_pad, max_region) * stages;   // alignment slack + stages
-  b = a16(b + 24 * static_cast<size_t>(stages));                         // full / empty / ready
+  size_t b = 1024 + mix_stage_bytes(S, rows_pad, max_region, mode) * stages;   // alignment slack + stages
+  b = a16(b + 12 * static_cast<size_t>(max_region) * list_slots);        // entry ring
+  b = a16(b + 24 * static_cast<size_t>(stages) + 12 * static_cast<size_t>(list_slots));   // mbarriers, entry counts
   b = a16(b + 16 * (kMixThreads / 32));                                   // block-sum scratch (two fp32 pairs a warp)
   b = a16(b + 16);                                                        // flags
   b = a16(b + 4 * 32);                                                    // NOTIFY bitmap
@@ -908,17 +1125,17 @@ size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_r
   return b + 4 * static_cast<size_t>(N) * kp1;                            // weights
 }
 
-cudaError_t mix_configure(bool complete, bool fused, int kp1, bool shadow) {
-  return dispatch(complete, fused, kp1, shadow, [&](auto k) { return decltype(k)::attr(); });
+cudaError_t mix_configure(bool complete, int mode, int kp1, bool shadow) {
+  return dispatch(complete, mode, kp1, shadow, [&](auto k) { return decltype(k)::attr(); });
 }
 
-cudaError_t mix_occupancy(bool complete, bool fused, int kp1, bool shadow, size_t smem, int* blocks) {
-  return dispatch(complete, fused, kp1, shadow, [&](auto k) { return decltype(k)::occ(smem, blocks); });
+cudaError_t mix_occupancy(bool complete, int mode, int kp1, bool shadow, size_t smem, int* blocks) {
+  return dispatch(complete, mode, kp1, shadow, [&](auto k) { return decltype(k)::occ(smem, blocks); });
 }
 
-cudaError_t launch_mix(const CUtensorMap& tmap, const MixArgs& a, bool complete, bool fused, int grid, size_t smem,
+cudaError_t launch_mix(const CUtensorMap& tmap, const MixArgs& a, bool complete, int mode, int grid, size_t smem,
                        cudaStream_t s) {
-  return dispatch(complete, fused, a.kp1, a.shadow != nullptr,
+  return dispatch(complete, mode, a.kp1, a.shadow != nullptr,
                   [&](auto k) { return decltype(k)::launch(tmap, a, grid, smem, s); });
 }
 

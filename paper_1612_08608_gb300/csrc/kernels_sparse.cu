@@ -759,23 +759,6 @@ __global__ void __launch_bounds__(kThreads) k_apply_update(float* __restrict__ W
 
 }  // namespace
 
-// One CTA per slab while the CTAs of one wave cover all slabs (nothing is
-// gained by packing slabs then) or where a region is longer than a CTA's
-// four entries a thread; else one warp per slab, whose walk is a few
-// latencies long and which needs an eighth of the CTAs.
-constexpr int kWarpRegion = 4 * kThreads;
-
-static bool slab_per_cta(long long n_slabs, int max_region, int sm_count) {
-  return n_slabs <= 8LL * sm_count || max_region > kWarpRegion;
-}
-
-static int slab_grid(long long n_slabs, int sm_count, int slabs_per_cta) {
-  const long long ctas = (n_slabs + slabs_per_cta - 1) / slabs_per_cta;
-  const long long cap = 8LL * sm_count;
-  const long long g = ctas < cap ? ctas : cap;
-  return static_cast<int>(g > 0 ? g : 1);
-}
-
 cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
                                 int S, int max_region, const float* gsum, float scale, int sm_count, cudaStream_t s) {
   if (slab_per_cta(n_slabs, max_region, sm_count))

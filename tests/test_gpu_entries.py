@@ -1,0 +1,136 @@
+"""GPU parity of the entry layout (columns spread evenly over the reduce's
+slabs: products exported by the reduce, row sums, updates from the rows' r
+inside the reduce) against the oracle, round by round (1e-5 normwise per
+worker), at the edges of its row passes, runs and regions, and on both sides
+of the rule that chooses it.  Which layout a context uses shows in the bytes of
+a minibatch block: 10 an entry (plus padding) against 16."""
+import numpy as np
+import pytest
+
+from oracle import rounds
+from paper_1612_08608_gb300 import inputs
+from parity import sparse_round_matching
+
+pytestmark = pytest.mark.gpu
+
+
+def _uses_entries(ctx, sh, B):
+    E = sum(int(sh.rowptr[i][B]) for i in range(sh.N))
+    return ctx.shard_block_bytes(0) < 13 * E + 6 * sh.N * B + 512
+
+
+def _make(sh, N, k, kind, loss, B, lr, l2=0.0, tau=1, residency="device", sync="bsp", regen=False):
+    from paper_1612_08608_gb300 import Context
+    ctx = Context(N, sh.d, graph_seed=7, k=k)
+    ctx.set_model(loss, batch=B, lr=lr, l2=l2)
+    ctx.set_graph(kind, regenerate=regen)
+    ctx.set_schedule(local_steps=tau)
+    ctx.set_shard_residency(residency)
+    ctx.set_sync_mode(sync)
+    ctx.load_shards(sh)
+    return ctx
+
+
+def _check(ctx, sh, T, B, loss, lr, sched, l2=0.0, tau=1, W0=None):
+    if W0 is not None:
+        ctx.write_params(W0, 0)
+    W_t, _ = ctx.read_params()
+    for t in range(T):
+        ctx.round(1)
+        W_n, _ = ctx.read_params()
+        nbr, wgt = sched(t)
+        err, lref, cref = sparse_round_matching(W_t.astype(np.float64), W_n, sh, t, B, loss, lr, nbr, wgt, 1e-5,
+                                                l2=l2, tau=tau)
+        assert err <= 1e-5, (t, err)
+        lg, cg = ctx.read_metrics(t, 1)
+        assert abs(lg[0] - lref) <= 1e-5 * max(1.0, abs(lref)), (t, lg[0], lref)
+        assert abs(cg[0] - cref) <= 1e-4 * cref + 1e-6 * np.abs(W_n).max() * np.sqrt(W_n.size)
+        W_t = W_n
+
+
+# rows of a CTA's pass are 32: minibatches of 1, 31, 33 and 100 rows; rows of 0 to 260 entries (eight lanes
+# cover 32 places a load and 128 a pass)
+@pytest.mark.parametrize("B", [1, 31, 33, 100])
+@pytest.mark.parametrize("N,k,kind", [(1, 0, "identity"), (3, 1, "ring"), (9, 2, "root"), (7, 5, "random_regular"),
+                                      (6, 5, "complete")])
+def test_rows_and_graphs(B, N, k, kind):
+    d = 160003
+    rng = np.random.default_rng(B)
+    edge = np.array([0, 1, 3, 4, 5, 31, 32, 33, 127, 128, 129, 260])
+    # every length occurs; most rows are 100 to 260 long, so that padding to 260 wastes little
+    lengths = [np.where(rng.random(3 * B) < 0.4, rng.choice(edge, 3 * B), rng.integers(100, 261, 3 * B))
+               for _ in range(N)]
+    for ln in lengths:
+        ln[0] = 200
+    sh = inputs.sparse_custom(seed=B, N=N, d=d, rows=3 * B, lengths=lengths)
+    W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
+    with _make(sh, N, k, kind, "logistic", B, 0.5, regen=kind == "random_regular") as ctx:
+        if B >= 31:
+            assert _uses_entries(ctx, sh, B)
+        sched = rounds.graph_schedule(kind, N, k, graph_seed=7, regenerate=kind == "random_regular")
+        _check(ctx, sh, 4, B, "logistic", 0.5, sched, W0=W0)
+
+
+@pytest.mark.parametrize("residency", ["device", "host"])
+@pytest.mark.parametrize("sync", ["bsp", "notify_ack"])
+def test_local_steps_l2_and_residency(residency, sync):
+    N, d, B, tau = 10, 30011, 48, 3
+    sh = inputs.sparse_custom(seed=2, N=N, d=d, rows=7 * B, max_len=40)
+    sched = rounds.graph_schedule("random_regular", N, 3, graph_seed=7, regenerate=True)
+    with _make(sh, N, 3, "random_regular", "hinge", B, 0.4, l2=0.02, tau=tau, residency=residency, sync=sync,
+               regen=True) as ctx:
+        assert _uses_entries(ctx, sh, B)
+        _check(ctx, sh, 3, B, "hinge", 0.4, sched, l2=0.02, tau=tau)
+
+
+# The longest run a column may have is 32 entries and the longest region 1,024: on either side of both the rounds
+# match the oracle, and the layout changes where the rule says.
+@pytest.mark.parametrize("hot_rows,entries", [(1, True), (2, True), (31, True), (32, True), (33, False), (64, False)])
+def test_runs_up_to_the_rule(hot_rows, entries):
+    N, d, B = 4, 20000, 64
+    rng = np.random.default_rng(hot_rows)
+    sh = inputs.sparse_custom(seed=hot_rows, N=N, d=d, rows=2 * B, lengths=[np.full(2 * B, 12)] * N)
+    for i in range(N):
+        sh.col[i] += 1 - (sh.col[i] == d - 1)              # column 0 unused, the last kept inside
+        for t in range(2):
+            for b in rng.choice(B, hot_rows, replace=False):
+                sh.col[i][sh.rowptr[i][t * B + b]] = 0
+        for r in range(2 * B):                             # distinct within a row still
+            a, e = sh.rowptr[i][r], sh.rowptr[i][r + 1]
+            u = np.unique(sh.col[i][a:e])
+            while u.shape[0] < e - a:
+                u = np.unique(np.concatenate([u, rng.integers(1, d, 1).astype(np.int32)]))
+            sh.col[i][a:e] = u
+    with _make(sh, N, 2, "root", "logistic", B, 0.5) as ctx:
+        assert _uses_entries(ctx, sh, B) == entries
+        _check(ctx, sh, 4, B, "logistic", 0.5, rounds.graph_schedule("root", N, 2))
+
+
+@pytest.mark.parametrize("per_row,entries", [(8, True), (15, True), (16, False)])
+def test_regions_up_to_the_rule(per_row, entries):
+    # one slab of 1,024 columns (N = 8) holds 64 rows x per_row entries of worker 0, and about 20 entries of
+    # padding at 960 (before runs that would cross a multiple of 32)
+    N, d, B = 8, 1024, 64
+    ln = [np.full(2 * B, per_row)] + [np.zeros(2 * B, np.int64)] * (N - 1)
+    sh = inputs.sparse_custom(seed=per_row, N=N, d=d, rows=2 * B, lengths=ln)
+    with _make(sh, N, 1, "ring", "logistic", B, 0.5) as ctx:
+        assert _uses_entries(ctx, sh, B) == entries
+        _check(ctx, sh, 3, B, "logistic", 0.5, rounds.graph_schedule("ring", N, 1))
+
+
+def test_empty_minibatches_and_two_runs_bit_identical():
+    N, d, B = 5, 5000, 40
+    rng = np.random.default_rng(0)
+    lengths = [rng.integers(0, 12, 3 * B) for _ in range(N)]
+    for ln in lengths:
+        ln[B:2 * B] = 0
+    sh = inputs.sparse_custom(seed=9, N=N, d=d, rows=3 * B, lengths=lengths)
+    outs = []
+    for mode in ("bsp", "bsp", "notify_ack"):
+        with _make(sh, N, 1, "ring", "logistic", B, 0.5, sync=mode) as ctx:
+            assert _uses_entries(ctx, sh, B)
+            ctx.round(7)
+            outs.append((ctx.read_params()[0], ctx.read_metrics(0, 7)))
+    for W, (lm, cm) in outs[1:]:
+        assert np.array_equal(W, outs[0][0]) and np.array_equal(lm, outs[0][1][0]) and np.array_equal(cm, outs[0][1][1])
+    assert abs(outs[0][1][0][1] - np.log(2.0)) <= 1e-6    # minibatch 1 is empty: the loss of m = 0
