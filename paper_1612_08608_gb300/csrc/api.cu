@@ -347,23 +347,16 @@ asap_status configure_mix_launch(asap_ctx* c, int mode) {
   const long long key = (complete ? 1 : 0) | (shadow ? 2 : 0) | (mode << 2) |
                         (static_cast<long long>(c->tab_kp1) << 4) | (static_cast<long long>(region) << 12);
   if (key == c->configured_key) return ASAP_OK;
-  // Stages of ~32 KB slabs: three keep enough bytes in flight per SM to
-  // stream at full rate; more only queue in the memory system (on GB300 the
-  // reduce alone and the dense reduce run 3-10 % faster with 3 than with 5).
-  // The fused reduce holds each slab longer (the update precedes the mix)
-  // and wants one more.  Fewer when the footprint does not fit.
-  // On the entry layout the entries run kEntryAhead slabs ahead of the slabs.
-  const int want = fused ? 4 : 3;
+  // Four stages of ~32 KB slabs, fewer where four do not fit; two compute
+  // groups (all but the entry layout) need an even number.  On the entry
+  // layout the entries run kEntryAhead slabs ahead of the slabs.
   const int ahead = mode == kMixEntries ? kEntryAhead : 0;
   auto smem_of = [&](int st) {
     return mix_smem_bytes(c->N, c->tab_kp1, c->S, c->rows_pad, st, region, mode, ahead ? st + ahead : 0);
   };
-  c->stages = 2;
-  for (int st = want; st > 2; --st)
-    if (smem_of(st) <= (224u << 10)) {
-      c->stages = st;
-      break;
-    }
+  c->stages = 4;
+  while (c->stages > 2 && (smem_of(c->stages) > (224u << 10) || (mode != kMixEntries && c->stages % 2 != 0)))
+    --c->stages;
   c->list_slots = ahead ? c->stages + ahead : 0;
   c->mix_smem = smem_of(c->stages);
   if (c->mix_smem > (227u << 10)) return fail(c, ASAP_ERR_ARG, "reduce stages do not fit in shared memory");

@@ -124,11 +124,11 @@ constexpr uint32_t kEntryNext = 0x8000u;      // so has the entry before (set in
 // kEntryRegion entries and no column of a worker's minibatch more than
 // kEntryRun: both bound the chain of the reduce's updater warps, which look
 // up an r per entry (480 entries in one pass), and a region's 10 bytes an
-// entry in every stage and 12 in the entry ring must leave the reduce its
-// shared-memory stages; a run must fit the 32 entries a warp holds.  Above, the list layout's column sums, formed
+// entry in every stage and 12 in the entry ring must leave the reduce
+// three shared-memory stages or more; a run must fit the 32 entries a warp holds.  Above, the list layout's column sums, formed
 // outside the reduce, are the better split.  The table of products is
 // rectangular, kEntryWaste bounds what padding to the longest row may cost.
-constexpr int kEntryRegion = 1024;
+constexpr int kEntryRegion = 704;
 constexpr int kEntryRun = 32;
 constexpr int kEntryWaste = 8;
 constexpr int kEntryAhead = 2;           // slabs by which the reduce's entry ring runs ahead of its slabs

@@ -16,8 +16,8 @@
 // Against the list layout (kernels_sparse.cu), which fetches w by list
 // position, exchanges partial margins across a cluster and scans column sums,
 // the local step of hashed logistic regression (N = 64, d = 2^20, B = 512, 100
-// entries a row) went from 47 to 11.5 us and the reduce from 106 to 140 us (150
-// to 144 us a round), and a minibatch takes 10 instead of 16 bytes an entry
+// entries a row) went from 47 to 11.5 us and the reduce from 106 to 128 us (150
+// to 132 us a round), and a minibatch takes 10 instead of 16 bytes an entry
 // (250 to 160 us a round with host-resident shards, which the copy bounds).  It needs slabs with few
 // entries and columns with short runs (kEntryRegion, kEntryRun); skewed
 // columns stay with the list layout.

@@ -56,7 +56,19 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned long long kTmaWaitNs = 2000000000ull;   // 2 s: a TMA load never takes this long
-constexpr int kCompute = kMixComputeWarps * 32;            // compute threads
+// The compute warps work in groups, on alternate slabs.  A slab costs a warp a
+// chain of shared-memory accesses, a few hundred cycles each: one group of
+// sixteen warps goes through every slab's chain in step, the pipe idle at its
+// ends.  Two groups overlap two chains, and with half the threads a thread
+// has twice the rows, hence loads, in flight (N = 256, d = 10^6, k = 4: 414 ->
+// 363 us a reduce).  On the entry layout, where the stages' turnaround is the
+// bound, the shorter life of a slab in one group is worth more (hashed
+// workload: 141 us against 147 with two groups).  The number of stages is a multiple of the
+// groups, so that a stage always belongs to the same group (its warps wait for
+// every phase of the stage's barriers, which parities need).
+constexpr int mix_groups(int mode) { return mode == kMixEntries ? 1 : 2; }
+// Threads of a group: at least the 256 column quads of the widest slab.
+constexpr int mix_group_threads(int mode) { return kMixComputeWarps * 32 / mix_groups(mode); }
 constexpr int kProducerWarp = kMixComputeWarps;
 constexpr int kUpdater0 = kMixComputeWarps + 1;             // first updater warp
 
@@ -102,6 +114,12 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(bar)), "r"(bytes)
+               : "memory");
+}
+
+// Adds to the bytes the current phase waits for, without an arrival.
+__device__ __forceinline__ void mbar_expect_only(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(bar)), "r"(bytes)
                : "memory");
 }
 
@@ -271,14 +289,19 @@ __device__ __forceinline__ void block_sum2_f2(F2& u, F2& v, F2* scratch) {
   v = tv;
 }
 
-__device__ __forceinline__ void compute_bar() { asm volatile("bar.sync 1, %0;" :: "n"(kCompute) : "memory"); }
+// Barrier of a compute group.
+template <int THREADS>
+__device__ __forceinline__ void compute_bar(int group) {
+  asm volatile("bar.sync %0, %1;" :: "r"(group + 1), "n"(THREADS) : "memory");
+}
 
-// Barrier among the compute warps that also returns the OR of `v` over them.
-__device__ __forceinline__ bool compute_bar_or(bool v) {
+// Barrier of a compute group that also returns the OR of `v` over it.
+template <int THREADS>
+__device__ __forceinline__ bool compute_bar_or(int group, bool v) {
   uint32_t r;
   asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
-      : "=r"(r) : "r"(static_cast<uint32_t>(v)), "n"(kCompute) : "memory");
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, %3, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r) : "r"(static_cast<uint32_t>(v)), "n"(THREADS), "r"(group + 1) : "memory");
   return r != 0;
 }
 
@@ -288,7 +311,7 @@ struct MixSmem {
   uint64_t* full;
   uint64_t* empty;
   uint64_t* ready;   // FUSED: the producer has applied the slab's update
-  float4* part;      // [stages][warps][nq]: per-warp column sums (consensus / complete-graph mean)
+  float4* part;      // [stages][kCompute]: per-thread column sums (consensus / complete-graph mean)
   int* info;         // [stages][4]: n_upd, n_exp, exp_base
   // entry layout: ring of a.list_slots slots of code, value and r [max_region]
   unsigned char* lists;
@@ -337,7 +360,7 @@ __device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, i
   m.info = reinterpret_cast<int*>(raw + off);
   off = a16(off + 16 * a.stages);
   m.part = reinterpret_cast<float4*>(raw + off);
-  off = a16(off + 16 * static_cast<size_t>(a.stages) * kCompute);
+  off = a16(off + 16 * static_cast<size_t>(a.stages) * mix_group_threads(mode));
   m.nbr = reinterpret_cast<int*>(raw + off);
   off = a16(off + 4 * static_cast<size_t>(a.N) * kp1);
   m.wgt = reinterpret_cast<float*>(raw + off);
@@ -356,7 +379,8 @@ __device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, i
 // lane of its first entry, the column's only writer.  Hashed workload (N =
 // 64, d = 2^20, ~400 entries a slab, 1.6 us a slab streamed): codes and r looked
 // up in the landed slab 167 us a reduce; r early, runs read in a loop 144; so,
-// 140 us (129 us with the update left out).  In a gated reduce r is read only after the NOTIFY of its worker:
+// 140 us then, 128 us now that the producer issues a slab before it adds up the
+// last one's column sums.  In a gated reduce r is read only after the NOTIFY of its worker:
 // early for slabs the producer has passed (sm.flags[3]), else in the landed
 // slab.
 __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs& a, int n_slabs, bool gated, int lS,
@@ -475,6 +499,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   extern __shared__ unsigned char smem_raw[];
   constexpr bool FUSED = MODE != kMixPlain;
   constexpr bool ENTRIES = MODE == kMixEntries;
+  constexpr int kGroups = mix_groups(MODE), kCompute = mix_group_threads(MODE);
   const int kp1 = KP1 > 0 ? KP1 : (KP1 == 0 ? a.kp1 : 0);
   MixSmem sm = carve(smem_raw, a, kp1, MODE);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -532,7 +557,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     if (tid == 0) {
       for (int s = 0; s < a.stages; ++s) {
         mbar_init(sm.full + s, 1);
-        mbar_init(sm.empty + s, kMixComputeWarps);
+        mbar_init(sm.empty + s, kMixComputeWarps / kGroups);
         mbar_init(sm.ready + s, kMixUpdaterWarps);
       }
       for (int s = 0; s < a.list_slots; ++s) mbar_init(sm.lfull + s, 1);
@@ -541,7 +566,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     __syncthreads();
 
     const long long stride = gridDim.x;
-    const long long n_my = (a.n_slabs - blockIdx.x + stride - 1) / stride;   // slabs of this CTA
+    const int n_my = static_cast<int>((a.n_slabs - blockIdx.x + stride - 1) / stride);   // slabs of this CTA
     const float inv_n = 1.0f / static_cast<float>(a.N);
 
     const uint64_t policy = evict_first_policy();
@@ -555,9 +580,11 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // that issuing a stage never waits on a global load.
       int4 offs = make_int4(0, 0, 0, 0);
       int2 loffs = make_int2(0, 0);                   // entry ring: the same, list_slots - stages slabs ahead
-      for (long long it = 0; it < n_my + a.stages; ++it) {
+      int st = 0, done_st = 0;                        // stages of slab it, and of the slab that came back
+      uint32_t done_ph = 0;
+      for (int it = 0; it < n_my + a.stages; ++it) {
         if (FUSED && (it & 31) == 0 && it < n_my) {
-          const long long sl = blockIdx.x + (it + lane) * stride;
+          const long long sl = blockIdx.x + static_cast<long long>(it + lane) * stride;
           if (it + lane < n_my)
             offs = ENTRIES ? make_int4(__ldg(a.upd.off + sl), __ldg(a.upd.off + sl + 1), __ldg(a.exp.off + sl),
                                        __ldg(a.exp.off + sl + 1))
@@ -566,17 +593,14 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         }
         int4 o = make_int4(0, 0, 0, 0);
         if (FUSED) {
-          const int src = static_cast<int>(it & 31);
+          const int src = it & 31;
           o.x = __shfl_sync(kFull, offs.x, src);
           o.y = __shfl_sync(kFull, offs.y, src);
           o.z = __shfl_sync(kFull, offs.z, src);
           o.w = __shfl_sync(kFull, offs.w, src);
         }
         if (it >= a.stages) {
-          const long long done = it - a.stages;
-          const int st = static_cast<int>(done % a.stages);
-          bool ok = (lane == 0) ? mbar_wait_bounded(sm.empty + st, static_cast<uint32_t>((done / a.stages) & 1))
-                                : true;
+          bool ok = (lane == 0) ? mbar_wait_bounded(sm.empty + done_st, done_ph) : true;
           ok = __shfl_sync(kFull, ok, 0) != 0;   // warp-uniform outcome
           __syncwarp();
           if (!ok) {
@@ -584,15 +608,6 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             failed = true;
             break;
           }
-          if (KP1 >= 0) {
-            const float4* p = sm.part + static_cast<size_t>(st) * kCompute;
-            for (int q = lane; q < nq; q += 32) {
-              float4 t = p[q];
-              for (int g = 1; g < G; ++g) t = f4_add(t, p[g * nq + q]);
-              term = fmaf(fmaf(t.x, t.x, fmaf(t.y, t.y, fmaf(t.z, t.z, t.w * t.w))), inv_n_term, term);
-            }
-          }
-          __syncwarp();
         }
         if (FUSED && gated && it < n_my) {
           // The slab's updates come from workers w0 .. w1 (a region is sorted
@@ -647,34 +662,9 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             if (acquired && lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
           }
         }
-        if (ENTRIES) {
-          // The entries of the slab list_slots - stages ahead: their slot is
-          // that of the slab whose stage has just come back.  (At first, also
-          // those of the slabs before.)
-          const int ahead = a.list_slots - a.stages;
-          for (long long j = it > 0 ? it + ahead : 0; j <= it + ahead && j < n_my; ++j) {
-            if ((j & 31) == 0) {
-              const long long sl = blockIdx.x + (j + lane) * stride;
-              if (j + lane < n_my) loffs = make_int2(__ldg(a.upd.off + sl), __ldg(a.upd.off + sl + 1));
-            }
-            const int u0 = __shfl_sync(kFull, loffs.x, static_cast<int>(j & 31));
-            const int n = __shfl_sync(kFull, loffs.y, static_cast<int>(j & 31)) - u0;
-            if (lane != 0) continue;
-            const int slot = static_cast<int>(j % a.list_slots);
-            unsigned char* dst = sm.lists + slot * sm.list_bytes;
-            sm.linfo[slot] = n;
-            mbar_expect_tx(sm.lfull + slot, 8u * n);
-            if (n > 0) {
-              bulk_load(dst, a.upd.code + u0, 4u * n, sm.lfull + slot);
-              bulk_load(dst + 4 * static_cast<size_t>(a.max_region), a.upd.val + u0, 4u * n, sm.lfull + slot);
-            }
-          }
-          __syncwarp();
-        }
-        if (ENTRIES && gated && it < n_my && lane == 0) st_release_cta(sm.flags + 3, static_cast<int>(it + 1));
+        if (ENTRIES && gated && it < n_my && lane == 0) st_release_cta(sm.flags + 3, it + 1);
         if (it < n_my && lane == 0) {
           const long long slab = blockIdx.x + it * stride;
-          const int st = static_cast<int>(it % a.stages);
           unsigned char* base = sm.stage0 + st * sm.stage_bytes;
           uint32_t bytes = static_cast<uint32_t>(a.n_boxes) * a.box_rows * S * 4u;
           int n_upd = 0, n_exp = 0, x0 = 0, u0 = 0;
@@ -685,12 +675,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             n_exp = o.w - o.z;
             bytes += ENTRIES ? 10u * n_exp : 8u * n_upd + 4u * n_exp;
           }
-          int* info = sm.info + 4 * st;
-          info[0] = n_upd;
-          info[1] = n_exp;
-          info[2] = x0;
-          info[3] = u0;
-          mbar_expect_tx(sm.full + st, bytes);
+          *reinterpret_cast<int4*>(sm.info + 4 * st) = make_int4(n_upd, n_exp, x0, u0);
+          mbar_expect_only(sm.full + st, bytes);
           // Slab layout in shared memory: [column box][row][QB quads].
           for (int xb = 0; xb < nq / QB; ++xb)
             for (int b = 0; b < a.n_boxes; ++b)
@@ -710,7 +696,50 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             if (n_exp > 0) bulk_load(base + list_off + 2 * list_bytes, a.exp_list + x0, 4u * n_exp, sm.full + st);
           }
         }
+        if (ENTRIES) {
+          // The entries of the slab list_slots - stages ahead: their slot is
+          // that of the slab whose stage has just come back.  (At first, also
+          // those of the slabs before.)
+          const int ahead = a.list_slots - a.stages;
+          for (int j = it > 0 ? it + ahead : 0; j <= it + ahead && j < n_my; ++j) {
+            if ((j & 31) == 0) {
+              const long long sl = blockIdx.x + static_cast<long long>(j + lane) * stride;
+              if (j + lane < n_my) loffs = make_int2(__ldg(a.upd.off + sl), __ldg(a.upd.off + sl + 1));
+            }
+            const int u0 = __shfl_sync(kFull, loffs.x, j & 31);
+            const int n = __shfl_sync(kFull, loffs.y, j & 31) - u0;
+            if (lane != 0) continue;
+            const int slot = j % a.list_slots;
+            unsigned char* dst = sm.lists + slot * sm.list_bytes;
+            sm.linfo[slot] = n;
+            mbar_expect_tx(sm.lfull + slot, 8u * n);
+            if (n > 0) {
+              bulk_load(dst, a.upd.code + u0, 4u * n, sm.lfull + slot);
+              bulk_load(dst + 4 * static_cast<size_t>(a.max_region), a.upd.val + u0, 4u * n, sm.lfull + slot);
+            }
+          }
+          __syncwarp();
+        }
+        // The column sums of the slab that came back, while the next one's
+        // copies fly: its stage cannot be handed on before the arrival below.
+        // (Added up before the copies were issued, they lengthened every
+        // stage's turnaround by about a microsecond: the hashed workload's
+        // reduce took 141 us instead of 128.)
+        if (it >= a.stages && KP1 >= 0) {
+          const float4* p = sm.part + done_st * kCompute;
+          for (int q = lane; q < nq; q += 32) {
+            float4 t = p[q];
+            for (int g = 1; g < G; ++g) t = f4_add(t, p[g * nq + q]);
+            term = fmaf(fmaf(t.x, t.x, fmaf(t.y, t.y, fmaf(t.z, t.z, t.w * t.w))), inv_n_term, term);
+          }
+        }
         __syncwarp();
+        if (it < n_my && lane == 0) mbar_arrive(sm.full + st);
+        if (it >= a.stages && ++done_st == a.stages) {
+          done_st = 0;
+          done_ph ^= 1u;
+        }
+        if (++st == a.stages) st = 0;
       }
       s2 = -term;
       if (gated && lane == 0 && n_read) {
@@ -722,12 +751,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // Once a slab has landed, apply w -= eta/B (1 - eta l2)^-1 g to it and
       // release it to the compute warps.
       if constexpr (ENTRIES) {
-        update_entries(sm, a, static_cast<int>(n_my), gated, lS, lqb, box_col, failed);
+        update_entries(sm, a, n_my, gated, lS, lqb, box_col, failed);
       } else if (FUSED) {
         const int ut = tid - kUpdater0 * 32;
-        for (long long it = 0; it < n_my; ++it) {
-          const int st = static_cast<int>(it % a.stages);
-          const bool ok = __all_sync(kFull, mbar_wait_bounded(sm.full + st, static_cast<uint32_t>((it / a.stages) & 1)));
+        int st = 0;
+        uint32_t ph = 0;
+        for (int it = 0; it < n_my; ++it) {
+          const bool ok = __all_sync(kFull, mbar_wait_bounded(sm.full + st, ph));
           if (!ok) {
             if (lane == 0) record_error(a.st, ASAP_ERR_CUDA, 0xfffffffdu, a.round);
             failed = true;
@@ -765,13 +795,19 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before this stage's next TMA
           __syncwarp();
           if (lane == 0) mbar_arrive(sm.ready + st);
+          if (++st == a.stages) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
       }
     } else {
       // ================= compute warps =================
-      // Thread t owns column quad q = t mod nq of every slab for the rows
-      // i = g, g + G, ... (g = t / nq): with ~32 KB slabs that is 4 rows.
-      const int q_t = tid & (nq - 1), g_t = tid >> lq;
+      // Group k takes the slabs k, k + kGroups, ... of the CTA; its thread t
+      // owns column quad q = t mod nq of them for the rows i = g, g + G, ...
+      // (g = t / nq): with ~32 KB slabs that is 4 or 8 rows.
+      const int group = tid / kCompute, gt = tid - group * kCompute;
+      const int q_t = gt & (nq - 1), g_t = gt >> lq;
       const uint64_t keep = evict_last_policy();
       const int qoff = (q_t >> lqb) * box_col + (q_t & (QB - 1));   // float4 offset of (row 0, quad q_t)
       const int rows_t = (a.N - g_t + G - 1) / G;
@@ -787,7 +823,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // thread, the neighbour offsets of the thread's rows (its quad folded
       // in) stay in registers as 16-bit pairs, and an equal weight in one
       // register: the slab loop then reads only the slab from shared memory.
-      constexpr int kCacheRows = 4;
+      constexpr int kCacheRows = 4 * kGroups;   // all of a thread's rows, with 32 KB slabs
       constexpr int kC = KP1 > 0 ? KP1 : 1;
       constexpr int kPk = (kCacheRows * kC + 1) / 2;
       const bool cached = KP1 > 0 && rows_t <= kCacheRows;
@@ -806,24 +842,28 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       }
       const bool uni = a.uniform_w != 0;
       const float wu = uni && KP1 >= 0 ? sm.wgt[0] : 0.f;
-      for (long long it = 0; it < n_my; ++it) {
+      int st = group;
+      uint32_t ph = 0;
+      for (int it = group; it < n_my; it += kGroups) {
+        if (st >= a.stages) {
+          st = group;
+          ph ^= 1u;
+        }
         const long long slab = blockIdx.x + it * stride;
-        const int st = static_cast<int>(it % a.stages);
-        bool ok = __all_sync(kFull, mbar_wait_bounded(FUSED ? sm.ready + st : sm.full + st,
-                                                      static_cast<uint32_t>((it / a.stages) & 1)));
+        bool ok = __all_sync(kFull, mbar_wait_bounded(FUSED ? sm.ready + st : sm.full + st, ph));
         unsigned char* base = sm.stage0 + st * sm.stage_bytes;
         float* x = reinterpret_cast<float*>(base);
         const float4* x4 = reinterpret_cast<const float4*>(base);
         const int* info = sm.info + 4 * st;
-        float4* part = sm.part + static_cast<size_t>(st) * kCompute;
+        float4* part = sm.part + st * kCompute;
         const long long c0 = slab * S;
         if (ok && KP1 < 0) {
           // Complete graph: this thread's share of its column's sum.
           float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
           for (int r = 0; r < rows_t; ++r) cs = f4_add(cs, x4[(g_t + r * G) * QB + qoff]);
-          part[tid] = cs;
+          part[gt] = cs;
         }
-        if (KP1 < 0) ok = !compute_bar_or(!ok);   // uniform decision; the column sums are visible
+        if (KP1 < 0) ok = !compute_bar_or<kCompute>(group, !ok);   // uniform decision; the column sums are visible
         if (!ok) {
           if (lane == 0) record_error(a.st, ASAP_ERR_CUDA, 0xffffffffu, a.round);
           failed = true;
@@ -831,13 +871,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         }
         if constexpr (KP1 < 0) {
           // Complete graph: column means (threads t < nq), then every row gets them.
-          if (tid < nq) {
-            float4 t = part[tid];
-            for (int g = 1; g < G; ++g) t = f4_add(t, part[g * nq + tid]);
+          if (gt < nq) {
+            float4 t = part[gt];
+            for (int g = 1; g < G; ++g) t = f4_add(t, part[g * nq + gt]);
             const float sc = inv_n * a.wscale;
-            part[tid] = make_float4(t.x * sc, t.y * sc, t.z * sc, t.w * sc);
+            part[gt] = make_float4(t.x * sc, t.y * sc, t.z * sc, t.w * sc);
           }
-          compute_bar();
+          compute_bar<kCompute>(group);
           const float4 mean = part[q_t];
           for (int r = 0; r < rows_t; ++r) {
             const int i = g_t + r * G;
@@ -858,7 +898,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off + (ENTRIES ? 0 : 2 * list_bytes));
             const int n_exp = info[1], xbase = info[2];
             const float* means = reinterpret_cast<const float*>(part);
-            for (int e = tid; e < n_exp; e += kCompute) {
+            for (int e = gt; e < n_exp; e += kCompute) {
               const uint32_t code = xl[e];
               if (code == kListPad) continue;
               if constexpr (ENTRIES)
@@ -867,7 +907,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
                 a.wv_out[xbase + e] = means[code & 0xffffu];
             }
           }
-          compute_bar();   // the means are read before the next slab's sums overwrite them
+          compute_bar<kCompute>(group);   // the means are read before the next slab's sums overwrite them
         } else {
           const float4 K = x4[qoff];        // shift: row 0 of the (updated) slab
           float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -939,13 +979,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             if (r < rows_t) emit(g_t + r * G, mix_one(g_t + r * G));
           }
           s2 += sq;
-          part[tid] = s1;
+          part[gt] = s1;
           if (FUSED) {
             // w_{t+1} at the next round's columns, recomputed with the same
             // operations in the same order as the stored outputs.
             const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off + (ENTRIES ? 0 : 2 * list_bytes));
             const int n_exp = info[1], xbase = info[2];
-            for (int e = tid; e < n_exp; e += kCompute) {
+            for (int e = gt; e < n_exp; e += kCompute) {
               const uint32_t code = xl[e];
               if (code == kListPad) continue;
               const int i = static_cast<int>(ENTRIES ? (code & kEntryOff) >> lS : code >> 16);
@@ -966,6 +1006,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(sm.empty + st);
+        st += kGroups;
       }
     }
   }
@@ -1120,7 +1161,7 @@ size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_r
   b = a16(b + 16);                                                        // flags
   b = a16(b + 4 * 32);                                                    // NOTIFY bitmap
   b = a16(b + 16 * static_cast<size_t>(stages));                          // stage info
-  b = a16(b + 16 * static_cast<size_t>(stages) * kMixComputeWarps * 32);  // partial sums
+  b = a16(b + 16 * static_cast<size_t>(stages) * mix_group_threads(mode));   // partial sums
   b = a16(b + 4 * static_cast<size_t>(N) * kp1);                          // neighbour offsets
   return b + 4 * static_cast<size_t>(N) * kp1;                            // weights
 }

@@ -83,7 +83,7 @@ def test_local_steps_l2_and_residency(residency, sync):
         _check(ctx, sh, 3, B, "hinge", 0.4, sched, l2=0.02, tau=tau)
 
 
-# The longest run a column may have is 32 entries and the longest region 1,024: on either side of both the rounds
+# The longest run a column may have is 32 entries and the longest region 704: on either side of both the rounds
 # match the oracle, and the layout changes where the rule says.
 @pytest.mark.parametrize("hot_rows,entries", [(1, True), (2, True), (31, True), (32, True), (33, False), (64, False)])
 def test_runs_up_to_the_rule(hot_rows, entries):
@@ -106,10 +106,10 @@ def test_runs_up_to_the_rule(hot_rows, entries):
         _check(ctx, sh, 4, B, "logistic", 0.5, rounds.graph_schedule("root", N, 2))
 
 
-@pytest.mark.parametrize("per_row,entries", [(8, True), (15, True), (16, False)])
+@pytest.mark.parametrize("per_row,entries", [(8, True), (10, True), (11, False)])
 def test_regions_up_to_the_rule(per_row, entries):
-    # one slab of 1,024 columns (N = 8) holds 64 rows x per_row entries of worker 0, and about 20 entries of
-    # padding at 960 (before runs that would cross a multiple of 32)
+    # one slab of 1,024 columns (N = 8) holds 64 rows x per_row entries of worker 0, and about 15 entries of
+    # padding at 640 (before runs that would cross a multiple of 32)
     N, d, B = 8, 1024, 64
     ln = [np.full(2 * B, per_row)] + [np.zeros(2 * B, np.int64)] * (N - 1)
     sh = inputs.sparse_custom(seed=per_row, N=N, d=d, rows=2 * B, lengths=ln)
