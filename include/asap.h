@@ -397,7 +397,7 @@ asap_status asap_build_graph(asap_graph_kind kind, int N, int k, uint64_t graph_
  * address is kept per device together with the id of the CUDA context it
  * was found in; a call from a different context (after cudaDeviceReset, or
  * a host framework that reset its primary context) looks it up again.  Every
- * call shares the array and clears what must start at zero; calls that
+ * call shares the array and leaves at zero what must start there; calls that
  * overlap on the GPU (other streams, other threads) race on it and must be
  * serialised by the caller.  Async on cuda_stream (NULL: legacy default
  * stream); no device-side error is reported. */

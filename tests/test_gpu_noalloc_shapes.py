@@ -1,0 +1,58 @@
+"""asap_mix_noalloc over its range (GPU): every number of inputs per row its
+kernel is built for and the general one, slabs from 32 to 1,024 columns,
+leading dimensions from 4 up, tables that are not doubly stochastic, against
+the oracle's reduce and ||W_out - 1 wbar^T||_F with wbar the column mean of the
+input.  Tolerances: 1e-6 per worker for at most 32 fp32 multiply-adds of
+values of like size (32 x 2^-24 = 2e-6 at worst, a few 2^-24 in practice), 1e-5
+for the error norm."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from parity import rel_err_rows
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(W, d, nbr, wgt, calls=1):
+    import torch
+
+    from paper_1612_08608_gb300._lib import load_library
+    lib = load_library()
+    N, ld = W.shape
+    W_in, W_out = torch.from_numpy(W).cuda(), torch.full((N, ld), float("nan"), device="cuda")
+    n, w = torch.from_numpy(nbr.astype(np.int32)).cuda(), torch.from_numpy(wgt.astype(np.float32)).cuda()
+    cons = torch.empty(1, device="cuda")
+    p = C.c_void_p
+    for _ in range(calls):
+        st = lib.asap_mix_noalloc(p(W_in.data_ptr()), p(W_out.data_ptr()), N, d, ld, p(n.data_ptr()), p(w.data_ptr()),
+                                  nbr.shape[1], p(cons.data_ptr()), p(torch.cuda.current_stream().cuda_stream))
+        assert st == 0, lib.asap_last_error(None)
+    torch.cuda.synchronize()
+    return W_out.cpu().numpy(), cons.item()
+
+
+@pytest.mark.parametrize("N,ld", [(1, 4), (1, 4100), (2, 20), (3, 36), (7, 9732), (8, 4096), (9, 500000), (33, 1028),
+                                  (100, 30004), (255, 644), (256, 40000)])
+@pytest.mark.parametrize("kp1", [1, 2, 3, 5, 7, 32])
+def test_matches_the_reduce(N, ld, kp1):
+    rng = np.random.default_rng(N * 100 + kp1)
+    W = rng.standard_normal((N, ld)).astype(np.float32) + 3.0 * rng.standard_normal(ld).astype(np.float32)
+    nbr = rng.integers(0, N, (N, kp1))              # repeated ids and rows without the worker itself are allowed
+    wgt = rng.random((N, kp1)).astype(np.float32)
+    wgt /= wgt.sum(axis=1, keepdims=True)
+    got, cons = _run(W, ld, nbr, wgt, calls=2)
+    want = np.einsum("im,imc->ic", wgt.astype(np.float64), W.astype(np.float64)[nbr]) if N * ld * kp1 < 4e6 else \
+        sum(wgt[:, m:m + 1].astype(np.float64) * W.astype(np.float64)[nbr[:, m]] for m in range(kp1))
+    assert rel_err_rows(got, want) <= 1e-6
+    err = np.sqrt(((want - W.astype(np.float64).mean(axis=0)) ** 2).sum())
+    # the norm is off by at most the norm of the elements' errors: kp1 roundings of the output and about two of
+    # the mean, each at most 2^-24 of values no larger than W's (rms)
+    assert abs(cons - err) <= 1e-5 * err + (kp1 + 2) * 2.0 ** -24 * np.linalg.norm(W), (cons, err)
+
+
+def test_ids_outside_the_range_are_clamped():
+    W = np.arange(4 * 64, dtype=np.float32).reshape(4, 64)
+    got, _ = _run(W, 64, np.array([[-5], [4], [100], [1]]), np.ones((4, 1)))
+    assert np.array_equal(got, W[[0, 3, 3, 1]])
