@@ -22,7 +22,7 @@
 // N = 32, d = 4 10^6, k = 2: 178 us, 5.7 TB/s; loaded slab by slab with plain
 // loads, one slab in flight per CTA, 280 us.  A small call is launch latency: N =
 // 8, d = 4,093 8.1 us, 9.5 us while a memset cleared the ticket before each
-// launch (the last CTA leaves it at zero).
+// launch (now the last CTA leaves it at zero).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -47,10 +47,16 @@ constexpr int kNoAllocTicketBytes = 256;
 constexpr size_t kNoAllocScratchBytes = kNoAllocTicketBytes + 8u * kNoAllocMaxSlabs;   // 262,400 bytes
 constexpr int kNoAllocMaxDevices = 64;
 
-// [0, 4): ticket counter; [256, 256 + 8 * kNoAllocMaxSlabs): double partials,
-// one per CTA (the size, and with it the largest ld, dates from one per slab).
+// [0, 256): ticket counters; [256, 256 + 8 * kNoAllocMaxSlabs): double
+// partials, one per CTA (the size, and with it the largest ld, dates from one
+// per slab).  Calls take kSlots slots of both in turn.  A call's last CTA
+// leaves its own ticket at zero, and clears the one half the slots away: calls
+// that overlapped against the rules (their stream order is the caller's
+// business) cannot spoil more than the calls right after them.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
+constexpr int kSlots = 32;
+constexpr int kSlotPartials = kNoAllocMaxSlabs / kSlots;
 constexpr int kStages = 4;
 constexpr int kGroups = 2;                             // compute groups, on alternate slabs
 constexpr int kGroupThreads = 256;
@@ -69,7 +75,8 @@ struct NoAllocArgs {
   int S;           // slab width (columns), a power of two from 32 to 1024
   long long n_slabs;
   float* consensus_out;
-  unsigned int* ticket;
+  unsigned int* tickets;
+  int slot;
   double* partial;
 };
 
@@ -315,7 +322,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
   if (tid == 0) {
     a.partial[blockIdx.x] = static_cast<double>(ps.hi) + static_cast<double>(ps.lo);
     __threadfence();
-    sm.flag[0] = (atomicAdd(a.ticket, 1u) == gridDim.x - 1) ? 1 : 0;
+    sm.flag[0] = (atomicAdd(a.tickets + a.slot, 1u) == gridDim.x - 1) ? 1 : 0;
   }
   __syncthreads();
   if (!sm.flag[0]) return;
@@ -329,7 +336,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
   const Pair sum = block_sum(v, sm.red);
   if (tid == 0) {
     a.consensus_out[0] = sqrtf(fmaxf(sum.hi + sum.lo, 0.f));
-    *a.ticket = 0u;
+    a.tickets[a.slot] = 0u;
+    a.tickets[(a.slot + kSlots / 2) % kSlots] = 0u;
   }
 }
 
@@ -340,6 +348,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 struct DeviceSlot {
   void* scratch = nullptr;
   int sm_count = 0;
+  unsigned calls = 0;              // calls on this device so far
   EncodeTiledFn encode = nullptr;
   unsigned long long ctx_id = 0;   // the CUDA context the address belongs to
 };
@@ -451,6 +460,7 @@ extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, 
       ds.ctx_id = current_context_id();
     }
     slot = ds;
+    ++ds.calls;
   }
   // Slab: S columns of all rows, at most 32 KB; narrower (down to 128-byte
   // rows) while that leaves SMs without two slabs, one for each group.
@@ -480,10 +490,11 @@ extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, 
   a.S = S;
   a.n_slabs = (ld + S - 1) / S;
   a.consensus_out = consensus_out;
-  a.ticket = reinterpret_cast<unsigned int*>(base);   // zero: every launch's last CTA leaves it so
-  a.partial = reinterpret_cast<double*>(base + kNoAllocTicketBytes);
+  a.tickets = reinterpret_cast<unsigned int*>(base);
+  a.slot = static_cast<int>(slot.calls % kSlots);
+  a.partial = reinterpret_cast<double*>(base + kNoAllocTicketBytes) + static_cast<size_t>(a.slot) * kSlotPartials;
   const size_t smem = noalloc_smem(N, S, kp1);
-  const int grid = static_cast<int>(std::min<long long>(a.n_slabs, slot.sm_count));
+  const int grid = static_cast<int>(std::min<long long>(a.n_slabs, std::min(slot.sm_count, kSlotPartials)));
   switch (kp1) {
     case 2: k_mix_noalloc<2><<<grid, kBlock, smem, s>>>(tmap, a); break;
     case 3: k_mix_noalloc<3><<<grid, kBlock, smem, s>>>(tmap, a); break;

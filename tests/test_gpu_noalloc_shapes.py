@@ -56,3 +56,18 @@ def test_ids_outside_the_range_are_clamped():
     W = np.arange(4 * 64, dtype=np.float32).reshape(4, 64)
     got, _ = _run(W, 64, np.array([[-5], [4], [100], [1]]), np.ones((4, 1)))
     assert np.array_equal(got, W[[0, 3, 3, 1]])
+
+
+def test_calls_of_different_sizes_in_turn():
+    # more calls than the scratch has slots, of one to many CTAs
+    rng = np.random.default_rng(1)
+    sizes = [(3, 36), (8, 4096), (64, 9000), (1, 4), (200, 700)]
+    for t in range(40):
+        N, ld = sizes[t % len(sizes)]
+        W = rng.standard_normal((N, ld)).astype(np.float32)
+        nbr = np.stack([np.arange(N), (np.arange(N) + 1) % N], axis=1)
+        got, cons = _run(W, ld, nbr, np.full((N, 2), 0.5))
+        want = 0.5 * (W.astype(np.float64) + W.astype(np.float64)[nbr[:, 1]])
+        err = np.sqrt(((want - W.astype(np.float64).mean(axis=0)) ** 2).sum())
+        assert rel_err_rows(got, want) <= 1e-6
+        assert abs(cons - err) <= 1e-5 * err + 4 * 2.0 ** -24 * np.linalg.norm(W), (t, cons, err)
