@@ -96,7 +96,7 @@ struct asap_ctx {
   bool sharded = false;
   int own_lo = 0, own_n = 0;
   std::vector<unsigned char> delivered;   // [N] row j written this round (asap_write_rows)
-  double* cons_part = nullptr;
+  float2* cons_part = nullptr;
   int cons_cap = 0;
   int32_t* d_nbr = nullptr;
   float* d_wgt = nullptr;
@@ -279,9 +279,12 @@ asap_status setup_mix(asap_ctx* c) {
   // aligned in shared memory (S >= 8 floats per row).
   c->box_rows = ((N + c->n_boxes - 1) / c->n_boxes + 3) / 4 * 4;
   c->rows_pad = c->n_boxes * c->box_rows;
-  // Slab: S columns of all rows, about 32 KB (8 <= S <= 1024, a power of 2).
+  // Slab: S columns of all rows, about 32 KB (8 <= S <= 1024, a power of 2);
+  // narrower, down to 128-byte rows, while that leaves SMs without two slabs:
+  // a small problem is one slab's latency, and its hottest slab's list.
   int S = 1024;
   while (S > 8 && static_cast<size_t>(c->rows_pad) * S * 4 > 32768) S >>= 1;
+  while (S > 32 && (c->ld + S - 1) / S < 2LL * c->sm_count) S >>= 1;
   int maxS = 8;
   while (static_cast<int64_t>(maxS) * 2 <= c->ld && maxS < 1024) maxS <<= 1;
   c->S = std::min(std::min(S, maxS), c->s_cap);

@@ -187,7 +187,7 @@ struct MixArgs {
   int64_t row_stride;
   int B;
   // metrics and protocol
-  double* cons_part;           // scratch [gridDim.x]
+  float2* cons_part;           // scratch [gridDim.x]: float-float pairs
   const float* loss_part;      // [n_loss_part] from the local step
   int n_loss_part;
   float loss_norm;             // 1 / (N B)

@@ -35,9 +35,9 @@
 // lo, a fixed order).  The complete graph (all-reduce, equal weights) writes
 // the column mean to every row and adds nothing.
 //
-// Protocol (Section 4, NOTIFY-ACK): before touching any input each CTA waits,
+// Protocol (Section 4, NOTIFY-ACK): before it writes anything each CTA waits,
 // with a time limit, until ready[j] == round+1 for every worker j and
-// consumed[j] >= round.  The last CTA to finish (ticket) reduces the metric
+// consumed[j] >= round (a gated reduce: before it reads).  The last CTA to finish (ticket) reduces the metric
 // partials in a fixed order and ACKs: consumed[j] = round+1,
 // stamp_next[j] = round+1.
 #include <cuda.h>
@@ -241,37 +241,31 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
   return F2{hi, e - (hi - s)};
 }
 
-__device__ __forceinline__ F2 f2_of(double v) {
-  const float h = static_cast<float>(v);
-  return F2{h, static_cast<float>(v - static_cast<double>(h))};
-}
-
-// Sum over all threads of the block (kMixThreads) in a fixed order; valid in
-// thread 0.
-__device__ __forceinline__ F2 block_sum_f2(F2 v, F2* scratch) {
+__device__ __forceinline__ F2 warp_sum_f2(F2 v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
     v = f2_add(v, F2{__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o)});
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  F2 t{0.f, 0.f};
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kMixThreads / 32; ++k) t = f2_add(t, scratch[k]);
-  return t;
+  return v;
 }
 
-// Two block sums at once, each in the order block_sum_f2 takes (so each
-// result equals that of a separate call); valid in thread 0.  `scratch`
-// holds two pairs per warp.
-__device__ __forceinline__ void block_sum2_f2(F2& u, F2& v, F2* scratch) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    u = f2_add(u, F2{__shfl_xor_sync(kFull, u.hi, o), __shfl_xor_sync(kFull, u.lo, o)});
-    v = f2_add(v, F2{__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o)});
-  }
+// Sum over all threads of the block (kMixThreads) in a fixed order, a warp
+// tree over the lanes and one over the warps; valid in thread 0.
+__device__ __forceinline__ F2 block_sum_f2(F2 v, F2* scratch) {
   constexpr int kW = kMixThreads / 32;
+  static_assert(kW <= 32, "one lane per warp");
+  v = warp_sum_f2(v);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) scratch[warp] = v;
+  __syncthreads();
+  return warp == 0 ? warp_sum_f2(lane < kW ? scratch[lane] : F2{0.f, 0.f}) : F2{0.f, 0.f};
+}
+
+// Two block sums at once, each in the order block_sum_f2 takes; valid in
+// thread 0.  `scratch` holds two pairs per warp.
+__device__ __forceinline__ void block_sum2_f2(F2& u, F2& v, F2* scratch) {
+  constexpr int kW = kMixThreads / 32;
+  u = warp_sum_f2(u);
+  v = warp_sum_f2(v);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __syncthreads();
   if (lane == 0) {
@@ -279,14 +273,20 @@ __device__ __forceinline__ void block_sum2_f2(F2& u, F2& v, F2* scratch) {
     scratch[kW + warp] = v;
   }
   __syncthreads();
-  F2 tu{0.f, 0.f}, tv{0.f, 0.f};
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kW; ++k) {
-      tu = f2_add(tu, scratch[k]);
-      tv = f2_add(tv, scratch[kW + k]);
-    }
-  u = tu;
-  v = tv;
+  if (warp == 0) {
+    u = warp_sum_f2(lane < kW ? scratch[lane] : F2{0.f, 0.f});
+    v = warp_sum_f2(lane < kW ? scratch[kW + lane] : F2{0.f, 0.f});
+  }
+}
+
+// Barrier of all warps but the producer's, and at its own time the
+// producer's, that also returns the OR of `v` over them.
+__device__ __forceinline__ bool start_bar_or(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 4, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r) : "r"(static_cast<uint32_t>(v)), "n"(kMixThreads) : "memory");
+  return r != 0;
 }
 
 // Barrier of a compute group.
@@ -320,7 +320,7 @@ struct MixSmem {
   int* linfo;        // [list_slots]: entries of the slab
   int* nbr;
   float* wgt;
-  double* dscratch;
+  F2* scratch;       // two pairs per warp
   int* flags;        // [0]: fail, [1]: last, [2]: failed CTAs of the launch (last CTA), [3]: slabs whose NOTIFY
                      // the producer has seen (gated reduces on the entry layout)
   unsigned* seen;    // [32]: bitmap of workers whose NOTIFY this CTA has seen (gated reduces)
@@ -351,7 +351,7 @@ __device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, i
   off += 8 * a.list_slots;
   m.linfo = reinterpret_cast<int*>(raw + off);
   off = a16(off + 4 * a.list_slots);
-  m.dscratch = reinterpret_cast<double*>(raw + off);
+  m.scratch = reinterpret_cast<F2*>(raw + off);
   off = a16(off + 16 * (kMixThreads / 32));
   m.flags = reinterpret_cast<int*>(raw + off);
   off = a16(off + 16);
@@ -514,8 +514,30 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   const size_t list_off = (slab_floats * 4 + 15) & ~static_cast<size_t>(15);
   const size_t list_bytes = (static_cast<size_t>(a.max_region) * 4 + 15) & ~static_cast<size_t>(15);
 
-  if (tid == 0) { sm.flags[0] = 0; sm.flags[1] = 0; sm.flags[3] = 0; }
+  // Before the previous kernel is waited for: barriers, and the mixing table,
+  // which is complete on the device before the kernels of its round begin.
+  // (With these and the flags after the wait and before the first loads, and
+  // slabs of 32 KB for every size, a reduce of N = 8, d = 10^5 took 10.8 us in a
+  // row of reduces, now 9.7; the RCV1-shaped one 18.5 us, now 16.7.)
+  if (tid == 0) {
+    sm.flags[0] = 0;
+    sm.flags[1] = 0;
+    sm.flags[3] = 0;
+    for (int s = 0; s < a.stages; ++s) {
+      mbar_init(sm.full + s, 1);
+      mbar_init(sm.empty + s, kMixComputeWarps / kGroups);
+      mbar_init(sm.ready + s, kMixUpdaterWarps);
+    }
+    for (int s = 0; s < a.list_slots; ++s) mbar_init(sm.lfull + s, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   if (tid < 32) sm.seen[tid] = 0u;
+  if (KP1 >= 0) {
+    for (int idx = tid; idx < a.N * kp1; idx += kMixThreads) {
+      sm.nbr[idx] = a.nbr[idx] * QB;       // float4 offset of the neighbour's row within a box column
+      sm.wgt[idx] = a.wgt[idx] * a.wscale;
+    }
+  }
   __syncthreads();
   // A gated reduce (NOTIFY_ACK or ASYNC, sparse models) runs while the local
   // step may still be running: it reads the column sums of worker j only
@@ -532,39 +554,38 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   }
 
   // ---- NOTIFY / ACK checks (time-limited waits) ----
-  for (int j = tid; j < a.N; j += kMixThreads) {
-    unsigned e = 0;
-    const bool own = j >= a.own_lo && j < a.own_lo + a.own_n;
-    if (a.expect_notify && !gated && own) e = wait_flag(a.ready + j, a.round + 1u, true, a.wait_ns);
-    if (!e) e = wait_flag(a.consumed + j, a.round, false, a.wait_ns);
-    if (e) {
-      record_error(a.st, e, j, a.round);
-      if (e == ASAP_ERR_TIMEOUT) atomicAdd(&a.st->timeouts, 1ull);
-      atomicOr(&sm.flags[0], 1);
+  // A gated reduce checks the ACKs before it reads anything.  Otherwise the
+  // grid before has finished and its flags are final: they are checked while
+  // the first slabs fly, by all warps but the producer's, and before anything
+  // is written.
+  auto check_flags = [&](int first, int step) {
+    bool bad = false;
+    for (int j = first; j < a.N; j += step) {
+      unsigned e = 0;
+      const bool own = j >= a.own_lo && j < a.own_lo + a.own_n;
+      if (a.expect_notify && !gated && own) e = wait_flag(a.ready + j, a.round + 1u, true, a.wait_ns);
+      if (!e) e = wait_flag(a.consumed + j, a.round, false, a.wait_ns);
+      if (e) {
+        record_error(a.st, e, j, a.round);
+        if (e == ASAP_ERR_TIMEOUT) atomicAdd(&a.st->timeouts, 1ull);
+        atomicOr(&sm.flags[0], 1);
+        bad = true;
+      }
     }
+    __syncwarp();
+    return bad;
+  };
+  if (gated) {
+    check_flags(tid, kMixThreads);
+    __syncthreads();
   }
-  __syncthreads();
-  bool failed = sm.flags[0] != 0;
+  bool failed = gated && sm.flags[0] != 0;
+  bool quiet = false;                    // a flag was missing: pass the slabs on, write nothing
+  if (!gated && warp != kProducerWarp)
+    quiet = start_bar_or(check_flags(tid < kProducerWarp * 32 ? tid : tid - 32, kMixThreads - 32));
 
   float s2 = 0.f;      // compute threads: sum of (w - K)^2;  producer lanes: -sum of S1^2 / N
   if (!failed) {
-    if (KP1 >= 0) {
-      for (int idx = tid; idx < a.N * kp1; idx += kMixThreads) {
-        sm.nbr[idx] = a.nbr[idx] * QB;       // float4 offset of the neighbour's row within a box column
-        sm.wgt[idx] = a.wgt[idx] * a.wscale;
-      }
-    }
-    if (tid == 0) {
-      for (int s = 0; s < a.stages; ++s) {
-        mbar_init(sm.full + s, 1);
-        mbar_init(sm.empty + s, kMixComputeWarps / kGroups);
-        mbar_init(sm.ready + s, kMixUpdaterWarps);
-      }
-      for (int s = 0; s < a.list_slots; ++s) mbar_init(sm.lfull + s, 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-
     const long long stride = gridDim.x;
     const int n_my = static_cast<int>((a.n_slabs - blockIdx.x + stride - 1) / stride);   // slabs of this CTA
     const float inv_n = 1.0f / static_cast<float>(a.N);
@@ -583,6 +604,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       int st = 0, done_st = 0;                        // stages of slab it, and of the slab that came back
       uint32_t done_ph = 0;
       for (int it = 0; it < n_my + a.stages; ++it) {
+        if (!gated && it == min(a.stages, n_my)) start_bar_or(false);
         if (FUSED && (it & 31) == 0 && it < n_my) {
           const long long sl = blockIdx.x + static_cast<long long>(it + lane) * stride;
           if (it + lane < n_my)
@@ -750,7 +772,18 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // ================= updater warps (FUSED) =================
       // Once a slab has landed, apply w -= eta/B (1 - eta l2)^-1 g to it and
       // release it to the compute warps.
-      if constexpr (ENTRIES) {
+      if (FUSED && quiet) {
+        int st = 0;
+        uint32_t ph = 0;
+        for (int it = 0; it < n_my; ++it) {
+          if (!__all_sync(kFull, mbar_wait_bounded(sm.full + st, ph))) break;
+          if (lane == 0) mbar_arrive(sm.ready + st);
+          if (++st == a.stages) {
+            st = 0;
+            ph ^= 1u;
+          }
+        }
+      } else if constexpr (ENTRIES) {
         update_entries(sm, a, n_my, gated, lS, lqb, box_col, failed);
       } else if (FUSED) {
         const int ut = tid - kUpdater0 * 32;
@@ -857,6 +890,13 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         const int* info = sm.info + 4 * st;
         float4* part = sm.part + st * kCompute;
         const long long c0 = slab * S;
+        if (quiet) {                     // the same for every compute thread
+          __syncwarp();
+          if (lane == 0) mbar_arrive(sm.empty + st);
+          st += kGroups;
+          if (!ok) break;
+          continue;
+        }
         if (ok && KP1 < 0) {
           // Complete graph: this thread's share of its column's sum.
           float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1012,11 +1052,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   }
 
   // ---- per-CTA partial, ticket, and the last CTA's finalisation ----
-  F2* scratch = reinterpret_cast<F2*>(sm.dscratch);
+  F2* scratch = sm.scratch;
+  if (failed && lane == 0) atomicOr(&sm.flags[0], 1);
   const F2 csum = block_sum_f2(F2{s2, 0.f}, scratch);
-  if (failed) atomicOr(&sm.flags[0], 1);
-  __syncthreads();
-  if (tid == 0) a.cons_part[blockIdx.x] = static_cast<double>(csum.hi) + static_cast<double>(csum.lo);
+  if (tid == 0) a.cons_part[blockIdx.x] = make_float2(csum.hi, csum.lo);
   __threadfence();
   __syncthreads();
   if (tid == 0) {
@@ -1039,7 +1078,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   const int n_lp = a.have_loss ? a.n_loss_part : 0;
   F2 ctot{0.f, 0.f}, ltot{0.f, 0.f};
   for (int b = tid; b < (loss_after_notify ? n_cons : max(n_cons, n_lp)); b += kMixThreads) {
-    if (b < n_cons) ctot = f2_add(ctot, f2_of(__ldcg(a.cons_part + b)));
+    if (b < n_cons) {
+      const float2 p = __ldcg(a.cons_part + b);
+      ctot = f2_add(ctot, F2{p.x, p.y});
+    }
     if (!loss_after_notify && b < n_lp) ltot = f2_add(ltot, F2{__ldcg(a.loss_part + b), 0.f});
   }
   if (loss_after_notify) {
@@ -1056,6 +1098,11 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     }
     for (int b = tid; b < n_lp; b += kMixThreads) ltot = f2_add(ltot, F2{__ldcg(a.loss_part + b), 0.f});
   }
+  if (!any_fail)           // ACK, while the sums below are formed
+    for (int j = tid; j < a.N; j += kMixThreads) {
+      a.stamp_next[j] = a.round + 1u;
+      st_release_u32(a.consumed + j, a.round + 1u);
+    }
   block_sum2_f2(ctot, ltot, scratch);
   if (tid == 0) {
     const int slot = static_cast<int>(a.round % kMetricsCap);
@@ -1068,13 +1115,6 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         atomicAdd(&a.st->consistent_inputs, static_cast<unsigned long long>(a.own_n) * (KP1 < 0 ? a.N : kp1));
     }
     a.st->mix_ticket = 0u;
-  }
-  if (!any_fail) {
-    __threadfence();
-    for (int j = tid; j < a.N; j += kMixThreads) {
-      a.stamp_next[j] = a.round + 1u;
-      st_release_u32(a.consumed + j, a.round + 1u);
-    }
   }
 }
 

@@ -65,7 +65,7 @@ def test_rows_and_graphs(B, N, k, kind):
     sh = inputs.sparse_custom(seed=B, N=N, d=d, rows=3 * B, lengths=lengths)
     W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
     with _make(sh, N, k, kind, "logistic", B, 0.5, regen=kind == "random_regular") as ctx:
-        if B >= 31:
+        if N * B >= 93:                                # enough entries to tell by
             assert _uses_entries(ctx, sh, B)
         sched = rounds.graph_schedule(kind, N, k, graph_seed=7, regenerate=kind == "random_regular")
         _check(ctx, sh, 4, B, "logistic", 0.5, sched, W0=W0)
@@ -87,7 +87,7 @@ def test_local_steps_l2_and_residency(residency, sync):
 # match the oracle, and the layout changes where the rule says.
 @pytest.mark.parametrize("hot_rows,entries", [(1, True), (2, True), (31, True), (32, True), (33, False), (64, False)])
 def test_runs_up_to_the_rule(hot_rows, entries):
-    N, d, B = 4, 20000, 64
+    N, d, B = 4, 4000, 64
     rng = np.random.default_rng(hot_rows)
     sh = inputs.sparse_custom(seed=hot_rows, N=N, d=d, rows=2 * B, lengths=[np.full(2 * B, 12)] * N)
     for i in range(N):
@@ -108,11 +108,12 @@ def test_runs_up_to_the_rule(hot_rows, entries):
 
 @pytest.mark.parametrize("per_row,entries", [(8, True), (10, True), (11, False)])
 def test_regions_up_to_the_rule(per_row, entries):
-    # one slab of 1,024 columns (N = 8) holds 64 rows x per_row entries of worker 0, and about 15 entries of
+    # 313 slabs of 1,024 columns (N = 8); the first holds 64 rows x per_row entries of worker 0, and about 15 entries of
     # padding at 640 (before runs that would cross a multiple of 32)
-    N, d, B = 8, 1024, 64
+    N, d, B = 8, 320000, 64
     ln = [np.full(2 * B, per_row)] + [np.zeros(2 * B, np.int64)] * (N - 1)
-    sh = inputs.sparse_custom(seed=per_row, N=N, d=d, rows=2 * B, lengths=ln)
+    sh = inputs.sparse_custom(seed=per_row, N=N, d=1024, rows=2 * B, lengths=ln)
+    sh.d = d
     with _make(sh, N, 1, "ring", "logistic", B, 0.5) as ctx:
         assert _uses_entries(ctx, sh, B) == entries
         _check(ctx, sh, 3, B, "logistic", 0.5, rounds.graph_schedule("ring", N, 1))
@@ -121,7 +122,7 @@ def test_regions_up_to_the_rule(per_row, entries):
 def test_empty_minibatches_and_two_runs_bit_identical():
     N, d, B = 5, 5000, 40
     rng = np.random.default_rng(0)
-    lengths = [rng.integers(0, 12, 3 * B) for _ in range(N)]
+    lengths = [rng.integers(0, 60, 3 * B) for _ in range(N)]
     for ln in lengths:
         ln[B:2 * B] = 0
     sh = inputs.sparse_custom(seed=9, N=N, d=d, rows=3 * B, lengths=lengths)

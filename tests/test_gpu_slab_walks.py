@@ -12,10 +12,10 @@ from parity import sparse_round_matching
 pytestmark = pytest.mark.gpu
 
 
-# d = 3,000 and 1,300,000 at N = 8: 3 slabs (one CTA each) and 1,270 slabs
-# (more than one wave of CTAs, so a warp per slab unless a region is long);
-# the first slab holds 8 x cols distinct (worker, column) pairs at most: a
-# few (one partial pass of a warp), 1,024 exactly, and more.
+# d = 3,000 and 1,300,000 at N = 8: 94 slabs of 32 columns (one CTA each) and
+# 1,270 of 1,024 (more than one wave of CTAs, so a warp per slab unless a region
+# is long); the wide slabs' first region holds about 8 x cols distinct (worker,
+# column) pairs: a few (one partial pass of a warp), 1,017, and 2,128.
 @pytest.mark.parametrize("d", [3000, 1300000])
 @pytest.mark.parametrize("cols", [3, 128, 300])
 def test_slab_walks_match_oracle(d, cols):
