@@ -49,6 +49,9 @@ namespace asap {
 void set_thread_error(const char* msg) { g_last_error = msg; }
 }  // namespace asap
 
+// Rounds of metrics that one read fetches through pinned memory.
+constexpr int kReadMetrics = 1024;
+
 struct asap_ctx {
   int dev = 0, sm_count = 0;
   int N = 0;
@@ -78,11 +81,19 @@ struct asap_ctx {
 
   float* W[2] = {nullptr, nullptr};
   uint16_t* Wbf[2] = {nullptr, nullptr};
+  unsigned* flags = nullptr;     // one block of 5 N words: the four arrays below
   unsigned* ready = nullptr;
   unsigned* consumed = nullptr;
   unsigned* stamp = nullptr;     // [2][N]
   unsigned* ticket = nullptr;    // [N]
+  unsigned* h_flags = nullptr;   // pinned image of the block, for resets
   DevState* st = nullptr;
+  // pinned landing place of small reads: device state, then metrics
+  struct HostReads {
+    DevState st;
+    float loss[kReadMetrics], cons[kReadMetrics];
+  };
+  HostReads* h_read = nullptr;
   float* m_loss = nullptr;
   float* m_cons = nullptr;
   float* r_scr = nullptr;
@@ -373,12 +384,15 @@ asap_status configure_mix_launch(asap_ctx* c, int mode) {
   return ASAP_OK;
 }
 
+// Flags of round rnd, after everything queued on the context stream; waits for
+// the stream (the pinned image is free again).
 asap_status reset_protocol(asap_ctx* c, int64_t rnd) {
-  std::vector<unsigned> v(c->N, static_cast<unsigned>(rnd));
-  CU(cudaMemcpy(c->ready, v.data(), 4 * c->N, cudaMemcpyHostToDevice), "resetting NOTIFY flags");
-  CU(cudaMemcpy(c->consumed, v.data(), 4 * c->N, cudaMemcpyHostToDevice), "resetting ACK flags");
-  CU(cudaMemcpy(c->stamp + (rnd & 1) * c->N, v.data(), 4 * c->N, cudaMemcpyHostToDevice), "resetting stamps");
-  CU(cudaMemset(c->ticket, 0, 4 * c->N), "resetting tickets");
+  const int N = c->N;
+  std::fill(c->h_flags, c->h_flags + 4 * N, static_cast<unsigned>(rnd));   // NOTIFY, ACK, stamps
+  std::fill(c->h_flags + 4 * N, c->h_flags + 5 * N, 0u);                   // tickets
+  CU(cudaMemcpyAsync(c->flags, c->h_flags, 20 * static_cast<size_t>(N), cudaMemcpyHostToDevice, c->stream),
+     "resetting the protocol flags");
+  CU(cudaStreamSynchronize(c->stream), "resetting the protocol flags");
   c->round = rnd;
   c->step_pending = false;
   c->graph_ready_round = -1;
@@ -499,9 +513,8 @@ void time_end(asap_ctx* c) {
   ++c->tused;
 }
 
-asap_status check_device_error(asap_ctx* c) {
-  DevState h;
-  CU(cudaMemcpy(&h, c->st, sizeof(DevState), cudaMemcpyDeviceToHost), "reading device state");
+// Reports the error in a copy of the device state, if any, and clears it.
+asap_status check_device_error(asap_ctx* c, const DevState& h) {
   if (h.err_code == 0) return ASAP_OK;
   const unsigned zero = 0;
   CU(cudaMemcpy(&c->st->err_code, &zero, 4, cudaMemcpyHostToDevice), "clearing device error");
@@ -517,9 +530,11 @@ asap_status check_device_error(asap_ctx* c) {
 }
 
 asap_status sync_all(asap_ctx* c) {
+  CU(cudaMemcpyAsync(&c->h_read->st, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream),
+     "reading device state");
   CU(cudaStreamSynchronize(c->stream), "synchronising the context stream");
   if (c->copy_stream) CU(cudaStreamSynchronize(c->copy_stream), "synchronising the copy stream");
-  return check_device_error(c);
+  return check_device_error(c, c->h_read->st);
 }
 
 // The device image of minibatch t (host only): per worker the labels, the
@@ -1047,11 +1062,14 @@ static asap_status init_ctx(asap_ctx* c) {
     CU(cudaEventCreateWithFlags(&c->staged_ev[b], cudaEventDisableTiming), "creating events");
     CU(cudaEventCreateWithFlags(&c->free_ev[b], cudaEventDisableTiming), "creating events");
   }
-  CU(cudaMalloc(&c->ready, 4 * N), "allocating flags");
-  CU(cudaMalloc(&c->consumed, 4 * N), "allocating flags");
-  CU(cudaMalloc(&c->stamp, 8 * N), "allocating stamps");
-  CU(cudaMemset(c->stamp, 0, 8 * N), "zeroing stamps");
-  CU(cudaMalloc(&c->ticket, 4 * N), "allocating tickets");
+  CU(cudaMalloc(&c->flags, 20 * static_cast<size_t>(N)), "allocating flags");
+  CU(cudaMemset(c->flags, 0, 20 * static_cast<size_t>(N)), "zeroing flags");
+  CU(cudaHostAlloc(&c->h_flags, 20 * static_cast<size_t>(N), cudaHostAllocDefault), "allocating pinned flags");
+  CU(cudaHostAlloc(&c->h_read, sizeof(asap_ctx::HostReads), cudaHostAllocDefault), "allocating pinned reads");
+  c->ready = c->flags;
+  c->consumed = c->flags + N;
+  c->stamp = c->flags + 2 * N;
+  c->ticket = c->flags + 4 * N;
   CU(cudaMalloc(&c->d_worker_of, 4 * static_cast<size_t>(N)), "allocating the local-step map");
   CU(cudaMalloc(&c->st, sizeof(DevState)), "allocating device state");
   CU(cudaMemset(c->st, 0, sizeof(DevState)), "zeroing device state");
@@ -1108,10 +1126,9 @@ void asap_destroy(asap_ctx* c) {
     dfree(c->W[b]);
     dfree(c->Wbf[b]);
   }
-  dfree(c->ready);
-  dfree(c->consumed);
-  dfree(c->stamp);
-  dfree(c->ticket);
+  dfree(c->flags);
+  if (c->h_flags) cudaFreeHost(c->h_flags);
+  if (c->h_read) cudaFreeHost(c->h_read);
   dfree(c->d_worker_of);
   dfree(c->st);
   dfree(c->m_loss);
@@ -1849,9 +1866,8 @@ asap_status asap_write_params_device(asap_ctx* c, const float* dev_in, int64_t l
     CU(launch_cast_bf16(dst, c->Wbf[round & 1], static_cast<int64_t>(c->N) * c->ld, c->stream), "bf16 copy");
     c->launches += 1;
   }
-  CU(cudaStreamSynchronize(c->stream), "writing parameters");
   c->wv_step = -1;
-  return reset_protocol(c, round);
+  return reset_protocol(c, round);   // waits for the copy too
 }
 
 asap_status asap_read_param_columns(asap_ctx* c, int64_t first, int64_t count, float* host_out) {
@@ -1876,14 +1892,28 @@ asap_status asap_read_metrics(asap_ctx* c, int64_t first, int64_t count, float* 
     if (s != ASAP_OK) return s;
   } else {
     // Wait for round `last` only; rounds queued after it keep running.  A
-    // device error recorded by then is reported after a full drain.
+    // device error recorded by then is reported after a full drain.  The error
+    // code and a few rounds' metrics come in one go.
     CU(cudaStreamWaitEvent(c->read_stream, c->round_ev[ev], 0), "waiting for the round");
-    unsigned code = 0;
-    CU(cudaMemcpyAsync(&code, &c->st->err_code, 4, cudaMemcpyDeviceToHost, c->read_stream), "reading device state");
+    asap_ctx::HostReads* h = c->h_read;
+    CU(cudaMemcpyAsync(&h->st.err_code, &c->st->err_code, 4, cudaMemcpyDeviceToHost, c->read_stream),
+       "reading device state");
+    const int64_t slot = first % kMetricsCap;
+    const bool small = count <= kReadMetrics && slot + count <= kMetricsCap;
+    if (small && loss_out)
+      CU(cudaMemcpyAsync(h->loss, c->m_loss + slot, 4 * count, cudaMemcpyDeviceToHost, c->read_stream), "metrics");
+    if (small && cons_out)
+      CU(cudaMemcpyAsync(h->cons, c->m_cons + slot, 4 * count, cudaMemcpyDeviceToHost, c->read_stream), "metrics");
     CU(cudaStreamSynchronize(c->read_stream), "waiting for the round");
-    if (code != 0) {
+    if (h->st.err_code != 0) {
       asap_status s = sync_all(c);
       if (s != ASAP_OK) return s;
+    }
+    if (small) {
+      if (loss_out) std::copy(h->loss, h->loss + count, loss_out);
+      if (cons_out) std::copy(h->cons, h->cons + count, cons_out);
+      if (c->sharded && cons_out) std::fill(cons_out, cons_out + count, std::numeric_limits<float>::quiet_NaN());
+      return ASAP_OK;
     }
   }
   // Pageable destinations: each copy returns once it is done.
