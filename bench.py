@@ -232,9 +232,9 @@ def kernel_work(sh):
         # a label and a length and writes r per row
         out["local_step"] = ("GB/s", 4.0 * nnz + 10.0 * N * B, "hbm")
         out["reduce"] = ("GB/s", 8.0 * N * ld, "hbm")
-        # local steps before the round's last: code, value and r per entry, w read and written per column; then
-        # code, value, place and w per entry, a product written
-        out["apply"] = ("GB/s", 12.0 * nnz + 8.0 * touched, "hbm")
+        # local steps before the round's last: code, value and r per entry, w read and written per column, and for
+        # the next step's entries code, value, place and w read and a product written
+        out["apply"] = ("GB/s", 30.0 * nnz + 8.0 * touched, "hbm")
         out["gather"] = ("GB/s", 18.0 * nnz, "hbm")
         return out
     # list layout: the fused local step reads every entry once (list position,

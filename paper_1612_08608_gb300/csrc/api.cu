@@ -953,6 +953,33 @@ EntryList entry_list(const asap_ctx* c, const unsigned char* block, int t) {
   return x;
 }
 
+// The slab geometry of a reduce (configure_mix_launch comes first).
+void fill_slab_args(const asap_ctx* c, MixArgs* a) {
+  a->ld = c->ld;
+  a->N = c->N;
+  a->kp1 = c->tab_kp1;
+  a->S = c->S;
+  a->rows_pad = c->rows_pad;
+  a->box_rows = c->box_rows;
+  a->n_boxes = c->n_boxes;
+  a->stages = c->stages;
+  a->list_slots = c->list_slots;
+  a->n_slabs = c->n_slabs;
+}
+
+// The entries whose update is applied (minibatch t in block `bt`) and those
+// whose products are formed (tn in `bn`, into `prod`).
+void fill_entry_args(const asap_ctx* c, MixArgs* a, const unsigned char* bt, int t, const unsigned char* bn, int tn,
+                     float* prod) {
+  a->max_region = c->max_region;
+  a->upd = entry_list(c, bt, t);
+  a->exp = entry_list(c, bn, tn);
+  a->r = c->r_ent;
+  a->prod_out = prod;
+  a->row_stride = c->row_stride;
+  a->B = c->B;
+}
+
 // eta_k of global local step k.
 float lr_at(const asap_ctx* c, int64_t k) {
   if (c->lr_kind == ASAP_LR_INVERSE) return static_cast<float>(c->lr / (1.0 + c->lr_gamma * static_cast<double>(k)));
@@ -1668,8 +1695,31 @@ asap_status asap_local_step(asap_ctx* c) {
       // w_stored -= eta / (B s') g at the step's columns; the reduce applies
       // the round's last update itself, except in a worker-sharded context,
       // whose owned rows must hold x - eta g before they are sent.
+      // Where W does not stay in L2 between two kernels (64 MB: half of it), the
+      // slabs are streamed once for the update and the next step's products.
+      const bool stream_slabs = c->entries && !last && static_cast<size_t>(c->N) * c->ld * 4 > (64u << 20);
+      const unsigned char* next = nullptr;
+      if (stream_slabs) {
+        asap_status sn = block_of(c, k + 1, &next);
+        if (sn != ASAP_OK) return sn;
+        sn = configure_mix_launch(c, kMixEntries);
+        if (sn != ASAP_OK) return sn;
+        CU(entry_step_configure(), "configuring the local update kernel");
+      }
       time_begin(c, ASAP_KERNEL_APPLY);
-      if (c->entries)
+      if (stream_slabs) {
+        MixArgs m = {};
+        fill_slab_args(c, &m);
+        m.upd_scale = upd;
+        fill_entry_args(c, &m, block, tk, next, static_cast<int>((k + 1) % c->nb), c->wv[r & 1]);
+        m.step_w = c->W[r & 1];
+        m.st = c->st;
+        m.round = static_cast<unsigned>(r);
+        m.sync_mode = kSyncBsp;
+        CU(launch_entry_step(c->tmap[r & 1], m, c->mix_grid, c->mix_smem, c->stream),
+           "launching the local update kernel");
+        c->wv_step = k + 1;
+      } else if (c->entries)
         CU(launch_entry_update(c->W[r & 1], c->ld, entry_list(c, block, tk), c->n_slabs, c->S, c->max_region,
                                c->r_ent, c->B, upd, c->sm_count, c->stream),
            "launching the local update kernel");
@@ -1732,20 +1782,11 @@ asap_status asap_stochastic_reduce(asap_ctx* c) {
   MixArgs a = {};
   a.out = c->W[(r + 1) & 1];
   a.shadow = c->Wbf[(r + 1) & 1];
-  a.ld = c->ld;
-  a.N = c->N;
-  a.kp1 = c->tab_kp1;
+  fill_slab_args(c, &a);
   a.nbr = nbr;
   a.wgt = wgt;
   a.wscale = (c->step_pending && sparse) ? c->pend_wscale : 1.0f;
   a.uniform_w = uniform;
-  a.S = c->S;
-  a.rows_pad = c->rows_pad;
-  a.box_rows = c->box_rows;
-  a.n_boxes = c->n_boxes;
-  a.stages = c->stages;
-  a.list_slots = c->list_slots;
-  a.n_slabs = c->n_slabs;
   if (fused) {
     const unsigned char* bt = nullptr;
     const unsigned char* bn = nullptr;
@@ -1758,12 +1799,7 @@ asap_status asap_stochastic_reduce(asap_ctx* c) {
     a.upd_scale = c->pend_upd;
     a.max_region = c->max_region;
     if (c->entries) {
-      a.upd = entry_list(c, bt, t);
-      a.exp = entry_list(c, bn, tn);
-      a.r = c->r_ent;
-      a.prod_out = c->wv[(r + 1) & 1];
-      a.row_stride = c->row_stride;
-      a.B = c->B;
+      fill_entry_args(c, &a, bt, t, bn, tn, c->wv[(r + 1) & 1]);
     } else {
       a.upd_list = reinterpret_cast<const uint32_t*>(bt + c->list_off[t]);
       a.upd_off = reinterpret_cast<const int*>(bt + c->soff_off[t]);

@@ -184,6 +184,7 @@ struct MixArgs {
   int list_slots;              // ring slots of upd's regions (0 without entries)
   const float* r;              // [N][B] r of this round's rows
   float* prod_out;             // [N][B][row_stride] products of the next step's entries
+  float* step_w;               // entry step (launch_entry_step): the parameters updated in place
   int64_t row_stride;
   int B;
   // metrics and protocol
@@ -259,6 +260,11 @@ ASAP_HD size_t mix_stage_bytes(int S, int rows_pad, int max_region, int mode);
 size_t mix_smem_bytes(int N, int kp1, int S, int rows_pad, int stages, int max_region, int mode, int list_slots);
 cudaError_t mix_configure(bool complete, int mode, int kp1, bool shadow);
 cudaError_t mix_occupancy(bool complete, int mode, int kp1, bool shadow, size_t smem, int* blocks);
+// The update of a local step before a round's last, in place, and the products
+// of the next step, with the slabs streamed as by the reduce (a.upd, a.exp, a.r,
+// a.upd_scale, a.prod_out, a.step_w; shared memory as for a kMixEntries reduce).
+cudaError_t entry_step_configure();
+cudaError_t launch_entry_step(const CUtensorMap& tmap, const MixArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_row_step(const RowStepArgs& a, int loss, int workers, cudaStream_t s);
 cudaError_t launch_entry_products(const float* W, int64_t ld, const EntryList& x, long long n_slabs, int S,
                                   int max_region, float* prod, int B, int64_t stride, int sm_count, cudaStream_t s);

@@ -383,6 +383,8 @@ __device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, i
 // last one's column sums.  In a gated reduce r is read only after the NOTIFY of its worker:
 // early for slabs the producer has passed (sm.flags[3]), else in the landed
 // slab.
+// STORE: each updated value also goes to the stored parameters (a.step_w).
+template <bool STORE>
 __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs& a, int n_slabs, bool gated, int lS,
                                                int lqb, int box_col, bool& failed) {
   constexpr int kUpd = kMixUpdaterWarps * 32, kU = 5, kAhead = 2;
@@ -465,7 +467,15 @@ __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs&
             more = cd & kEntryMore;
           }
         }
-        if ((c[u] & kEntryNext) == 0u) x[off[u]] = fmaf(-a.upd_scale, sum, w[u]);
+        if ((c[u] & kEntryNext) == 0u) {
+          const float v = fmaf(-a.upd_scale, sum, w[u]);
+          x[off[u]] = v;
+          if (STORE) {
+            const long long slab = blockIdx.x + static_cast<long long>(it) * gridDim.x;
+            const uint32_t o = c[u] & kEntryOff;
+            a.step_w[static_cast<int64_t>(o >> lS) * a.ld + (slab << lS) + (o & (S - 1))] = v;
+          }
+        }
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before this stage's next TMA
@@ -493,12 +503,21 @@ __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs&
 
 // KP1 > 0: sparse graph with KP1 neighbours per row (compile-time);
 // KP1 == 0: sparse graph, runtime a.kp1 (<= kMaxKp1Sparse);
-// KP1 < 0: complete graph with equal weights.
+// KP1 == -1: complete graph with equal weights;
+// KP1 == kStepOnly (entry layout): no mixing, but the update of a local step
+// before a round's last, stored in place, and the next step's products, for
+// parameters that do not stay in L2.  The slabs are streamed whole: touched one
+// by one (kernels_entry.cu), two thirds of a hashed slab's 32-byte sectors cost a
+// 64-byte DRAM access each, twice (N = 64, d = 2^20, ~400 entries a slab:
+// update 75.5 us, products 57.3; so, both 105.8 us).
+constexpr int kStepOnly = -2;
+
 template <int KP1, bool SHADOW, int MODE>
 __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ CUtensorMap tmap, const MixArgs a) {
   extern __shared__ unsigned char smem_raw[];
   constexpr bool FUSED = MODE != kMixPlain;
   constexpr bool ENTRIES = MODE == kMixEntries;
+  constexpr bool STEP = KP1 == kStepOnly;
   constexpr int kGroups = mix_groups(MODE), kCompute = mix_group_threads(MODE);
   const int kp1 = KP1 > 0 ? KP1 : (KP1 == 0 ? a.kp1 : 0);
   MixSmem sm = carve(smem_raw, a, kp1, MODE);
@@ -581,7 +600,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   }
   bool failed = gated && sm.flags[0] != 0;
   bool quiet = false;                    // a flag was missing: pass the slabs on, write nothing
-  if (!gated && warp != kProducerWarp)
+  if (!STEP && !gated && warp != kProducerWarp)
     quiet = start_bar_or(check_flags(tid < kProducerWarp * 32 ? tid : tid - 32, kMixThreads - 32));
 
   float s2 = 0.f;      // compute threads: sum of (w - K)^2;  producer lanes: -sum of S1^2 / N
@@ -604,7 +623,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       int st = 0, done_st = 0;                        // stages of slab it, and of the slab that came back
       uint32_t done_ph = 0;
       for (int it = 0; it < n_my + a.stages; ++it) {
-        if (!gated && it == min(a.stages, n_my)) start_bar_or(false);
+        if (!STEP && !gated && it == min(a.stages, n_my)) start_bar_or(false);
         if (FUSED && (it & 31) == 0 && it < n_my) {
           const long long sl = blockIdx.x + static_cast<long long>(it + lane) * stride;
           if (it + lane < n_my)
@@ -784,7 +803,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
           }
         }
       } else if constexpr (ENTRIES) {
-        update_entries(sm, a, n_my, gated, lS, lqb, box_col, failed);
+        update_entries<STEP>(sm, a, n_my, gated, lS, lqb, box_col, failed);
       } else if (FUSED) {
         const int ut = tid - kUpdater0 * 32;
         int st = 0;
@@ -897,19 +916,28 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
           if (!ok) break;
           continue;
         }
-        if (ok && KP1 < 0) {
+        if (ok && KP1 == -1) {
           // Complete graph: this thread's share of its column's sum.
           float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
           for (int r = 0; r < rows_t; ++r) cs = f4_add(cs, x4[(g_t + r * G) * QB + qoff]);
           part[gt] = cs;
         }
-        if (KP1 < 0) ok = !compute_bar_or<kCompute>(group, !ok);   // uniform decision; the column sums are visible
+        if (KP1 == -1) ok = !compute_bar_or<kCompute>(group, !ok);   // uniform decision; the column sums are visible
         if (!ok) {
           if (lane == 0) record_error(a.st, ASAP_ERR_CUDA, 0xffffffffu, a.round);
           failed = true;
           break;
         }
-        if constexpr (KP1 < 0) {
+        if constexpr (STEP) {
+          const uint32_t* xl = reinterpret_cast<const uint32_t*>(base + list_off);
+          for (int e = gt; e < info[1]; e += kCompute) {
+            const uint32_t code = xl[e];
+            if (code == kListPad) continue;
+            const int cl = static_cast<int>(code & static_cast<uint32_t>(S - 1));
+            const int i = static_cast<int>((code & kEntryOff) >> lS);
+            export_product(code, e, base, x[4 * ((i << lqb) + xq(cl >> 2)) + (cl & 3)]);
+          }
+        } else if constexpr (KP1 == -1) {
           // Complete graph: column means (threads t < nq), then every row gets them.
           if (gt < nq) {
             float4 t = part[gt];
@@ -1050,6 +1078,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       }
     }
   }
+
+  if constexpr (STEP) return;
 
   // ---- per-CTA partial, ticket, and the last CTA's finalisation ----
   F2* scratch = sm.scratch;
@@ -1218,6 +1248,12 @@ cudaError_t launch_mix(const CUtensorMap& tmap, const MixArgs& a, bool complete,
                        cudaStream_t s) {
   return dispatch(complete, mode, a.kp1, a.shadow != nullptr,
                   [&](auto k) { return decltype(k)::launch(tmap, a, grid, smem, s); });
+}
+
+cudaError_t entry_step_configure() { return MixKernel<kStepOnly, false, kMixEntries>::attr(); }
+
+cudaError_t launch_entry_step(const CUtensorMap& tmap, const MixArgs& a, int grid, size_t smem, cudaStream_t s) {
+  return MixKernel<kStepOnly, false, kMixEntries>::launch(tmap, a, grid, smem, s);
 }
 
 cudaError_t launch_cast_bf16(const float* src, uint16_t* dst, int64_t n, cudaStream_t s) {

@@ -135,3 +135,23 @@ def test_empty_minibatches_and_two_runs_bit_identical():
     for W, (lm, cm) in outs[1:]:
         assert np.array_equal(W, outs[0][0]) and np.array_equal(lm, outs[0][1][0]) and np.array_equal(cm, outs[0][1][1])
     assert abs(outs[0][1][0][1] - np.log(2.0)) <= 1e-6    # minibatch 1 is empty: the loss of m = 0
+
+
+@pytest.mark.parametrize("residency", ["device", "host"])
+@pytest.mark.parametrize("kind,k", [("root", 2), ("complete", 20)])
+def test_local_steps_of_parameters_larger_than_l2_keeps(kind, k, residency):
+    # 21 workers x 900,011 columns are 76 MB: the updates between local steps stream the slabs; a ragged last
+    # slab, columns in every slab's first and last place, runs of several rows
+    N, d, B, tau, lr, l2 = 21, 900011, 24, 3, 0.4, 0.02
+    sh = inputs.sparse_custom(seed=8, N=N, d=d, rows=7 * B, max_len=300)
+    for i in range(N):
+        ends = sh.rowptr[i][1:][np.diff(sh.rowptr[i]) > 1] - 1
+        sh.col[i][ends[::3]] = d - 1
+        starts = sh.rowptr[i][:-1][np.diff(sh.rowptr[i]) > 1]
+        sh.col[i][starts[::5]] = 0
+    rng = np.random.default_rng(3)
+    W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
+    with _make(sh, N, k, kind, "logistic", B, lr, l2=l2, tau=tau, residency=residency) as ctx:
+        before = ctx.kernel_launches()
+        _check(ctx, sh, 2, B, "logistic", lr, rounds.graph_schedule(kind, N, k, graph_seed=7), l2=l2, tau=tau, W0=W0)
+        assert ctx.kernel_launches() - before == 1 + 2 * (2 * tau)   # no separate gathers: the slabs were streamed
