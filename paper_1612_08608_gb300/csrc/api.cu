@@ -156,6 +156,7 @@ struct asap_ctx {
   cudaEvent_t staged_ev[kStaging] = {}, free_ev[kStaging] = {};
   int step_q = 1;                   // CTAs per worker (cluster size) of the local step
   int step_stages = 3;              // ring stages of the local step
+  int step_warps = 4;               // consumer warps of the local step
   size_t step_smem = 0;
   int max_nnz = 0;
 
@@ -980,6 +981,24 @@ void fill_entry_args(const asap_ctx* c, MixArgs* a, const unsigned char* bt, int
   a->B = c->B;
 }
 
+// Consumer warps of a local-step CTA: four, or more while a CTA has more than
+// one tile of its worker's largest minibatch to walk, the grid's CTAs still fit
+// on the device at once, and partial margins fit shared memory.
+int local_step_warps(const asap_ctx* c, int max_nnz) {
+  int warps = 4;
+  if (c->B > kRSmemRows) return warps;
+  const int64_t ctas = static_cast<int64_t>(c->sharded ? c->own_n : c->N) * c->step_q;
+  const int64_t share = (static_cast<int64_t>(max_nnz) + c->step_q - 1) / c->step_q + kSlotSegment;
+  while (warps < 12 && share > static_cast<int64_t>(warps) * kSlotSegment) {
+    const int next = warps + 4;
+    const size_t smem = local_step_smem_bytes(c->B, c->step_stages, next);
+    const int64_t per_sm = std::min<int64_t>(next == 8 ? 3 : 2, (227 << 10) / static_cast<int64_t>(smem + 1024));
+    if (per_sm < 1 || ctas > per_sm * c->sm_count) break;
+    warps = next;
+  }
+  return warps;
+}
+
 // eta_k of global local step k.
 float lr_at(const asap_ctx* c, int64_t k) {
   if (c->lr_kind == ASAP_LR_INVERSE) return static_cast<float>(c->lr / (1.0 + c->lr_gamma * static_cast<double>(k)));
@@ -1287,14 +1306,13 @@ asap_status asap_set_model(asap_ctx* c, asap_loss loss, int num_classes, int bat
     // keep a CTA small enough for five per SM at the usual minibatch sizes
     // (the kernel's registers are bounded for five).
     c->step_stages = 2;
-    c->step_smem = local_step_smem_bytes(batch, c->step_stages);
+    c->step_smem = local_step_smem_bytes(batch, c->step_stages, 4);
     int smem_sm = 0;
     CU(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->dev),
        "querying shared memory per SM");
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(5, smem_sm / static_cast<int64_t>(c->step_smem + 1024)));
     c->step_q = kMaxStepCluster;
     while (c->step_q > 1 && static_cast<int64_t>(c->N) * c->step_q > per_sm * c->sm_count) c->step_q >>= 1;
-    CU(local_step_configure(), "configuring the local-step kernel");
     c->permuted = false;
   } else if (loss == ASAP_LOSS_SOFTMAX) {
     c->Cq = (num_classes + 255) / 256;
@@ -1476,6 +1494,9 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
       CU(cudaMalloc(&c->mpart_big, 16 * static_cast<size_t>(N) * Q * B), "allocating the partial margins");
       CU(cudaMalloc(&c->r_big, 4 * static_cast<size_t>(N) * Q * B), "allocating the step scratch");
     }
+    c->step_warps = local_step_warps(c, max_nnz);
+    c->step_smem = local_step_smem_bytes(B, c->step_stages, c->step_warps);
+    CU(local_step_configure(c->loss, c->step_warps), "configuring the local-step kernel");
     c->nb = nb;
     c->max_nnz = max_nnz;
     c->max_region = max_region;
@@ -1684,7 +1705,7 @@ asap_status asap_local_step(asap_ctx* c) {
       a.notify = last ? 1 : 0;
       a.skip_worker = skip;
       time_begin(c, ASAP_KERNEL_LOCAL_STEP);
-      CU(launch_local_step(a, c->loss, c->step_smem, c->stream), "launching the local-step kernel");
+      CU(launch_local_step(a, c->loss, c->step_warps, c->step_smem, c->stream), "launching the local-step kernel");
       time_end(c);
     }
     c->launches += 1;

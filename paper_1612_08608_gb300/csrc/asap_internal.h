@@ -74,14 +74,16 @@ struct BatchDesc {
   int32_t pad_;
 };
 
-// Entries per ring stage of the local step (a tile), and per margin slot
-// segment (a consumer warp's 256-entry share of a tile).
-constexpr int kTileEntries = 1024;
+// Entries per margin slot segment: a consumer warp's share of a ring stage of
+// the local step (a tile of 256 entries per consumer warp).
 constexpr int kSlotSegment = 256;
 // Per-warp partial margins and r stay in shared memory for minibatches of
 // at most this many rows (else in global scratch).
 constexpr int kRSmemRows = 2048;
-constexpr int kLocalStepThreads = 192;   // four consumer warps, a bulk-copy issuer warp, a gather warp
+// Local-step threads: 4, 8 or 12 consumer warps, a bulk-copy issuer warp, and a
+// gather warp (two beside twelve consumers).
+constexpr int local_step_gather_warps(int warps) { return warps > 8 ? 2 : 1; }
+constexpr int local_step_threads(int warps) { return 32 * (warps + 1 + local_step_gather_warps(warps)); }
 constexpr int kMaxStepCluster = 8;       // CTAs per worker (portable cluster size)
 
 // Arguments of the fused sparse local step (kernels_sparse.cu): one cluster
@@ -91,7 +93,7 @@ struct LocalStepArgs {
   const BatchDesc* desc;       // [N] descriptors of this step's batch
   const float* wv;             // w values at the step's list positions
   float* gsum;                 // column sums at the step's list positions
-  float* mpart_big;            // [N][Q][4][B] per-warp partial margins (B > kRSmemRows only)
+  float* mpart_big;            // [N][Q][4][B] per-warp partial margins (B > kRSmemRows only: four warps)
   float* r_big;                // [N][Q][B] r (B > kRSmemRows only)
   float* loss_part;            // [N]: minibatch loss sum per worker
   unsigned int* ready;         // NOTIFY flags [N]
@@ -238,9 +240,9 @@ asap_status build_graph_host(asap_graph_kind kind, int N, int k, uint64_t seed, 
                              int32_t* nbr, const char** why);
 
 // Launchers (kernels_*.cu).  Each returns the cudaError_t of the launch.
-cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cudaStream_t s);
-size_t local_step_smem_bytes(int B, int stages);
-cudaError_t local_step_configure();
+cudaError_t launch_local_step(const LocalStepArgs& a, int loss, int warps, size_t smem, cudaStream_t s);
+size_t local_step_smem_bytes(int B, int stages, int warps);
+cudaError_t local_step_configure(int loss, int warps);
 cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
                                 int S, int max_region, const float* gsum, float scale, int sm_count, cudaStream_t s);
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,

@@ -20,18 +20,19 @@
 // streamed twice through a ring of shared-memory stages by an issuer warp
 // with bulk copies (cp.async.bulk, mbarrier completion) -- a gather warp
 // fetches a margin tile's w values as soon as the tile lands -- while four
-// consumer warps work on the stage that has landed, each on its own
-// 256-entry share of the 1024-entry tile and without CTA-wide barriers:
+// consumer warps (eight or twelve where workers are few) work on the stage that
+// has landed, each on its own 256-entry share of the tile and without CTA-wide
+// barriers:
 //   pass 1 (margins): CTA q takes the 256-entry segments s = q nseg/Q ...
-//     in tiles of four; a warp's products val * wv[pos] and their rows go to
+//     in tiles of one segment per warp; a warp's products val * wv[pos] and their rows go to
 //     shared memory at the entry's slot (slots of a 256-entry segment
 //     ordered by row, then column), a segmented scan over the slots keyed by
 //     row sums each row's products in order, and the warp adds them to its
-//     own partial margins.  The four warps' partials are added in order; a
+//     own partial margins.  The warps' partials are added in order; a
 //     cluster barrier; every CTA then adds the Q partials of each row in rank
 //     order (distributed shared memory), forms r and, in CTA 0, the loss sum.
 //   pass 2 (column sums): CTA q takes the entries [bnd[q], bnd[q+1]), cut
-//     at column boundaries, in 1024-entry tiles; a warp's segmented scan
+//     at column boundaries, in tiles; a warp's segmented scan
 //     keyed by list position sums each column's r_row * val; runs that end
 //     inside the warp's share are stored by the warp, and the two runs at
 //     its edges are fragments that the gather warp, idle by then, adds up
@@ -52,8 +53,7 @@ namespace asap {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kConsumers = kLocalStepThreads - 64;          // four consumer warps
-constexpr int kPerThread = kTileEntries / kConsumers;       // consecutive entries per consumer thread
+constexpr int kPerThread = kSlotSegment / 32;               // consecutive entries per consumer thread
 static_assert(kPerThread == 8, "a consumer thread takes 8 consecutive entries of a tile");
 constexpr unsigned long long kCopyWaitNs = 2000000000ull;   // a bulk copy never takes this long
 
@@ -148,8 +148,9 @@ __device__ __forceinline__ float ld_dsmem(const float* local, uint32_t rank) {
 }
 
 // Barrier among the consumer warps only (the producer warp keeps streaming).
+template <int THREADS>
 __device__ __forceinline__ void consumer_bar() {
-  asm volatile("bar.sync 1, %0;" :: "n"(kConsumers) : "memory");
+  asm volatile("bar.sync 1, %0;" :: "n"(THREADS) : "memory");
 }
 
 __device__ __forceinline__ void record_error(DevState* st, unsigned code, unsigned worker, unsigned round) {
@@ -188,21 +189,19 @@ struct StepSmem {
   uint64_t* gath;       // [stages]: the w values of a margin tile are in the stage
   uint64_t* fready;     // [kFragRing]: every warp has left its fragments of a column-sum tile
   uint64_t* ffree;      // [kFragRing]: the merger has read a slot's fragments
-  float* prod;          // [kTileEntries]: warp w uses [256 w, 256 w + 256)
-  int* okey;            // [kTileEntries]: list position of a run ending at the pair, else -1
-  float* mpart;         // [4][B]: per-warp partial margins (warp 0's row holds the CTA's sum after pass 1)
+  float* prod;          // [256 W]: warp w uses [256 w, 256 w + 256)
+  int* okey;            // [256 W]: list position of a run ending at the pair, else -1
+  float* mpart;         // [W][B]: per-warp partial margins (warp 0's row holds the CTA's sum after pass 1)
   float* r;             // [B]
-  int* fkey;            // [kFragRing][4][2]: first / last column-run fragment of each warp's sub-tile
-  float* fval;          // [kFragRing][4][2]
-  float* red;           // [kConsumers / 32]
+  int* fkey;            // [kFragRing][W][2]: first / last column-run fragment of each warp's sub-tile
+  float* fval;          // [kFragRing][W][2]
+  float* red;           // [W]
   int* ctl;             // [1]: a copy timed out
 };
 
 // pos (in margin tiles overwritten by the gathered w values), val and two
 // uint16 arrays
-constexpr size_t kStageBytes = static_cast<size_t>(kTileEntries) * 12;
-constexpr int kWarps = kConsumers / 32;
-constexpr int kIssuerWarp = kWarps, kGatherWarp = kWarps + 1;
+constexpr size_t stage_bytes(int W) { return static_cast<size_t>(W) * kSlotSegment * 12; }
 // Fragments of a column-sum tile wait in a ring until the merger (the gather
 // warp, idle in pass 2) has added them up; a consumer waits for the slot's
 // "free" barrier before it reuses it.
@@ -213,11 +212,13 @@ constexpr int kNoKey = -2;
 // integer round trip of the address), so that the compiler keeps the
 // pointers in the shared address space and emits plain shared-memory
 // accesses.
+template <int kWarps>
 __device__ __forceinline__ StepSmem carve_step(unsigned char* raw, int B, int stages) {
+  constexpr int kTileEntries = kWarps * kSlotSegment;
   StepSmem m;
   size_t off = (128u - (smem_u32(raw) & 127u)) & 127u;   // 128-byte aligned stages
   m.stage0 = raw + off;
-  off += kStageBytes * stages;
+  off += stage_bytes(kWarps) * stages;
   m.full = reinterpret_cast<uint64_t*>(raw + off);
   off += 8 * stages;
   m.empty = reinterpret_cast<uint64_t*>(raw + off);
@@ -295,11 +296,22 @@ __device__ __forceinline__ void seg_scan_warp(const int (&key)[kPerThread], floa
   }
 }
 
-template <int LOSS>
-__global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const LocalStepArgs a) {   // five CTAs per SM
+// kWarps consumer warps, each with its own 256-entry share of a tile.  Four keep
+// a CTA small enough for five per SM (the registers are bounded for that).  Few
+// workers leave an SM one or two CTAs, and a CTA several tiles to walk in each
+// pass, about 1.3 and 1.5 us each: then eight or twelve (local_step_warps; the
+// RCV1-shaped round, 2,670 entries a CTA: 34.4 us with four, 29.2 with eight,
+// 25.7 with twelve; sixteen, one CTA per SM, 31.0).
+template <int LOSS, int kWarps>
+__global__ void __launch_bounds__(local_step_threads(kWarps), kWarps == 4 ? 5 : kWarps == 8 ? 3 : 2)
+    k_local_step(const LocalStepArgs a) {
+  constexpr int kLocalStepThreads = local_step_threads(kWarps), kConsumers = kWarps * 32;
+  constexpr int kTileEntries = kWarps * kSlotSegment;
+  constexpr size_t kStageBytes = stage_bytes(kWarps);
+  constexpr int kIssuerWarp = kWarps, kGatherWarp = kWarps + 1, kGatherWarps = local_step_gather_warps(kWarps);
   extern __shared__ unsigned char step_smem_raw[];
   const bool big = a.B > kRSmemRows;           // partial margins and r in global memory
-  const StepSmem sm = carve_step(step_smem_raw, big ? 0 : a.B, a.stages);
+  const StepSmem sm = carve_step<kWarps>(step_smem_raw, big ? 0 : a.B, a.stages);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = static_cast<int>(cluster_rank());
   const int Q = a.Q;
@@ -329,7 +341,7 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
     for (int st = 0; st < a.stages; ++st) {
       mbar_init(sm.full + st, 1);
       mbar_init(sm.empty + st, kWarps);
-      mbar_init(sm.gath + st, 32);
+      mbar_init(sm.gath + st, 32 * kGatherWarps);
     }
     for (int f = 0; f < kFragRing; ++f) {
       mbar_init(sm.fready + f, kWarps);
@@ -388,8 +400,8 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
     }
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  } else if (warp == kGatherWarp) {
-    // ================= gather warp =================
+  } else if (warp >= kGatherWarp) {
+    // ================= gather warp(s) =================
     // As soon as margin tile k has landed, every lane gathers 32 of its w
     // values with 4-byte asynchronous copies, each over the list position
     // it was addressed by (read before the copy is issued), and arrives on
@@ -405,7 +417,7 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
       const int len = min(kTileEntries, p1_end - (p1_begin + k * kTileEntries));
       // four consecutive positions per lane and vector load, two loads ahead
       // of their copies, so that no copy waits on its own position's load
-      for (int j0 = lane * 4; j0 < len; j0 += 256) {
+      for (int j0 = lane * 4 + (warp - kGatherWarp) * 256; j0 < len; j0 += 256 * kGatherWarps) {
         const int j1 = j0 + 128;
         const int4 p0 = *reinterpret_cast<const int4*>(spos + j0);
         const int4 p1 = j1 < len ? *reinterpret_cast<const int4*>(spos + j1) : make_int4(0, 0, 0, 0);
@@ -427,37 +439,40 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
     int open_key = kNoKey;                     // lane 0: the run the fragments continue
     float open_sum = 0.f;
     bool mok = gok;
-    for (int k = 0; k < n2 && mok; ++k) {
+    for (int k = 0; k < n2 && mok && warp == kGatherWarp; ++k) {
       const int slot = k % kFragRing;
       mok = __all_sync(kFull, mbar_wait_bounded(sm.fready + slot, (k / kFragRing) & 1));
       if (!mok) break;
       if (lane == 0) {
-        static_assert(kWarps * 2 == 8, "a tile leaves eight fragments");
+        static_assert(kWarps % 4 == 0, "a tile's fragments are read eight at a time");
         const int fb = slot * kWarps * 2;
-        const int4 k0 = *reinterpret_cast<const int4*>(sm.fkey + fb);
-        const int4 k1 = *reinterpret_cast<const int4*>(sm.fkey + fb + 4);
-        const float4 v0 = *reinterpret_cast<const float4*>(sm.fval + fb);
-        const float4 v1 = *reinterpret_cast<const float4*>(sm.fval + fb + 4);
-        const int fks[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-        const float fvs[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-        mbar_arrive(sm.ffree + slot);          // the slot is read
 #pragma unroll
-        for (int f = 0; f < 8; ++f) {
-          const int fk = fks[f];
-          if (fk == kNoKey) continue;
-          const float fv = fvs[f];
-          if (fk == open_key) {
-            open_sum += fv;
-          } else {
-            if (open_key >= 0) g[open_key] = open_sum;
-            open_key = fk;
-            open_sum = fv;
+        for (int f0 = 0; f0 < kWarps * 2; f0 += 8) {
+          const int4 k0 = *reinterpret_cast<const int4*>(sm.fkey + fb + f0);
+          const int4 k1 = *reinterpret_cast<const int4*>(sm.fkey + fb + f0 + 4);
+          const float4 v0 = *reinterpret_cast<const float4*>(sm.fval + fb + f0);
+          const float4 v1 = *reinterpret_cast<const float4*>(sm.fval + fb + f0 + 4);
+          const int fks[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+          const float fvs[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+          if (f0 + 8 == kWarps * 2) mbar_arrive(sm.ffree + slot);   // the slot is read
+#pragma unroll
+          for (int f = 0; f < 8; ++f) {
+            const int fk = fks[f];
+            if (fk == kNoKey) continue;
+            const float fv = fvs[f];
+            if (fk == open_key) {
+              open_sum += fv;
+            } else {
+              if (open_key >= 0) g[open_key] = open_sum;
+              open_key = fk;
+              open_sum = fv;
+            }
           }
         }
       }
       __syncwarp();
     }
-    if (lane == 0 && mok && open_key >= 0) g[open_key] = open_sum;
+    if (lane == 0 && mok && open_key >= 0) g[open_key] = open_sum;   // (the other gather warps have none)
     if (!mok && lane == 0) {
       record_error(a.st, ASAP_ERR_CUDA, static_cast<unsigned>(i), a.round);
       sm.ctl[0] = 1;
@@ -530,7 +545,7 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
       }
     }
     // ---- the CTA's partial margins: the four warps' rows added in order ----
-    consumer_bar();
+    consumer_bar<kConsumers>();
     for (int b = tid; b < a.B; b += kConsumers) {
       if (big) {
         float m = gpart[b];
@@ -580,7 +595,7 @@ __global__ void __launch_bounds__(kLocalStepThreads, 5) k_local_step(const Local
       lsum = warp_sum(lsum);
       if (lane == 0) sm.red[warp] = lsum;
     }
-    consumer_bar();
+    consumer_bar<kConsumers>();
     if (q == 0 && tid == 0) {
       float tot = 0.f;
       for (int w2 = 0; w2 < kWarps; ++w2) tot += sm.red[w2];
@@ -770,26 +785,37 @@ cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, cons
   return cudaGetLastError();
 }
 
-size_t local_step_smem_bytes(int B, int stages) {
+size_t local_step_smem_bytes(int B, int stages, int warps) {
   const size_t b_smem = B > kRSmemRows ? 0 : static_cast<size_t>(B);
-  return 128 + kStageBytes * stages + 24 * static_cast<size_t>(stages) + 16 * kFragRing + 16 + 8 * kTileEntries +
-         4 * (kWarps + 1) * b_smem + 16 + 8 * kFragRing * kWarps * 2 + 4 * kWarps + 4;
+  return 128 + stage_bytes(warps) * stages + 24 * static_cast<size_t>(stages) + 16 * kFragRing + 16 +
+         8 * static_cast<size_t>(warps) * kSlotSegment + 4 * (static_cast<size_t>(warps) + 1) * b_smem + 16 +
+         8 * static_cast<size_t>(kFragRing) * warps * 2 + 4 * static_cast<size_t>(warps) + 4;
+}
+
+// Calls f with the kernel for a loss and a number of consumer warps.
+template <typename F>
+static cudaError_t with_kernel(int loss, int warps, F&& f) {
+  if (loss == ASAP_LOSS_HINGE)
+    return warps == 12  ? f(k_local_step<ASAP_LOSS_HINGE, 12>)
+           : warps == 8 ? f(k_local_step<ASAP_LOSS_HINGE, 8>)
+                        : f(k_local_step<ASAP_LOSS_HINGE, 4>);
+  return warps == 12  ? f(k_local_step<ASAP_LOSS_LOGISTIC, 12>)
+         : warps == 8 ? f(k_local_step<ASAP_LOSS_LOGISTIC, 8>)
+                      : f(k_local_step<ASAP_LOSS_LOGISTIC, 4>);
 }
 
 // The limit is the functions', shared by contexts of other minibatch sizes:
 // always the device's (227 KB).
-cudaError_t local_step_configure() {
-  cudaError_t e = cudaFuncSetAttribute(k_local_step<ASAP_LOSS_HINGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       227 << 10);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_local_step<ASAP_LOSS_LOGISTIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              227 << 10);
+cudaError_t local_step_configure(int loss, int warps) {
+  return with_kernel(loss, warps, [](auto kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
+  });
 }
 
-cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cudaStream_t s) {
+cudaError_t launch_local_step(const LocalStepArgs& a, int loss, int warps, size_t smem, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.N * a.Q);
-  cfg.blockDim = dim3(kLocalStepThreads);
+  cfg.blockDim = dim3(local_step_threads(warps));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -803,8 +829,7 @@ cudaError_t launch_local_step(const LocalStepArgs& a, int loss, size_t smem, cud
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (loss == ASAP_LOSS_HINGE) return cudaLaunchKernelEx(&cfg, k_local_step<ASAP_LOSS_HINGE>, a);
-  return cudaLaunchKernelEx(&cfg, k_local_step<ASAP_LOSS_LOGISTIC>, a);
+  return with_kernel(loss, warps, [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, a); });
 }
 
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
