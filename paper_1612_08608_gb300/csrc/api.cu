@@ -139,6 +139,7 @@ struct asap_ctx {
     size_t y, len, soff, code, val, place;
   };
   bool entries = false;
+  bool stream_slabs = false;        // local steps before a round's last stream the slabs (launch_entry_step)
   std::vector<EntryOffsets> entry_off;
   int64_t row_stride = 0;           // floats per row of the table of products
   int row_q = 0, row_rows = 0;      // local-step CTAs per worker, rows per CTA
@@ -250,6 +251,7 @@ void free_shards(asap_ctx* c) {
   dfree(c->r_big);
   dfree(c->r_ent);
   c->entries = false;
+  c->stream_slabs = false;
   c->entry_off.clear();
   for (int b = 0; b < asap_ctx::kStaging; ++b) {
     dfree(c->staging[b]);
@@ -940,6 +942,14 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   c->row_stride = stride;
   c->max_region = max_region;
   c->entries = true;
+  // A local step before a round's last: stream every slab once, for its update
+  // and the next step's products, or touch the entries' parameters one by one,
+  // twice.  Streaming pays from about one parameter in 24 touched (N = 64, d =
+  // 2^20, one in 20: 106 us against 75 + 57; N = 20, d = 200,000, one in 17: 16.0
+  // against 10.2 + 8.7; N = 16, d = 10^6, one in 83: 22.6 against 11.2 + 9.6; N =
+  // 70, d = 230,000, one in 230: 33 against 8 + 8) and two slabs' worth of them.
+  const int64_t params = static_cast<int64_t>(N) * c->ld;
+  c->stream_slabs = 24 * max_nnz >= params && params >= 16384;
   return ASAP_OK;
 }
 
@@ -1716,9 +1726,7 @@ asap_status asap_local_step(asap_ctx* c) {
       // w_stored -= eta / (B s') g at the step's columns; the reduce applies
       // the round's last update itself, except in a worker-sharded context,
       // whose owned rows must hold x - eta g before they are sent.
-      // Where W does not stay in L2 between two kernels (64 MB: half of it), the
-      // slabs are streamed once for the update and the next step's products.
-      const bool stream_slabs = c->entries && !last && static_cast<size_t>(c->N) * c->ld * 4 > (64u << 20);
+      const bool stream_slabs = c->stream_slabs && !last;
       const unsigned char* next = nullptr;
       if (stream_slabs) {
         asap_status sn = block_of(c, k + 1, &next);

@@ -203,7 +203,7 @@ __device__ __forceinline__ void slab_update(float* W, int64_t ld, const EntryLis
 }
 
 template <int TPS>
-__global__ void __launch_bounds__(kThreads) k_entry_products(const float* W, int64_t ld, const EntryList x,
+__global__ void __launch_bounds__(kThreads, 4) k_entry_products(const float* W, int64_t ld, const EntryList x,
                                                              long long n_slabs, int lS, float* prod, int B,
                                                              int64_t stride) {
   const int t = threadIdx.x % TPS;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThreads) k_entry_products(const float* W, int
 }
 
 template <int TPS>
-__global__ void __launch_bounds__(kThreads) k_entry_update(float* W, int64_t ld, const EntryList x,
+__global__ void __launch_bounds__(kThreads, 4) k_entry_update(float* W, int64_t ld, const EntryList x,
                                                            long long n_slabs, int lS, const float* r, int B,
                                                            float scale) {
   const int t = threadIdx.x % TPS;

@@ -505,11 +505,11 @@ __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs&
 // KP1 == 0: sparse graph, runtime a.kp1 (<= kMaxKp1Sparse);
 // KP1 == -1: complete graph with equal weights;
 // KP1 == kStepOnly (entry layout): no mixing, but the update of a local step
-// before a round's last, stored in place, and the next step's products, for
-// parameters that do not stay in L2.  The slabs are streamed whole: touched one
-// by one (kernels_entry.cu), two thirds of a hashed slab's 32-byte sectors cost a
-// 64-byte DRAM access each, twice (N = 64, d = 2^20, ~400 entries a slab:
-// update 75.5 us, products 57.3; so, both 105.8 us).
+// before a round's last, stored in place, and the next step's products.  The
+// slabs are streamed whole: touched one by one (kernels_entry.cu), a third of a
+// hashed slab's 32-byte sectors cost a 64-byte DRAM access each, twice (N = 64,
+// d = 2^20, ~400 entries a slab: update 75.5 us, products 57.3; so, both 105.8
+// us).  Where entries are few it is the other way round (load_entries).
 constexpr int kStepOnly = -2;
 
 template <int KP1, bool SHADOW, int MODE>
