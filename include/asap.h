@@ -147,7 +147,8 @@ asap_status asap_set_stream(asap_ctx* ctx, void* cuda_stream);
 asap_status asap_set_shard_residency(asap_ctx* ctx, asap_residency residency);
 
 /* Bytes of the minibatch block that round `round` reads (all workers: the
- * padded CSR rows, labels and the column-sorted copy).  With HOST residency
+ * labels and the entries with their index, about 10 bytes an entry where
+ * columns are spread evenly, 16 where they are skewed).  With HOST residency
  * this is what one round copies to the GPU.  Host only. */
 asap_status asap_shard_block_bytes(asap_ctx* ctx, int64_t round, uint64_t* bytes);
 
@@ -156,8 +157,10 @@ asap_status asap_shard_block_bytes(asap_ctx* ctx, int64_t round, uint64_t* bytes
  * at 0; col[i] / val[i] have rowptr[i][n_rows[i]] entries; col ids in
  * [0, d), distinct within a row; y[i] has n_rows[i] labels in {-1, +1}.
  * Every worker needs n_rows[i] >= B.  The library builds, once, the batch
- * layout the kernels read (rows padded to 4 entries; per batch a copy
- * sorted by (column, row)).  Synchronous. */
+ * layout the kernels read: per minibatch the entries by the reduce's column
+ * slabs where columns are spread evenly (no slab and no column with many
+ * entries), else sorted by (column, row) per worker with a list of distinct
+ * columns.  Synchronous. */
 asap_status asap_load_shards(asap_ctx* ctx, const int64_t* const* rowptr, const int32_t* const* col,
                              const float* const* val, const float* const* y, const int64_t* n_rows);
 
@@ -344,12 +347,13 @@ asap_status asap_debug_batch_image(int N, int64_t d, int batch, int slab_cols, i
 
 /* Kernel kinds for per-kernel timing. */
 typedef enum {
-  ASAP_KERNEL_LOCAL_STEP = 0, /* sparse margins, loss derivative, column sums,
-                                 NOTIFY (a2-a4), one fused kernel               */
+  ASAP_KERNEL_LOCAL_STEP = 0, /* sparse margins, loss derivative, NOTIFY (a2-a4),
+                                 and for skewed columns the column sums        */
   ASAP_KERNEL_REDUCE = 1,     /* stochastic reduce + ACK + metrics (a5-a7, a9)  */
   ASAP_KERNEL_DENSE_FWD = 2,  /* dense logits, softmax, R^T (a3')               */
   ASAP_KERNEL_DENSE_GRAD = 3, /* dense gradient GEMM + update + NOTIFY (a3')    */
-  ASAP_KERNEL_APPLY = 4,      /* update of a local step before the round's last */
+  ASAP_KERNEL_APPLY = 4,      /* update of a local step before the round's last,
+                                 where W is streamed with the next step's gather */
   ASAP_KERNEL_GATHER = 5,     /* w at a step's columns from the stored W        */
   ASAP_KERNEL_KINDS = 6
 } asap_kernel_kind;

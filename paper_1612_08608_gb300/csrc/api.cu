@@ -142,6 +142,7 @@ struct asap_ctx {
   bool stream_slabs = false;        // local steps before a round's last stream the slabs (launch_entry_step)
   std::vector<EntryOffsets> entry_off;
   int64_t row_stride = 0;           // floats per row of the table of products
+  int row_shift = 16;               // EntryList::row_shift
   int row_q = 0, row_rows = 0;      // local-step CTAs per worker, rows per CTA
   float* r_ent = nullptr;           // [N][B] r of the last local step's rows
   float* wv[2] = {nullptr, nullptr};  // w at the list positions (entries: the products) of round t's steps: wv[t & 1]
@@ -724,8 +725,9 @@ bool count_entries(int N, int B, int64_t d, int lS, int t, const int64_t* const*
   return true;
 }
 
-void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int t, const int64_t* const* rowptr,
-                       const int32_t* const* col, const float* const* val, const float* const* y, EntryImage& im) {
+void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int row_shift, int t,
+                       const int64_t* const* rowptr, const int32_t* const* col, const float* const* val,
+                       const float* const* y, EntryImage& im) {
   const int lS = __builtin_ctz(static_cast<unsigned>(S));
   std::vector<int32_t> at(static_cast<size_t>(n_slabs) * N, 0);
   if (!count_entries(N, B, d, lS, t, rowptr, col, at, &im.err)) return;
@@ -735,6 +737,7 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int t,
     n = static_cast<int32_t>(tot);
     tot += c;
   }
+  const bool packed = row_shift > 16;   // the place is in the code
   // Entries by (slab, worker), in row order so far.
   struct Item {
     uint32_t code;
@@ -750,8 +753,9 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int t,
       for (int64_t e0 = rp[r0 + b], e = e0; e < rp[r0 + b + 1]; ++e) {
         const int32_t cc = col[i][e];
         items[at[static_cast<size_t>(cc >> lS) * N + i]++] =
-            Item{(static_cast<uint32_t>(b) << 16) | static_cast<uint32_t>(i * S + (cc & (S - 1))), val[i][e],
-                 static_cast<uint16_t>(e - e0)};
+            Item{(static_cast<uint32_t>(b) << row_shift) | (packed ? static_cast<uint32_t>(e - e0) << 16 : 0u) |
+                     static_cast<uint32_t>(i * S + (cc & (S - 1))),
+                 val[i][e], static_cast<uint16_t>(e - e0)};
       }
   }
   // Then by column, keeping that order within a column, and into regions of
@@ -813,7 +817,7 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int t,
   im.off.soff = take(4 * soff.size());
   im.off.code = take(4 * code.size());
   im.off.val = take(4 * code.size());
-  im.off.place = take(2 * code.size());
+  im.off.place = packed ? 0 : take(2 * code.size());
   im.img.assign(align_up(off, 256), 0);
   unsigned char* base = im.img.data();
   float* y_o = reinterpret_cast<float*>(base + im.off.y);
@@ -822,7 +826,7 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int t,
   if (!code.empty()) {
     std::memcpy(base + im.off.code, code.data(), 4 * code.size());
     std::memcpy(base + im.off.val, vals.data(), 4 * code.size());
-    std::memcpy(base + im.off.place, place.data(), 2 * code.size());
+    if (!packed) std::memcpy(base + im.off.place, place.data(), 2 * code.size());
   }
   for (int i = 0; i < N; ++i) {
     const int64_t* rp = rowptr[i];
@@ -918,7 +922,14 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
     }
   }
   std::vector<EntryImage> built(nb);
-  for_batches(nb, [&](int t) { build_entry_image(N, B, c->d, c->S, c->n_slabs, t, rowptr, col, val, y, built[t]); });
+  // Row and place share 16 bits of the code where both fit.
+  int place_bits = 1, row_bits = 0;
+  while ((1ll << place_bits) < max_len) ++place_bits;
+  while ((1 << row_bits) < B) ++row_bits;
+  c->row_shift = place_bits + row_bits <= 16 && place_bits < 16 ? 16 + place_bits : 16;
+  for_batches(nb, [&](int t) {
+    build_entry_image(N, B, c->d, c->S, c->n_slabs, c->row_shift, t, rowptr, col, val, y, built[t]);
+  });
   int max_region = 0;
   for (const EntryImage& im : built) {
     if (im.err) return fail(c, ASAP_ERR_ARG, im.err);
@@ -950,6 +961,7 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   // 70, d = 230,000, one in 230: 33 against 8 + 8) and two slabs' worth of them.
   const int64_t params = static_cast<int64_t>(N) * c->ld;
   c->stream_slabs = 24 * max_nnz >= params && params >= 16384;
+  if (c->stream_slabs) CU(entry_step_configure(), "configuring the local update kernel");
   return ASAP_OK;
 }
 
@@ -959,7 +971,8 @@ EntryList entry_list(const asap_ctx* c, const unsigned char* block, int t) {
   EntryList x;
   x.code = reinterpret_cast<const uint32_t*>(block + o.code);
   x.val = reinterpret_cast<const float*>(block + o.val);
-  x.place = reinterpret_cast<const uint16_t*>(block + o.place);
+  x.place = c->row_shift > 16 ? nullptr : reinterpret_cast<const uint16_t*>(block + o.place);
+  x.row_shift = c->row_shift;
   x.off = reinterpret_cast<const int*>(block + o.soff);
   return x;
 }
@@ -1733,7 +1746,6 @@ asap_status asap_local_step(asap_ctx* c) {
         if (sn != ASAP_OK) return sn;
         sn = configure_mix_launch(c, kMixEntries);
         if (sn != ASAP_OK) return sn;
-        CU(entry_step_configure(), "configuring the local update kernel");
       }
       time_begin(c, ASAP_KERNEL_APPLY);
       if (stream_slabs) {

@@ -2,8 +2,8 @@
 // evenly (Eq. A.1, first line): the entry layout.
 //
 // The minibatch is stored once, cut into the column slabs of the stochastic
-// reduce: per slab its entries by (worker, column, row), each a code (row <<
-// 16 | run flags | worker * S + column in the slab), a value and a place in its row.  The
+// reduce: per slab its entries by (worker, column, row), each a code (row,
+// run flags, worker * S + column in the slab), a value and a place in its row.  The
 // kernels that hold a slab do all the work that is indexed by column:
 //   * the reduce of the round before (or the gather below) multiplies each
 //     entry's value by w at its column and stores the product at the entry's
@@ -17,8 +17,8 @@
 // position, exchanges partial margins across a cluster and scans column sums,
 // the local step of hashed logistic regression (N = 64, d = 2^20, B = 512, 100
 // entries a row) went from 47 to 11.5 us and the reduce from 106 to 128 us (150
-// to 132 us a round), and a minibatch takes 10 instead of 16 bytes an entry
-// (250 to 160 us a round with host-resident shards, which the copy bounds).  It needs slabs with few
+// to 132 us a round), and a minibatch takes 8 or 10 instead of 16 bytes an entry
+// (250 to 140 us a round with host-resident shards, which the copy bounds).
 // entries and columns with short runs (kEntryRegion, kEntryRun); skewed
 // columns stay with the list layout.
 #include <cuda_runtime.h>
@@ -153,14 +153,17 @@ __device__ __forceinline__ void slab_products(const float* W, int64_t ld, const 
       const int e = e0 + TPS * u;
       code[u] = e < a1 ? x.code[e] : kListPad;
       v[u] = e < a1 ? x.val[e] : 0.f;
-      k[u] = e < a1 ? x.place[e] : 0;
+      k[u] = e >= a1 ? 0
+             : x.place ? x.place[e]
+                       : static_cast<int>((code[u] >> 16) & ((1u << (x.row_shift - 16)) - 1u));
     }
 #pragma unroll
     for (int u = 0; u < kU; ++u) w[u] = code[u] != kListPad ? __ldcg(W + param_of(code[u], s, lS, ld)) : 0.f;
 #pragma unroll
     for (int u = 0; u < kU; ++u)
       if (code[u] != kListPad)
-        prod[(static_cast<int64_t>((code[u] & kEntryOff) >> lS) * B + (code[u] >> 16)) * stride + k[u]] = v[u] * w[u];
+        prod[(static_cast<int64_t>((code[u] & kEntryOff) >> lS) * B + (code[u] >> x.row_shift)) * stride + k[u]] =
+            v[u] * w[u];
   }
 }
 
@@ -185,7 +188,7 @@ __device__ __forceinline__ void slab_update(float* W, int64_t ld, const EntryLis
 #pragma unroll
     for (int u = 0; u < kU; ++u)
       if (head[u]) {
-        g[u] *= __ldcg(r + static_cast<int64_t>((code[u] & kEntryOff) >> lS) * B + (code[u] >> 16));
+        g[u] *= __ldcg(r + static_cast<int64_t>((code[u] & kEntryOff) >> lS) * B + (code[u] >> x.row_shift));
         w[u] = W[param_of(code[u], s, lS, ld)];
       }
 #pragma unroll
@@ -195,7 +198,7 @@ __device__ __forceinline__ void slab_update(float* W, int64_t ld, const EntryLis
         uint32_t c = code[u];
         for (int e = e0 + TPS * u + 1; c & kEntryMore; ++e) {
           c = x.code[e];
-          g[u] = fmaf(__ldcg(r + r0 + (c >> 16)), x.val[e], g[u]);
+          g[u] = fmaf(__ldcg(r + r0 + (c >> x.row_shift)), x.val[e], g[u]);
         }
         W[param_of(code[u], s, lS, ld)] = fmaf(-scale, g[u], w[u]);
       }

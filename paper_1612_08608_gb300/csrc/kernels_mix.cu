@@ -390,7 +390,9 @@ __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs&
   constexpr int kUpd = kMixUpdaterWarps * 32, kU = 5, kAhead = 2;
   const int ut = threadIdx.x - kUpdater0 * 32, lane = threadIdx.x & 31;
   const int S = 1 << lS, QB = 1 << lqb;
-  auto r_at = [&](uint32_t c) { return a.r + static_cast<int64_t>((c & kEntryOff) >> lS) * a.B + (c >> 16); };
+  auto r_at = [&](uint32_t c) {
+    return a.r + static_cast<int64_t>((c & kEntryOff) >> lS) * a.B + (c >> a.upd.row_shift);
+  };
   int fsl = 0, sl = 0, st = 0;         // ring positions: entries being fetched, entries and stage being used
   uint32_t fph = 0, ph = 0;            // and phases
   uint32_t early = 0;                  // bit d: r of the slab d ahead is on its way
@@ -714,7 +716,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             n_upd = o.y - o.x;
             x0 = o.z;
             n_exp = o.w - o.z;
-            bytes += ENTRIES ? 10u * n_exp : 8u * n_upd + 4u * n_exp;
+            bytes += ENTRIES ? (a.exp.place ? 10u : 8u) * n_exp : 8u * n_upd + 4u * n_exp;
           }
           *reinterpret_cast<int4*>(sm.info + 4 * st) = make_int4(n_upd, n_exp, x0, u0);
           mbar_expect_only(sm.full + st, bytes);
@@ -727,7 +729,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             if (n_exp > 0) {
               bulk_load(base + list_off, a.exp.code + x0, 4u * n_exp, sm.full + st);
               bulk_load(base + list_off + list_bytes, a.exp.val + x0, 4u * n_exp, sm.full + st);
-              bulk_load(base + list_off + 2 * list_bytes, a.exp.place + x0, 2u * n_exp, sm.full + st);
+              if (a.exp.place)
+                bulk_load(base + list_off + 2 * list_bytes, a.exp.place + x0, 2u * n_exp, sm.full + st);
             }
           } else if (FUSED) {
             if (n_upd > 0) {
@@ -867,8 +870,9 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // Entry layout: value * w of the stage's export entry e, to its row.
       auto export_product = [&](uint32_t code, int e, const unsigned char* base, float w) {
         const float val = reinterpret_cast<const float*>(base + list_off + list_bytes)[e];
-        const int place = reinterpret_cast<const uint16_t*>(base + list_off + 2 * list_bytes)[e];
-        const int64_t row = static_cast<int64_t>((code & kEntryOff) >> lS) * a.B + (code >> 16);
+        const uint32_t place = a.exp.place ? reinterpret_cast<const uint16_t*>(base + list_off + 2 * list_bytes)[e]
+                                           : (code >> 16) & ((1u << (a.exp.row_shift - 16)) - 1u);
+        const int64_t row = static_cast<int64_t>((code & kEntryOff) >> lS) * a.B + (code >> a.exp.row_shift);
         st_f32_hint(a.prod_out + row * a.row_stride + place, val * w, keep);
       };
       // With a compile-time neighbour count and at most kCacheRows rows per

@@ -3,7 +3,7 @@ slabs: products exported by the reduce, row sums, updates from the rows' r
 inside the reduce) against the oracle, round by round (1e-5 normwise per
 worker), at the edges of its row passes, runs and regions, and on both sides
 of the rule that chooses it.  Which layout a context uses shows in the bytes of
-a minibatch block: 10 an entry (plus padding) against 16."""
+a minibatch block: 8 or 10 an entry (plus padding) against 16."""
 import numpy as np
 import pytest
 
@@ -158,3 +158,16 @@ def test_local_steps_streamed_and_touched(kind, k, residency, max_len, streams):
         _check(ctx, sh, 2, B, "logistic", lr, rounds.graph_schedule(kind, N, k, graph_seed=7), l2=l2, tau=tau, W0=W0)
         # one gather at the start; per round tau steps, tau - 1 updates (and gathers, unless streamed), a reduce
         assert ctx.kernel_launches() - before == 1 + 2 * (2 * tau if streams else 3 * tau - 1)
+
+
+@pytest.mark.parametrize("B,row_len,packed", [(512, 128, True), (512, 129, False), (513, 128, False), (2, 4000, True),
+                                              (1, 5000, True), (1024, 64, True), (1025, 64, False)])
+def test_row_and_place_in_the_code(B, row_len, packed):
+    # row and place share 16 bits where they fit: bits of the row + bits of the place <= 16
+    N, d = 2, 600011
+    sh = inputs.sparse_custom(seed=B, N=N, d=d, rows=2 * B, lengths=[np.full(2 * B, row_len)] * N)
+    W0 = (0.1 * np.random.default_rng(2).standard_normal((N, d))).astype(np.float32)
+    with _make(sh, N, 1, "complete", "logistic", B, 0.5, tau=2) as ctx:
+        E = N * B * row_len
+        assert (ctx.shard_block_bytes(0) < 9.9 * E + 6 * N * B + 4096) == packed, ctx.shard_block_bytes(0) / E
+        _check(ctx, sh, 2, B, "logistic", 0.5, rounds.graph_schedule("complete", N, 1), tau=2, W0=W0)
