@@ -175,6 +175,7 @@ struct MixArgs {
   int box_rows;
   int n_boxes;
   int stages;
+  int depth;                   // slabs in flight at most, <= stages
   long long n_slabs;
   // fused sparse update / export (FUSED kernels only)
   const uint32_t* upd_list;    // this round's column list (slab-major)

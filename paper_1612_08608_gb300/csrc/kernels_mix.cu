@@ -570,8 +570,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     // The next round's local step (a programmatic dependent) may now be
     // scheduled as this grid drains; it waits for this grid before it reads
     // what this grid writes.  A gated reduce leaves the trigger to its exit,
-    // since the local step it overlaps is still running.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // since the local step it overlaps is still running; so does the update of
+    // an intermediate local step, or a gated reduce, let in by the next local
+    // step's own trigger, could read parameters this grid has yet to update.
+    if constexpr (!STEP) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   // ---- NOTIFY / ACK checks (time-limited waits) ----
@@ -624,8 +626,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       int2 loffs = make_int2(0, 0);                   // entry ring: the same, list_slots - stages slabs ahead
       int st = 0, done_st = 0;                        // stages of slab it, and of the slab that came back
       uint32_t done_ph = 0;
-      for (int it = 0; it < n_my + a.stages; ++it) {
-        if (!STEP && !gated && it == min(a.stages, n_my)) start_bar_or(false);
+      // a.depth slabs are asked for at most: a slab goes out when the one
+      // a.depth before has come back (its own stage has by then, a.stages >= a.depth).
+      for (int it = 0; it < n_my + a.depth; ++it) {
+        if (!STEP && !gated && it == min(a.depth, n_my)) start_bar_or(false);
         if (FUSED && (it & 31) == 0 && it < n_my) {
           const long long sl = blockIdx.x + static_cast<long long>(it + lane) * stride;
           if (it + lane < n_my)
@@ -642,7 +646,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
           o.z = __shfl_sync(kFull, offs.z, src);
           o.w = __shfl_sync(kFull, offs.w, src);
         }
-        if (it >= a.stages) {
+        if (it >= a.depth) {
           bool ok = (lane == 0) ? mbar_wait_bounded(sm.empty + done_st, done_ph) : true;
           ok = __shfl_sync(kFull, ok, 0) != 0;   // warp-uniform outcome
           __syncwarp();
@@ -769,7 +773,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         // (Added up before the copies were issued, they lengthened every
         // stage's turnaround by about a microsecond: the hashed workload's
         // reduce took 141 us instead of 128.)
-        if (it >= a.stages && KP1 >= 0) {
+        if (it >= a.depth && KP1 >= 0) {
           const float4* p = sm.part + done_st * kCompute;
           for (int q = lane; q < nq; q += 32) {
             float4 t = p[q];
@@ -779,7 +783,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
         }
         __syncwarp();
         if (it < n_my && lane == 0) mbar_arrive(sm.full + st);
-        if (it >= a.stages && ++done_st == a.stages) {
+        if (it >= a.depth && ++done_st == a.stages) {
           done_st = 0;
           done_ph ^= 1u;
         }

@@ -171,3 +171,20 @@ def test_row_and_place_in_the_code(B, row_len, packed):
         E = N * B * row_len
         assert (ctx.shard_block_bytes(0) < 9.9 * E + 6 * N * B + 4096) == packed, ctx.shard_block_bytes(0) / E
         _check(ctx, sh, 2, B, "logistic", 0.5, rounds.graph_schedule("complete", N, 1), tau=2, W0=W0)
+
+
+@pytest.mark.parametrize("B", [2, 24])
+def test_notify_ack_after_streamed_local_steps_equals_bsp(B):
+    # a gated reduce starts while the round's last local step runs, and reads parameters that the step before has
+    # updated by streaming the slabs
+    N, d = 21, 30011 if B == 24 else 2003
+    sh = inputs.sparse_custom(seed=4, N=N, d=d, rows=6 * B, max_len=300)
+    outs = []
+    for sync in ("bsp", "notify_ack"):
+        with _make(sh, N, 2, "root", "logistic", B, 0.4, l2=0.02, tau=2, sync=sync) as ctx:
+            before = ctx.kernel_launches()
+            ctx.round(40)
+            outs.append((ctx.read_params()[0], ctx.read_metrics(0, 40)))
+            assert ctx.kernel_launches() - before == 1 + 40 * 4      # streamed: two steps, one update, one reduce
+    assert np.array_equal(outs[0][0], outs[1][0])
+    assert np.array_equal(outs[0][1][0], outs[1][1][0]) and np.array_equal(outs[0][1][1], outs[1][1][1])
