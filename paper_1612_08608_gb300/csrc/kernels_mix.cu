@@ -1103,6 +1103,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     const unsigned t = atomicAdd(&a.st->mix_ticket, 1u);
     sm.flags[1] = ((t & 0xffffu) == gridDim.x - 1) ? 1 : 0;
     sm.flags[2] = static_cast<int>(t >> 16);
+    // The next reduce's tickets may come as soon as the ACK below is out.
+    if (sm.flags[1]) a.st->mix_ticket = 0u;
   }
   __syncthreads();
   if (!sm.flags[1]) return;
@@ -1136,12 +1138,12 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     }
     for (int b = tid; b < n_lp; b += kMixThreads) ltot = f2_add(ltot, F2{__ldcg(a.loss_part + b), 0.f});
   }
-  if (!any_fail)           // ACK, while the sums below are formed
+  block_sum2_f2(ctot, ltot, scratch);   // its barriers: every partial is read, the ticket reset, before the ACK
+  if (!any_fail)
     for (int j = tid; j < a.N; j += kMixThreads) {
       a.stamp_next[j] = a.round + 1u;
       st_release_u32(a.consumed + j, a.round + 1u);
     }
-  block_sum2_f2(ctot, ltot, scratch);
   if (tid == 0) {
     const int slot = static_cast<int>(a.round % kMetricsCap);
     a.metrics_cons[slot] = any_fail ? __int_as_float(0x7fc00000) : sqrtf(fmaxf(ctot.hi + ctot.lo, 0.f));
@@ -1152,7 +1154,6 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       if (a.expect_notify)
         atomicAdd(&a.st->consistent_inputs, static_cast<unsigned long long>(a.own_n) * (KP1 < 0 ? a.N : kp1));
     }
-    a.st->mix_ticket = 0u;
   }
 }
 
