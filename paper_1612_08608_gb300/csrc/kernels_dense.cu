@@ -92,18 +92,6 @@ __device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* m, uint64_t
       :: "r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
 }
 
-// The same 2-D load, written to the same shared-memory offset of every CTA of
-// the cluster in `mask` and completing on the mbarrier at `bar`'s offset in
-// each of them (the CTAs read the same tile of this GPU's memory).
-__device__ __forceinline__ void tma_2d_multicast(void* dst, const CUtensorMap* m, uint64_t* bar, int x, int y,
-                                                 uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-      " [%0], [%1, {%2, %3}], [%4], %5;"
-      :: "r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask)
-      : "memory");
-}
-
 __device__ __forceinline__ void tma_3d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, int y, int z) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -143,13 +131,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(smem_u32(bar))
                : "memory");
-}
-
-// The same arrival on the mbarrier at `bar`'s offset in every CTA of the
-// cluster in `mask`.
-__device__ __forceinline__ void umma_commit_multicast(uint64_t* bar, uint16_t mask) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               :: "r"(smem_u32(bar)), "h"(mask) : "memory");
 }
 
 // 32 consecutive fp32 accumulator columns of this thread's TMEM lane.
@@ -272,9 +253,6 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" :: "n
 //               reads local shared memory; then R = (softmax - onehot) / B is
 //               written to R^T from registers.
 constexpr int kFwdThreads = (2 + kEpiWarps) * 32;
-// X tiles are loaded in 32-row parts (4 KB each, 1024-byte aligned under the 128-byte swizzle)
-constexpr int kXPart = 32;
-constexpr uint32_t kXPartBytes = kXPart * kTileK * 2;
 constexpr int kMaxCq = 4;                                       // C <= 1024
 constexpr int kStatsSlot = kMaxCq * kEpiParts * 2 * kTileM;     // floats per stats slot
 
@@ -330,12 +308,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
   const int n_my = total > cl_id ? (total - cl_id + n_clusters - 1) / n_clusters : 0;
   const int k_tiles = a.d / kTileK;
   const int c0 = q * kTileN;
-  const uint16_t cmask = static_cast<uint16_t>((1u << Cq) - 1u);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kFwdStages; ++s) {
       mbar_init(sm.full + s, 1);
-      mbar_init(sm.empty + s, Cq);                         // every cluster CTA's MMA is done with the stage
+      mbar_init(sm.empty + s, 1);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(sm.acc_full + s, 1);
@@ -374,11 +351,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             break;
           }
           mbar_expect_tx(sm.full + s, kABytes + kBBytes);
-          // The X tile is the same for the cluster's CTAs: each loads its
-          // share of the 32-row parts and multicasts it to all of them.
-          for (int j = q; j < kTileM / kXPart; j += Cq)
-            tma_2d_multicast(sm.a + s * kABytes + j * kXPartBytes, &tmX, sm.full + s, kt * kTileK, row0 + j * kXPart,
-                             cmask);
+          // The X tile is the same for the cluster's CTAs: one of them reads it
+          // from memory, the others find it in L2.
+          tma_2d(sm.a + s * kABytes, &tmX, sm.full + s, kt * kTileK, row0);
           tma_3d(sm.b + s * kBBytes, &tmW, sm.full + s, kt * kTileK, c0, i);
         }
       }
@@ -412,7 +387,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             const uint64_t bd = smem_desc_sw128(sm.b + s * kBBytes + kk * 32);
             umma_bf16(acc, ad, bd, idesc, (kt | kk) != 0 ? 1u : 0u);
           }
-          umma_commit_multicast(sm.empty + s, cmask);   // the stage's X parts came from every CTA
+          umma_commit(sm.empty + s);
         }
         if (ok) umma_commit(sm.acc_full + ab);
       }
