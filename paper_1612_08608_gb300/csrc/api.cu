@@ -1367,7 +1367,6 @@ asap_status asap_set_model(asap_ctx* c, asap_loss loss, int num_classes, int bat
   }
   if (c->n_loss_part > 0) {
     CU(cudaMalloc(&c->loss_part, 4 * static_cast<size_t>(c->n_loss_part)), "allocating step scratch");
-    // Workers that a worker-sharded context does not step contribute 0.
     CU(cudaMemset(c->loss_part, 0, 4 * static_cast<size_t>(c->n_loss_part)), "zeroing step scratch");
   }
   return ASAP_OK;
@@ -1466,6 +1465,10 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
   asap_status s0 = asap_sync(c);
   if (s0 != ASAP_OK) return s0;
   free_shards(c);
+  // A worker's loss partials lie elsewhere in each layout, and the range of a
+  // worker-sharded context may have changed: entries that the steps to come do
+  // not write contribute 0.
+  CU(cudaMemsetAsync(c->loss_part, 0, 4 * static_cast<size_t>(c->n_loss_part), c->stream), "zeroing step scratch");
   c->s_cap = 1024;
   s0 = setup_mix(c);
   if (s0 != ASAP_OK) return s0;

@@ -189,3 +189,31 @@ def test_two_processes_gloo_share_the_gpu():
         err, _, _ = sparse_round_matching(W_t, W_n, sh, t, cfg["B"], cfg["loss"], cfg["lr"], nbr, wgt, TOL)
         assert err <= TOL, (t, err)
         W_t = W_n.astype(np.float64)
+
+
+@pytest.mark.parametrize("order", [("even", "hot"), ("hot", "even")])
+def test_loss_after_shards_of_the_other_layout(order):
+    # at W = 0 every sample's loss is ln 2, and a context that steps one of four workers reports a quarter of the
+    # mean: also after shards whose loss partials lay elsewhere (evenly spread columns: two per worker, by worker;
+    # one hot column: one per worker), and after another range
+    from paper_1612_08608_gb300 import Context
+    N, d, B = 4, 3000, 64
+    with Context(N, d, graph_seed=0, k=1) as ctx:
+        ctx.set_model("logistic", batch=B, lr=0.1)
+        ctx.set_graph("ring")
+        W0 = np.zeros((N, d), np.float32)
+        for i in (1, 3):
+            ctx.set_worker_range(i, 1)
+            for kind in order:
+                sh = inputs.sparse_custom(seed=1, N=N, d=d, rows=2 * B, max_len=60,
+                                          **({"hot_col": 5} if kind == "hot" else {}))
+                one = lambda a: [x if q == i else None for q, x in enumerate(a)]
+                ctx.load_shards(rowptr=one(sh.rowptr), col=one(sh.col), val=one(sh.val), y=one(sh.y))
+                E = int(sh.rowptr[i][B])
+                assert (ctx.shard_block_bytes(0) < 13 * E + 6 * N * B + 1024) == (kind == "even"), kind
+                ctx.write_params(W0, 0)
+                ctx.local_step()
+                others = np.array([q for q in range(N) if q != i])
+                ctx.write_rows(others, W0[others])
+                ctx.stochastic_reduce()
+                assert ctx.read_metrics(0, 1)[0][0] == pytest.approx(np.log(2.0) / N, rel=1e-6), (i, kind)
