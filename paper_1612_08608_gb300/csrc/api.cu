@@ -226,6 +226,22 @@ asap_status cuda_fail(asap_ctx* c, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(c, e_, what); \
   } while (0)
 
+// Set-up writes go to the context's stream like everything that reads them.
+// The legacy default stream is no substitute: the context's streams do not wait
+// for it, so a fill queued there behind the caller's own work could come after,
+// and wipe, what the first copies and kernels have written.
+asap_status to_device(asap_ctx* c, void* dst, const void* src, size_t bytes, const char* what) {
+  CU(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream), what);
+  CU(cudaStreamSynchronize(c->stream), what);   // the caller may reuse src
+  return ASAP_OK;
+}
+
+#define TO_DEVICE(c, dst, src, bytes, what)                  \
+  do {                                                       \
+    asap_status s_ = to_device(c, dst, src, bytes, what);    \
+    if (s_ != ASAP_OK) return s_;                            \
+  } while (0)
+
 template <typename T>
 void dfree(T*& p) {
   if (p) cudaFree(p);
@@ -425,10 +441,10 @@ asap_status alloc_params(asap_ctx* c) {
   const size_t bytes = static_cast<size_t>(c->N) * c->ld * 4;
   for (int b = 0; b < 2; ++b) {
     CU(cudaMalloc(&c->W[b], bytes), "allocating the parameter buffers");
-    CU(cudaMemset(c->W[b], 0, bytes), "zeroing the parameter buffers");
+    CU(cudaMemsetAsync(c->W[b], 0, bytes, c->stream), "zeroing the parameter buffers");
     if (c->loss == ASAP_LOSS_SOFTMAX) {
       CU(cudaMalloc(&c->Wbf[b], bytes / 2), "allocating the bf16 parameter copy");
-      CU(cudaMemset(c->Wbf[b], 0, bytes / 2), "zeroing the bf16 parameter copy");
+      CU(cudaMemsetAsync(c->Wbf[b], 0, bytes / 2, c->stream), "zeroing the bf16 parameter copy");
     }
   }
   asap_status s = setup_mix(c);
@@ -450,9 +466,8 @@ asap_status upload_fixed_graph(asap_ctx* c) {
   std::vector<float> wgt(n);
   asap_status s = graph_host(c, 0, nbr.data(), wgt.data());
   if (s != ASAP_OK) return s;
-  CU(cudaStreamSynchronize(c->stream), "synchronising before a graph upload");
-  CU(cudaMemcpy(c->d_nbr, nbr.data(), n * 4, cudaMemcpyHostToDevice), "uploading the graph");
-  CU(cudaMemcpy(c->d_wgt, wgt.data(), n * 4, cudaMemcpyHostToDevice), "uploading the graph weights");
+  TO_DEVICE(c, c->d_nbr, nbr.data(), n * 4, "uploading the graph");
+  TO_DEVICE(c, c->d_wgt, wgt.data(), n * 4, "uploading the graph weights");
   c->graph_round_in_slot0 = 0;
   return ASAP_OK;
 }
@@ -531,8 +546,7 @@ void time_end(asap_ctx* c) {
 // Reports the error in a copy of the device state, if any, and clears it.
 asap_status check_device_error(asap_ctx* c, const DevState& h) {
   if (h.err_code == 0) return ASAP_OK;
-  const unsigned zero = 0;
-  CU(cudaMemcpy(&c->st->err_code, &zero, 4, cudaMemcpyHostToDevice), "clearing device error");
+  CU(cudaMemsetAsync(&c->st->err_code, 0, 4, c->stream), "clearing device error");
   char buf[200];
   if (h.err_code == ASAP_ERR_TIMEOUT)
     snprintf(buf, sizeof buf, "device: NOTIFY/ACK wait ran out (worker %u, round %u); parameters are undefined "
@@ -887,8 +901,7 @@ asap_status upload_blocks(asap_ctx* c, int nb, Img&& img) {
     if (host)
       std::memcpy(c->pool + c->block_off[t], img(t).data(), img(t).size());
     else
-      CU(cudaMemcpy(c->pool + c->block_off[t], img(t).data(), img(t).size(), cudaMemcpyHostToDevice),
-         "copying shards to the device");
+      TO_DEVICE(c, c->pool + c->block_off[t], img(t).data(), img(t).size(), "copying shards to the device");
     std::vector<unsigned char>().swap(img(t));
   }
   if (host) {
@@ -957,10 +970,10 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   const size_t pb = 4 * static_cast<size_t>(table);
   for (int b = 0; b < 2; ++b) {
     CU(cudaMalloc(&c->wv[b], pb), "allocating the table of products");
-    CU(cudaMemset(c->wv[b], 0, pb), "zeroing the table of products");
+    CU(cudaMemsetAsync(c->wv[b], 0, pb, c->stream), "zeroing the table of products");
   }
   CU(cudaMalloc(&c->r_ent, 4 * static_cast<size_t>(N) * B), "allocating the step scratch");
-  CU(cudaMemset(c->r_ent, 0, 4 * static_cast<size_t>(N) * B), "zeroing the step scratch");
+  CU(cudaMemsetAsync(c->r_ent, 0, 4 * static_cast<size_t>(N) * B, c->stream), "zeroing the step scratch");
   c->row_stride = stride;
   c->max_region = max_region;
   c->entries = true;
@@ -1144,7 +1157,7 @@ static asap_status init_ctx(asap_ctx* c) {
     CU(cudaEventCreateWithFlags(&c->free_ev[b], cudaEventDisableTiming), "creating events");
   }
   CU(cudaMalloc(&c->flags, 20 * static_cast<size_t>(N)), "allocating flags");
-  CU(cudaMemset(c->flags, 0, 20 * static_cast<size_t>(N)), "zeroing flags");
+  CU(cudaMemsetAsync(c->flags, 0, 20 * static_cast<size_t>(N), c->stream), "zeroing flags");
   CU(cudaHostAlloc(&c->h_flags, 20 * static_cast<size_t>(N), cudaHostAllocDefault), "allocating pinned flags");
   CU(cudaHostAlloc(&c->h_read, sizeof(asap_ctx::HostReads), cudaHostAllocDefault), "allocating pinned reads");
   c->ready = c->flags;
@@ -1153,11 +1166,11 @@ static asap_status init_ctx(asap_ctx* c) {
   c->ticket = c->flags + 4 * N;
   CU(cudaMalloc(&c->d_worker_of, 4 * static_cast<size_t>(N)), "allocating the local-step map");
   CU(cudaMalloc(&c->st, sizeof(DevState)), "allocating device state");
-  CU(cudaMemset(c->st, 0, sizeof(DevState)), "zeroing device state");
+  CU(cudaMemsetAsync(c->st, 0, sizeof(DevState), c->stream), "zeroing device state");
   CU(cudaMalloc(&c->m_loss, 4 * kMetricsCap), "allocating metrics");
   CU(cudaMalloc(&c->m_cons, 4 * kMetricsCap), "allocating metrics");
-  CU(cudaMemset(c->m_loss, 0xff, 4 * kMetricsCap), "clearing metrics");
-  CU(cudaMemset(c->m_cons, 0xff, 4 * kMetricsCap), "clearing metrics");
+  CU(cudaMemsetAsync(c->m_loss, 0xff, 4 * kMetricsCap, c->stream), "clearing metrics");
+  CU(cudaMemsetAsync(c->m_cons, 0xff, 4 * kMetricsCap, c->stream), "clearing metrics");
   c->cons_cap = c->sm_count * 32;
   CU(cudaMalloc(&c->cons_part, 8 * static_cast<size_t>(c->cons_cap)), "allocating reduce scratch");
   const int kp1_tab = std::min(k + 1, kMaxKp1Sparse);
@@ -1354,7 +1367,7 @@ asap_status asap_set_model(asap_ctx* c, asap_loss loss, int num_classes, int bat
     c->n_loss_part = c->N * (batch / 128) * c->Cq;
     const size_t rt = static_cast<size_t>(c->N) * c->Cq * 256 * batch;
     CU(cudaMalloc(&c->RT, 2 * rt), "allocating the softmax residual scratch");
-    CU(cudaMemset(c->RT, 0, 2 * rt), "zeroing the softmax residual scratch");
+    CU(cudaMemsetAsync(c->RT, 0, 2 * rt, c->stream), "zeroing the softmax residual scratch");
     cuuint64_t dims[2] = {static_cast<cuuint64_t>(batch), static_cast<cuuint64_t>(c->N) * c->Cq * 256};
     cuuint64_t str[1] = {static_cast<cuuint64_t>(batch) * 2};
     cuuint32_t box[2] = {64, 128};
@@ -1367,7 +1380,7 @@ asap_status asap_set_model(asap_ctx* c, asap_loss loss, int num_classes, int bat
   }
   if (c->n_loss_part > 0) {
     CU(cudaMalloc(&c->loss_part, 4 * static_cast<size_t>(c->n_loss_part)), "allocating step scratch");
-    CU(cudaMemset(c->loss_part, 0, 4 * static_cast<size_t>(c->n_loss_part)), "zeroing step scratch");
+    CU(cudaMemsetAsync(c->loss_part, 0, 4 * static_cast<size_t>(c->n_loss_part), c->stream), "zeroing step scratch");
   }
   return ASAP_OK;
 }
@@ -1408,7 +1421,7 @@ asap_status asap_set_shard_residency(asap_ctx* c, asap_residency r) {
     unsigned char* np = nullptr;
     if (r == ASAP_SHARDS_DEVICE) {
       CU(cudaMalloc(&np, c->pool_bytes), "allocating device shard memory");
-      CU(cudaMemcpy(np, c->pool, c->pool_bytes, cudaMemcpyHostToDevice), "moving shards to the device");
+      TO_DEVICE(c, np, c->pool, c->pool_bytes, "moving shards to the device");
       cudaFreeHost(c->pool);
       for (int b = 0; b < asap_ctx::kStaging; ++b) dfree(c->staging[b]);
     } else {
@@ -1519,15 +1532,14 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
     s0 = upload_blocks(c, nb, [&](int t) -> std::vector<unsigned char>& { return built[t].img; });
     if (s0 != ASAP_OK) return s0;
     CU(cudaMalloc(&c->d_desc, desc.size() * sizeof(BatchDesc)), "allocating batch descriptors");
-    CU(cudaMemcpy(c->d_desc, desc.data(), desc.size() * sizeof(BatchDesc), cudaMemcpyHostToDevice),
-       "copying batch descriptors");
+    TO_DEVICE(c, c->d_desc, desc.data(), desc.size() * sizeof(BatchDesc), "copying batch descriptors");
     const size_t lb = 4 * static_cast<size_t>(std::max<int64_t>(max_list, 4));
     CU(cudaMalloc(&c->wv[0], lb), "allocating the list value buffer");
     CU(cudaMalloc(&c->wv[1], lb), "allocating the list value buffer");
     CU(cudaMalloc(&c->gsum, lb), "allocating the column-sum buffer");
-    CU(cudaMemset(c->wv[0], 0, lb), "zeroing the list value buffer");
-    CU(cudaMemset(c->wv[1], 0, lb), "zeroing the list value buffer");
-    CU(cudaMemset(c->gsum, 0, lb), "zeroing the column-sum buffer");
+    CU(cudaMemsetAsync(c->wv[0], 0, lb, c->stream), "zeroing the list value buffer");
+    CU(cudaMemsetAsync(c->wv[1], 0, lb, c->stream), "zeroing the list value buffer");
+    CU(cudaMemsetAsync(c->gsum, 0, lb, c->stream), "zeroing the column-sum buffer");
     if (B > kRSmemRows) {
       CU(cudaMalloc(&c->mpart_big, 16 * static_cast<size_t>(N) * Q * B), "allocating the partial margins");
       CU(cudaMalloc(&c->r_big, 4 * static_cast<size_t>(N) * Q * B), "allocating the step scratch");
@@ -1572,9 +1584,8 @@ asap_status asap_load_dense_shards(asap_ctx* c, const uint16_t* const* X, const 
   CU(cudaMalloc(&c->Yd, 4 * static_cast<size_t>(N) * rows), "allocating labels");
   std::vector<uint16_t> tr(rows * d);
   for (int i = 0; i < N; ++i) {
-    CU(cudaMemcpy(c->X + static_cast<size_t>(i) * rows * d, X[i], 2 * rows * d, cudaMemcpyHostToDevice),
-       "copying dense features");
-    CU(cudaMemcpy(c->Yd + static_cast<size_t>(i) * rows, y[i], 4 * rows, cudaMemcpyHostToDevice), "copying labels");
+    TO_DEVICE(c, c->X + static_cast<size_t>(i) * rows * d, X[i], 2 * rows * d, "copying dense features");
+    TO_DEVICE(c, c->Yd + static_cast<size_t>(i) * rows, y[i], 4 * rows, "copying labels");
     // Per minibatch, the features transposed to [d][B] (the K-major operand
     // of the gradient GEMM, whose reduction runs over the batch).
     const unsigned nthr = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
@@ -1589,8 +1600,7 @@ asap_status asap_load_dense_shards(asap_ctx* c, const uint16_t* const* X, const 
         }
       });
     for (auto& th : pool) th.join();
-    CU(cudaMemcpy(c->XT + static_cast<size_t>(i) * rows * d, tr.data(), 2 * rows * d, cudaMemcpyHostToDevice),
-       "copying transposed features");
+    TO_DEVICE(c, c->XT + static_cast<size_t>(i) * rows * d, tr.data(), 2 * rows * d, "copying transposed features");
   }
   {
     cuuint64_t dims[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(N) * rows};
@@ -1937,14 +1947,14 @@ asap_status asap_write_params(asap_ctx* c, const float* host_in, int64_t round) 
   asap_status s = sync_all(c);
   if (s != ASAP_OK) return s;
   float* dst = c->W[round & 1];
-  CU(cudaMemcpy2D(dst, c->ld * 4, host_in, c->P * 4, c->P * 4, c->N, cudaMemcpyHostToDevice), "writing parameters");
+  CU(cudaMemcpy2DAsync(dst, c->ld * 4, host_in, c->P * 4, c->P * 4, c->N, cudaMemcpyHostToDevice, c->stream),
+     "writing parameters");
   if (c->Wbf[round & 1]) {
     CU(launch_cast_bf16(dst, c->Wbf[round & 1], static_cast<int64_t>(c->N) * c->ld, c->stream), "bf16 copy");
     c->launches += 1;
-    CU(cudaStreamSynchronize(c->stream), "bf16 copy");
   }
   c->wv_step = -1;
-  return reset_protocol(c, round);
+  return reset_protocol(c, round);   // waits for the copy too
 }
 
 asap_status asap_write_params_device(asap_ctx* c, const float* dev_in, int64_t ld_in, int64_t round) {
@@ -2077,7 +2087,7 @@ asap_status asap_set_worker_order(asap_ctx* c, const int32_t* order) {
   }
   asap_status s0 = asap_sync(c);
   if (s0 != ASAP_OK) return s0;
-  CU(cudaMemcpy(c->d_worker_of, order, 4 * static_cast<size_t>(c->N), cudaMemcpyHostToDevice), "uploading the worker order");
+  TO_DEVICE(c, c->d_worker_of, order, 4 * static_cast<size_t>(c->N), "uploading the worker order");
   c->permuted = !identity;
   return ASAP_OK;
 }
@@ -2100,8 +2110,7 @@ asap_status asap_set_worker_range(asap_ctx* c, int first, int count) {
   c->sync_mode = kSyncBsp;
   std::vector<int32_t> own(c->N);
   for (int q = 0; q < c->N; ++q) own[q] = q < c->own_n ? c->own_lo + q : q;
-  CU(cudaMemcpy(c->d_worker_of, own.data(), 4 * static_cast<size_t>(c->N), cudaMemcpyHostToDevice),
-     "uploading the owned workers");
+  TO_DEVICE(c, c->d_worker_of, own.data(), 4 * static_cast<size_t>(c->N), "uploading the owned workers");
   return ASAP_OK;
 }
 

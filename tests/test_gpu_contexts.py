@@ -33,3 +33,48 @@ def test_contexts_of_different_sizes_side_by_side():
         err, _, _ = sparse_round_matching(W_t.astype(np.float64), W_n, sh, 1, B, "logistic", 0.3, nbr, wgt, 1e-5)
         assert err <= 1e-5
         ctx.close()
+
+
+@pytest.mark.parametrize("residency", ["device", "host"])
+def test_setup_behind_queued_work_of_the_default_stream(residency):
+    # the context's streams do not wait for the legacy default stream: nothing that a context sets up may be queued
+    # there, behind the caller's own work, and land after the first round's copies and kernels
+    import torch
+    from paper_1612_08608_gb300 import Context
+    N, d, B = 6, 8000, 32
+    rng = np.random.default_rng(1)
+    W0 = rng.standard_normal((N, d)).astype(np.float32)
+    sh = inputs.sparse_custom(seed=3, N=N, d=d, rows=4 * B, max_len=40)
+    dev = torch.from_numpy(W0).cuda()
+    torch.cuda.synchronize()
+    made = []
+    torch.cuda._sleep(400_000_000)                     # about 0.2 s of the default stream
+    for model in (False, True):
+        ctx = Context(N, d, graph_seed=0, k=N - 1)     # complete graph: no table is uploaded
+        ctx.set_graph("complete")
+        if model:
+            ctx.set_model("logistic", batch=B, lr=0.3)
+            ctx.set_shard_residency(residency)
+            ctx.load_shards(sh)
+            ctx.write_params(W0, 0)
+        else:
+            ctx.write_params_device(dev, 0)
+        ctx.round(1)
+        made.append(ctx)
+    torch.cuda.synchronize()                           # whatever was queued late has run
+    mean = W0.astype(np.float64).mean(axis=0)
+    got, rnd = made[0].read_params()
+    assert rnd == 1 and np.abs(got - mean).max() <= 1e-6 * np.abs(mean).max()
+    sched = rounds.graph_schedule("complete", N, N - 1)
+    W_t = W0
+    for t in range(3):
+        if t:
+            made[1].round(1)
+        W_n, _ = made[1].read_params()
+        nbr, wgt = sched(t)
+        err, lref, _ = sparse_round_matching(W_t.astype(np.float64), W_n, sh, t, B, "logistic", 0.3, nbr, wgt, 1e-5)
+        assert err <= 1e-5, (t, err)
+        assert abs(made[1].read_metrics(t, 1)[0][0] - lref) <= 1e-5
+        W_t = W_n
+    for ctx in made:
+        ctx.close()
