@@ -201,7 +201,9 @@ asap_status asap_write_params(asap_ctx* ctx, const float* host_in, int64_t round
 /* Set W_t from device memory: dev_in holds N rows of P floats with row
  * stride ld_in (>= P), on the context's device; the round counter becomes
  * `round`.  For parameters that already live in HBM (a resume, or inputs
- * drawn on the device), without a host round trip.  Synchronous. */
+ * drawn on the device), without a host round trip.  Comes after what the
+ * legacy default stream holds by then; work of other streams that fills
+ * dev_in must have finished.  Synchronous. */
 asap_status asap_write_params_device(asap_ctx* ctx, const float* dev_in, int64_t ld_in, int64_t round);
 
 /* Copy columns [first, first + count) of every worker's current

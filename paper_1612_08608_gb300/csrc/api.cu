@@ -120,6 +120,7 @@ struct asap_ctx {
   cudaEvent_t graph_half_ev[2] = {};   // the half's last upload
   bool graph_half_used[2] = {false, false};
   cudaEvent_t graph_order_ev = nullptr; // the stream's work before an upload
+  cudaEvent_t caller_ev = nullptr;      // the legacy default stream's work before asap_write_params_device
 
   // sparse shards
   asap_residency residency = ASAP_SHARDS_DEVICE;
@@ -1152,6 +1153,7 @@ static asap_status init_ctx(asap_ctx* c) {
     c->graph_half_used[h] = false;
   }
   CU(cudaEventCreateWithFlags(&c->graph_order_ev, cudaEventDisableTiming), "creating events");
+  CU(cudaEventCreateWithFlags(&c->caller_ev, cudaEventDisableTiming), "creating events");
   for (int b = 0; b < asap_ctx::kStaging; ++b) {
     CU(cudaEventCreateWithFlags(&c->staged_ev[b], cudaEventDisableTiming), "creating events");
     CU(cudaEventCreateWithFlags(&c->free_ev[b], cudaEventDisableTiming), "creating events");
@@ -1238,6 +1240,7 @@ void asap_destroy(asap_ctx* c) {
   for (int h = 0; h < 2; ++h)
     if (c->graph_half_ev[h]) cudaEventDestroy(c->graph_half_ev[h]);
   if (c->graph_order_ev) cudaEventDestroy(c->graph_order_ev);
+  if (c->caller_ev) cudaEventDestroy(c->caller_ev);
   for (auto& e : c->tev)
     if (e) cudaEventDestroy(e);
   for (int b = 0; b < asap_ctx::kStaging; ++b) {
@@ -1962,6 +1965,10 @@ asap_status asap_write_params_device(asap_ctx* c, const float* dev_in, int64_t l
   asap_status s = sync_all(c);
   if (s != ASAP_OK) return s;
   float* dst = c->W[round & 1];
+  // What the caller queued on the legacy default stream (the kernels that fill
+  // dev_in, usually) comes first.
+  CU(cudaEventRecord(c->caller_ev, cudaStreamLegacy), "ordering after the default stream");
+  CU(cudaStreamWaitEvent(c->stream, c->caller_ev, 0), "ordering after the default stream");
   CU(cudaMemcpy2DAsync(dst, c->ld * 4, dev_in, ld_in * 4, c->P * 4, c->N, cudaMemcpyDeviceToDevice, c->stream),
      "writing parameters");
   if (c->Wbf[round & 1]) {

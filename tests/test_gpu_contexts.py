@@ -78,3 +78,20 @@ def test_setup_behind_queued_work_of_the_default_stream(residency):
         W_t = W_n
     for ctx in made:
         ctx.close()
+
+
+@pytest.mark.parametrize("N,d", [(3, 100), (16, 200001)])
+def test_device_parameters_still_being_made_on_the_default_stream(N, d):
+    # parameters that the default stream is yet to fill when they are handed over
+    import torch
+    from paper_1612_08608_gb300 import Context
+    want = np.random.default_rng(N).standard_normal((N, d)).astype(np.float32)
+    src = torch.from_numpy(want).cuda()
+    with Context(N, d, graph_seed=0, k=1) as ctx:
+        dev = torch.zeros_like(src)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(200_000_000)                 # about 0.1 s
+        dev.copy_(src)
+        ctx.write_params_device(dev, 4)
+        got, rnd = ctx.read_params()
+    assert rnd == 4 and np.array_equal(got, want)
