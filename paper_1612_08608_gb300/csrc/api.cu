@@ -463,12 +463,12 @@ asap_status upload_fixed_graph(asap_ctx* c) {
   c->graph_half_batch[0] = c->graph_half_batch[1] = -1;
   if (c->tab_kp1 == 0 || c->regen) return ASAP_OK;
   const size_t n = static_cast<size_t>(c->N) * c->tab_kp1;
-  std::vector<int32_t> nbr(n);
-  std::vector<float> wgt(n);
-  asap_status s = graph_host(c, 0, nbr.data(), wgt.data());
+  // From the pinned ring: every caller has waited for the stream before, so no
+  // earlier upload still reads it.
+  asap_status s = graph_host(c, 0, c->h_nbr, c->h_wgt);
   if (s != ASAP_OK) return s;
-  TO_DEVICE(c, c->d_nbr, nbr.data(), n * 4, "uploading the graph");
-  TO_DEVICE(c, c->d_wgt, wgt.data(), n * 4, "uploading the graph weights");
+  CU(cudaMemcpyAsync(c->d_nbr, c->h_nbr, n * 4, cudaMemcpyHostToDevice, c->stream), "uploading the graph");
+  CU(cudaMemcpyAsync(c->d_wgt, c->h_wgt, n * 4, cudaMemcpyHostToDevice, c->stream), "uploading the graph weights");
   c->graph_round_in_slot0 = 0;
   return ASAP_OK;
 }
