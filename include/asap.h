@@ -213,7 +213,9 @@ asap_status asap_read_param_columns(asap_ctx* ctx, int64_t first, int64_t count,
 
 /* Per-round metrics of rounds [first_round, first_round + count): the mean
  * over workers of the minibatch loss at the pre-step parameters (NaN for a
- * reduce-only round) and the consensus error ||W_{t+1} - 1 wbar^T||_F.
+ * reduce-only round) and the consensus error ||W_{t+1} - 1 wbar^T||_F
+ * (NaN if W_{t+1} is not finite; on the complete graph, whose reduce makes all
+ * rows the same, always 0).
  * The last 65536 rounds are kept.  Either output pointer may be NULL.
  * Waits only until round first_round + count - 1 is complete when that is
  * one of the last 64 rounds launched since the last asap_write_params
@@ -391,7 +393,8 @@ asap_status asap_build_graph(asap_graph_kind kind, int N, int k, uint64_t graph_
  * int32 / float (row i = the ids in [0, N) and weights of worker i's
  * inputs, summed in the given order; ids outside [0, N) are clamped into
  * range, never read out of bounds); consensus_out one float, set to
- * ||W_out - 1 wbar^T||_F with wbar the column mean of W_in.  Limits:
+ * ||W_out - 1 wbar^T||_F with wbar the column mean of W_in (NaN if either is
+ * not finite).  Limits:
  * 1 <= N <= 256, 1 <= kp1 <= 32, and ld within the built-in scratch (32768
  * column slabs: ld <= 8,388,608 for N <= 16, ld <= 524,288 for N = 256);
  * larger sizes return ASAP_ERR_ARG without touching the GPU.

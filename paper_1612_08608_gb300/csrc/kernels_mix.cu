@@ -1146,7 +1146,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
     }
   if (tid == 0) {
     const int slot = static_cast<int>(a.round % kMetricsCap);
-    a.metrics_cons[slot] = any_fail ? __int_as_float(0x7fc00000) : sqrtf(fmaxf(ctot.hi + ctot.lo, 0.f));
+    // Rounding may leave a little below 0; a NaN (parameters that are not
+    // finite) stays one.
+    const float c2 = ctot.hi + ctot.lo;
+    a.metrics_cons[slot] = any_fail ? __int_as_float(0x7fc00000) : sqrtf(c2 < 0.f ? 0.f : c2);
     a.metrics_loss[slot] = (a.have_loss && !any_fail) ? (ltot.hi + ltot.lo) * a.loss_norm
                                                       : __int_as_float(0x7fc00000);
     if (!any_fail) {

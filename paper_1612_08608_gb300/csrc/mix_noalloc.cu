@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
   }
   const Pair sum = block_sum(v, sm.red);
   if (tid == 0) {
-    a.consensus_out[0] = sqrtf(fmaxf(sum.hi + sum.lo, 0.f));
+    const float c2 = sum.hi + sum.lo;
+    a.consensus_out[0] = sqrtf(c2 < 0.f ? 0.f : c2);   // a NaN stays one
     a.tickets[a.slot] = 0u;
     a.tickets[(a.slot + kSlots / 2) % kSlots] = 0u;
   }
