@@ -394,10 +394,10 @@ asap_status asap_build_graph(asap_graph_kind kind, int N, int k, uint64_t graph_
  * inputs, summed in the given order; ids outside [0, N) are clamped into
  * range, never read out of bounds); consensus_out one float, set to
  * ||W_out - 1 wbar^T||_F with wbar the column mean of W_in (NaN if either is
- * not finite).  Limits:
- * 1 <= N <= 256, 1 <= kp1 <= 32, and ld within the built-in scratch (32768
- * column slabs: ld <= 8,388,608 for N <= 16, ld <= 524,288 for N = 256);
- * larger sizes return ASAP_ERR_ARG without touching the GPU.
+ * not finite).  Limits: 1 <= N <= 256, 1 <= kp1 <= 32, and ld within the range
+ * that the built-in scratch was laid out for (32768 slabs of at most 16 KB: ld
+ * <= 8,388,608 for N <= 16, ld <= 524,288 for N = 256); larger sizes return
+ * ASAP_ERR_ARG without touching the GPU.
  * It calls no cudaMalloc, cudaFree or other allocating routine: its scratch
  * (about 256 KB) is a file-scope device array that every GPU loading this
  * library holds until the process exits.  The first call on each device
@@ -409,9 +409,18 @@ asap_status asap_build_graph(asap_graph_kind kind, int N, int k, uint64_t graph_
  * call shares the array and leaves at zero what must start there; calls that
  * overlap on the GPU (other streams, other threads) race on it and must be
  * serialised by the caller.  Async on cuda_stream (NULL: legacy default
- * stream); no device-side error is reported. */
+ * stream).  The kernel's waits on its own copies are time-limited (2 s); if
+ * one runs out, W_out is incomplete and consensus_out is NaN.  No other
+ * device-side error is reported. */
 asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, int64_t d, int64_t ld, const int32_t* nbr,
                              const float* wgt, int kp1, float* consensus_out, void* cuda_stream);
+
+/* Test only: asap_mix_noalloc with the waits limited to wait_ns, and without
+ * the copy of the drop_slab-th column slab (-1: none), so that the wait for it
+ * runs out. */
+asap_status asap_debug_mix_noalloc(const float* W_in, float* W_out, int N, int64_t d, int64_t ld, const int32_t* nbr,
+                                   const float* wgt, int kp1, float* consensus_out, void* cuda_stream,
+                                   uint64_t wait_ns, int64_t drop_slab);
 
 const char* asap_last_error(const asap_ctx* ctx);
 const char* asap_version(void);

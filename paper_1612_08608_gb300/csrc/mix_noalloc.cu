@@ -23,6 +23,10 @@
 // loads, one slab in flight per CTA, 280 us.  A small call is launch latency: N =
 // 8, d = 4,093 8.1 us, 9.5 us while a memset cleared the ticket before each
 // launch (now the last CTA leaves it at zero).
+//
+// Every wait is time-limited.  A CTA in which one runs out stops mixing, waits
+// (time-limited again) for its own copies in flight and turns the consensus
+// error into NaN, the only word a call can pass on.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -48,8 +52,8 @@ constexpr size_t kNoAllocScratchBytes = kNoAllocTicketBytes + 8u * kNoAllocMaxSl
 constexpr int kNoAllocMaxDevices = 64;
 
 // [0, 256): ticket counters; [256, 256 + 8 * kNoAllocMaxSlabs): double
-// partials, one per CTA (the size, and with it the largest ld, dates from one
-// per slab).  Calls take kSlots slots of both in turn.  A call's last CTA
+// partials, one per CTA.  (The largest ld that a call takes is 32,768 slabs of at
+// most 16 KB: the partials were one per slab when it was set.)  Calls take kSlots slots of both in turn.  A call's last CTA
 // leaves its own ticket at zero, and clears the one half the slots away: calls
 // that overlapped against the rules (their stream order is the caller's
 // business) cannot spoil more than the calls right after them.
@@ -62,7 +66,7 @@ constexpr int kGroups = 2;                             // compute groups, on alt
 constexpr int kGroupThreads = 256;
 constexpr int kBlock = kGroups * kGroupThreads + 32;   // and the producer warp
 constexpr size_t kSlabBytes = 32768;                   // at most
-constexpr unsigned long long kWaitNs = 2000000000ull;  // a TMA load never takes this long
+constexpr unsigned long long kWaitNs = 2000000000ull;  // a wait's limit: a TMA load never takes this long
 static_assert(kStages % kGroups == 0, "a stage belongs to one group: its warps wait for each of its phases");
 
 struct NoAllocArgs {
@@ -78,6 +82,8 @@ struct NoAllocArgs {
   unsigned int* tickets;
   int slot;
   double* partial;
+  unsigned long long wait_ns;
+  long long drop_slab;   // tests: the slab whose copy is left out, so that its wait runs out (-1: none)
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -112,12 +118,12 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 
 // Time-limited wait on an mbarrier phase; false if the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned long long limit_ns) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = now_ns();
   for (unsigned n = 1;; ++n) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((n & 255u) == 0 && now_ns() - t0 > kWaitNs) return false;
+    if ((n & 255u) == 0 && now_ns() - t0 > limit_ns) return false;
   }
 }
 
@@ -129,6 +135,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
 
 __device__ __forceinline__ void group_bar(int group) {
   asm volatile("bar.sync %0, %1;" :: "r"(group + 1), "n"(kGroupThreads) : "memory");
+}
+
+// The same barrier, which also returns the OR of `v` over the group.
+__device__ __forceinline__ bool group_bar_or(int group, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, %3, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r) : "r"(static_cast<uint32_t>(v)), "n"(kGroupThreads), "r"(group + 1) : "memory");
+  return r != 0;
 }
 
 // Sums are carried as float-float pairs hi + lo in fp32 arithmetic (this
@@ -232,16 +247,20 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
   }
   __syncthreads();
   Pair total{0.f, 0.f};
+  bool failed = false;                             // a wait of this thread's (or its group's) ran out
   if (warp == kBlock / 32 - 1) {
     // ---- producer ----
     if (lane == 0) {
-      int st = 0;
+      int st = 0, it = 0;
       uint32_t ph = 1;                             // "empty" passes at once the first time round
-      for (int it = 0; it < n_my; ++it) {
-        if (!mbar_wait(sm.empty + st, ph)) break;
-        const long long c0 = (blockIdx.x + static_cast<long long>(it) * gridDim.x) * a.S;
+      for (; it < n_my; ++it) {
+        if (!mbar_wait(sm.empty + st, ph, a.wait_ns)) {
+          failed = true;
+          break;
+        }
+        const long long slab = blockIdx.x + static_cast<long long>(it) * gridDim.x, c0 = slab * a.S;
         mbar_expect_tx(sm.full + st, static_cast<uint32_t>(a.N) * a.S * 4u);
-        for (int b = 0; b < nq / QB; ++b)          // [column box][row][QB quads]
+        for (int b = 0; b < nq / QB && slab != a.drop_slab; ++b)   // [column box][row][QB quads]
           tma_load_2d(sm.stage0 + st * sm.stage_bytes + static_cast<size_t>(b) * a.N * QB * 16, &tmap, sm.full + st,
                       static_cast<int>(c0 + b * QB * 4), 0);
         if (++st == kStages) {
@@ -249,6 +268,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
           ph ^= 1u;
         }
       }
+      // The CTA's shared memory is given back with no copy in flight: the last
+      // one into each stage has landed (as the groups see too, unless one gave up).
+      for (int s = 0; s < kStages && s < it; ++s)
+        failed = !mbar_wait(sm.full + s, static_cast<uint32_t>((it - 1 - s) / kStages) & 1u, a.wait_ns) || failed;
     }
     __syncwarp();
   } else {
@@ -268,13 +291,18 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
     int st = group;
     uint32_t ph = 0;
     for (int it = group; it < n_my; it += kGroups) {
-      if (!__all_sync(0xffffffffu, mbar_wait(sm.full + st, ph))) break;
+      const bool landed = __all_sync(0xffffffffu, mbar_wait(sm.full + st, ph, a.wait_ns));
       const float4* x = reinterpret_cast<const float4*>(sm.stage0 + st * sm.stage_bytes) + qoff;
       // column means of the input
       float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int i = g; i < a.N; i += G) cs = add4(cs, x[i << lqb]);
       part[gt] = cs;
-      group_bar(group);
+      // The group goes on or gives up as one: a warp that left alone would keep
+      // the others at their next barrier for good.
+      if (group_bar_or(group, !landed)) {
+        failed = true;
+        break;
+      }
       cs = part[q];
       for (int u = 1; u < G; ++u) cs = add4(cs, part[(u << lq) + q]);
       const float4 mu = make_float4(cs.x * inv_n, cs.y * inv_n, cs.z * inv_n, cs.w * inv_n);
@@ -318,6 +346,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mix_noalloc(const __grid_constant
 
   // The last CTA sums the partials in a fixed order (the result does not
   // depend on which CTA finishes last).
+  if (failed) total = Pair{__int_as_float(0x7fc00000), 0.f};
   const Pair ps = block_sum(total, sm.red);
   if (tid == 0) {
     a.partial[blockIdx.x] = static_cast<double>(ps.hi) + static_cast<double>(ps.lo);
@@ -399,11 +428,9 @@ asap_status reject(asap_status s, const char* msg) {
   return s;
 }
 
-}  // namespace
-
-extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, int64_t d, int64_t ld,
-                                        const int32_t* nbr, const float* wgt, int kp1, float* consensus_out,
-                                        void* cuda_stream) {
+asap_status mix_noalloc(const float* W_in, float* W_out, int N, int64_t d, int64_t ld, const int32_t* nbr,
+                        const float* wgt, int kp1, float* consensus_out, void* cuda_stream,
+                        unsigned long long wait_ns, long long drop_slab) {
   if (!W_in || !W_out || !nbr || !wgt || !consensus_out)
     return reject(ASAP_ERR_ARG, "asap_mix_noalloc: NULL pointer");
   if (N < 1 || N > kNoAllocMaxN) return reject(ASAP_ERR_ARG, "asap_mix_noalloc: need 1 <= N <= 256");
@@ -413,11 +440,11 @@ extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, 
   if ((reinterpret_cast<uintptr_t>(W_in) | reinterpret_cast<uintptr_t>(W_out)) & 15u)
     return reject(ASAP_ERR_ARG, "asap_mix_noalloc: W_in and W_out must be 16-byte aligned");
   {
-    // The built-in scratch bounds ld: 32,768 slabs of at most 16 KB.
+    // ld is limited to 32,768 slabs of at most 16 KB.
     int S_max = 256;
     while (S_max > 4 && static_cast<size_t>(N) * S_max * 4 > 16384) S_max >>= 1;
     if ((ld + S_max - 1) / S_max > kNoAllocMaxSlabs)
-      return reject(ASAP_ERR_ARG, "asap_mix_noalloc: ld too large for the built-in scratch "
+      return reject(ASAP_ERR_ARG, "asap_mix_noalloc: ld beyond the range its scratch was laid out for "
                                   "(at most 32768 slabs of 256 columns for N <= 16, 16 columns for N = 256)");
   }
   {
@@ -493,6 +520,8 @@ extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, 
   a.consensus_out = consensus_out;
   a.tickets = reinterpret_cast<unsigned int*>(base);
   a.slot = static_cast<int>(slot.calls % kSlots);
+  a.wait_ns = wait_ns;
+  a.drop_slab = drop_slab;
   a.partial = reinterpret_cast<double*>(base + kNoAllocTicketBytes) + static_cast<size_t>(a.slot) * kSlotPartials;
   const size_t smem = noalloc_smem(N, S, kp1);
   const int grid = static_cast<int>(std::min<long long>(a.n_slabs, std::min(slot.sm_count, kSlotPartials)));
@@ -504,4 +533,19 @@ extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, 
   }
   if (cudaGetLastError() != cudaSuccess) return reject(ASAP_ERR_CUDA, "asap_mix_noalloc: launch failed");
   return ASAP_OK;
+}
+
+}  // namespace
+
+extern "C" asap_status asap_mix_noalloc(const float* W_in, float* W_out, int N, int64_t d, int64_t ld,
+                                        const int32_t* nbr, const float* wgt, int kp1, float* consensus_out,
+                                        void* cuda_stream) {
+  return mix_noalloc(W_in, W_out, N, d, ld, nbr, wgt, kp1, consensus_out, cuda_stream, kWaitNs, -1);
+}
+
+extern "C" asap_status asap_debug_mix_noalloc(const float* W_in, float* W_out, int N, int64_t d, int64_t ld,
+                                              const int32_t* nbr, const float* wgt, int kp1, float* consensus_out,
+                                              void* cuda_stream, uint64_t wait_ns, int64_t drop_slab) {
+  if (wait_ns == 0) return reject(ASAP_ERR_ARG, "asap_debug_mix_noalloc: need wait_ns > 0");
+  return mix_noalloc(W_in, W_out, N, d, ld, nbr, wgt, kp1, consensus_out, cuda_stream, wait_ns, drop_slab);
 }

@@ -15,7 +15,7 @@ from parity import rel_err_rows
 pytestmark = pytest.mark.gpu
 
 
-def _run(W, d, nbr, wgt, calls=1):
+def _run(W, d, nbr, wgt, calls=1, drop_slab=None):
     import torch
 
     from paper_1612_08608_gb300._lib import load_library
@@ -25,9 +25,13 @@ def _run(W, d, nbr, wgt, calls=1):
     n, w = torch.from_numpy(nbr.astype(np.int32)).cuda(), torch.from_numpy(wgt.astype(np.float32)).cuda()
     cons = torch.empty(1, device="cuda")
     p = C.c_void_p
+    args = (p(W_in.data_ptr()), p(W_out.data_ptr()), N, d, ld, p(n.data_ptr()), p(w.data_ptr()), nbr.shape[1],
+            p(cons.data_ptr()), p(torch.cuda.current_stream().cuda_stream))
     for _ in range(calls):
-        st = lib.asap_mix_noalloc(p(W_in.data_ptr()), p(W_out.data_ptr()), N, d, ld, p(n.data_ptr()), p(w.data_ptr()),
-                                  nbr.shape[1], p(cons.data_ptr()), p(torch.cuda.current_stream().cuda_stream))
+        if drop_slab is None:
+            st = lib.asap_mix_noalloc(*args)
+        else:
+            st = lib.asap_debug_mix_noalloc(*args, 20_000_000, drop_slab)
         assert st == 0, lib.asap_last_error(None)
     torch.cuda.synchronize()
     return W_out.cpu().numpy(), cons.item()
@@ -71,3 +75,28 @@ def test_calls_of_different_sizes_in_turn():
         err = np.sqrt(((want - W.astype(np.float64).mean(axis=0)) ** 2).sum())
         assert rel_err_rows(got, want) <= 1e-6
         assert abs(cons - err) <= 1e-5 * err + 4 * 2.0 ** -24 * np.linalg.norm(W), (t, cons, err)
+
+
+# N = 24 and ld = 200,000 in slabs of 256 columns: 782 slabs, five or six for each of 152 CTAs (two groups on alternate
+# slabs, four stages); the slab that never lands is a CTA's first, one of the second group's, one that reuses a
+# stage, and the last
+@pytest.mark.parametrize("drop", [0, 152 + 7, 4 * 152 + 3, 781])
+def test_a_wait_that_runs_out_makes_the_consensus_error_nan(drop):
+    rng = np.random.default_rng(drop)
+    N, ld, S = 24, 200000, 256
+    W = rng.standard_normal((N, ld)).astype(np.float32)
+    nbr = np.stack([np.arange(N), (np.arange(N) + 1) % N], axis=1)
+    wgt = np.full((N, 2), 0.5)
+    want = 0.5 * (W.astype(np.float64) + W.astype(np.float64)[nbr[:, 1]])
+    got, cons = _run(W, ld, nbr, wgt, drop_slab=drop)
+    assert np.isnan(cons)
+    assert np.isnan(got[:, drop * S:(drop + 1) * S]).all()          # not written
+    # slabs of the other CTAs are there
+    other = [s for s in range(ld // S) if s % 152 != drop % 152]
+    for s in other[::50]:
+        assert rel_err_rows(got[:, s * S:(s + 1) * S], want[:, s * S:(s + 1) * S]) <= 1e-6
+    # the debug entry without a dropped slab, and the next calls, are whole
+    for d in (-1, None):
+        got, cons = _run(W, ld, nbr, wgt, drop_slab=d)
+        err = np.sqrt(((want - W.astype(np.float64).mean(axis=0)) ** 2).sum())
+        assert rel_err_rows(got, want) <= 1e-6 and abs(cons - err) <= 1e-5 * err
