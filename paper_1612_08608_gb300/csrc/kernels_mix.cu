@@ -653,6 +653,15 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
           if (!ok) {
             if (lane == 0) record_error(a.st, ASAP_ERR_CUDA, 0xfffffffeu, a.round);
             failed = true;
+            // A slab that never comes back: those who wait for copies may have
+            // given up, and the CTA's shared memory must not be given back with
+            // one in flight.  (A slab that comes back has landed, its entries too.)
+            const int slabs = min(it, n_my), lists = min(it + a.list_slots - a.stages, n_my);
+            if (lane < a.stages && lane < slabs)
+              mbar_wait_bounded(sm.full + lane, static_cast<uint32_t>((slabs - 1 - lane) / a.stages) & 1u);
+            if (ENTRIES && lane < a.list_slots && lane < lists)
+              mbar_wait_bounded(sm.lfull + lane, static_cast<uint32_t>((lists - 1 - lane) / a.list_slots) & 1u);
+            __syncwarp();
             break;
           }
         }
@@ -799,10 +808,18 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
       // Once a slab has landed, apply w -= eta/B (1 - eta l2)^-1 g to it and
       // release it to the compute warps.
       if (FUSED && quiet) {
-        int st = 0;
-        uint32_t ph = 0;
+        // The entry ring goes round with the stages: a slot is armed again when
+        // its slab's stage comes back, so its entries must have landed too.
+        int st = 0, sl = 0;
+        uint32_t ph = 0, lph = 0;
         for (int it = 0; it < n_my; ++it) {
-          if (!__all_sync(kFull, mbar_wait_bounded(sm.full + st, ph))) break;
+          bool here = mbar_wait_bounded(sm.full + st, ph);
+          if (ENTRIES) here = mbar_wait_bounded(sm.lfull + sl, lph) && here;
+          if (!__all_sync(kFull, here)) break;
+          if (ENTRIES && ++sl == a.list_slots) {
+            sl = 0;
+            lph ^= 1u;
+          }
           if (lane == 0) mbar_arrive(sm.ready + st);
           if (++st == a.stages) {
             st = 0;

@@ -188,3 +188,33 @@ def test_notify_ack_after_streamed_local_steps_equals_bsp(B):
             assert ctx.kernel_launches() - before == 1 + 40 * 4      # streamed: two steps, one update, one reduce
     assert np.array_equal(outs[0][0], outs[1][0])
     assert np.array_equal(outs[0][1][0], outs[1][1][0]) and np.array_equal(outs[0][1][1], outs[1][1][1])
+
+
+# A reduce that finds a flag missing passes its slabs on unwritten, and its entry ring with them: one slab a CTA,
+# and eight (the ring's six slots are used again)
+@pytest.mark.parametrize("sync", ["bsp", "notify_ack"])
+@pytest.mark.parametrize("N,d,max_len", [(6, 2003, 30), (8, 1300000, 300)])
+def test_missing_notify_and_the_rounds_after_it(N, d, max_len, sync):
+    from paper_1612_08608_gb300 import AsapError
+    B = 32
+    sh = inputs.sparse_custom(seed=5, N=N, d=d, rows=4 * B, max_len=max_len)
+    W0 = (0.1 * np.random.default_rng(2).standard_normal((N, d))).astype(np.float32)
+    outs = []
+    for stall in (False, True):
+        with _make(sh, N, 1, "ring", "logistic", B, 0.4, sync=sync) as ctx:
+            assert _uses_entries(ctx, sh, B)
+            ctx.write_params(W0, 0)
+            if stall:
+                for _ in range(3):
+                    ctx.set_wait_limit_ns(5_000_000)
+                    ctx.debug_skip_notify(N - 2)
+                    ctx.round(1)
+                    with pytest.raises(AsapError) as ei:
+                        ctx.sync()
+                    assert ei.value.name == "ASAP_ERR_TIMEOUT"
+                    ctx.write_params(W0, 0)
+                ctx.set_wait_limit_ns(200_000_000)
+            ctx.round(3)
+            outs.append((ctx.read_params()[0], ctx.read_metrics(0, 3)))
+    assert np.array_equal(outs[0][0], outs[1][0])
+    assert np.array_equal(outs[0][1][0], outs[1][1][0]) and np.array_equal(outs[0][1][1], outs[1][1][1])
