@@ -349,6 +349,13 @@ asap_status asap_debug_batch_image(int N, int64_t d, int batch, int slab_cols, i
                                    const float* const* y, unsigned char* image, int64_t cap, int64_t* image_bytes,
                                    int64_t* desc_out, int64_t* list_out);
 
+/* For tests and measurements: how the loaded CSR shards are laid out.
+ * out[0]: 1 column lists, 2 entries by column slab; out[1]: bytes of an entry
+ * (lists 12 and the list itself; entries 8 or 10); out[2]: 1 if the local steps
+ * before a round's last stream all of W instead of touching the entries'
+ * parameters one by one.  Host only. */
+asap_status asap_debug_shard_layout(asap_ctx* ctx, int32_t* out);
+
 /* Kernel kinds for per-kernel timing. */
 typedef enum {
   ASAP_KERNEL_LOCAL_STEP = 0, /* sparse margins, loss derivative, NOTIFY (a2-a4),

@@ -25,6 +25,7 @@ SIGNATURES = {
     "asap_set_stream": (C.c_int, [_P, _P]),
     "asap_set_shard_residency": (C.c_int, [_P, C.c_int]),
     "asap_shard_block_bytes": (C.c_int, [_P, C.c_int64, C.POINTER(C.c_uint64)]),
+    "asap_debug_shard_layout": (C.c_int, [_P, _P]),
     "asap_load_shards": (C.c_int, [_P, _P, _P, _P, _P, _P]),
     "asap_load_dense_shards": (C.c_int, [_P, _P, _P, _P]),
     "asap_local_step": (C.c_int, [_P]),

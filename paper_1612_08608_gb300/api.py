@@ -122,6 +122,13 @@ class Context:
         self._c(self._lib.asap_shard_block_bytes(self._h, rnd, C.byref(v)))
         return v.value
 
+    def debug_shard_layout(self):
+        """{"entries": by column slab (else column lists), "entry_bytes": bytes of an entry, "streams": local steps
+        before a round's last stream all of W}."""
+        v = np.empty(3, dtype=np.int32)
+        self._c(self._lib.asap_debug_shard_layout(self._h, _ptr(v)))
+        return {"entries": v[0] == 2, "entry_bytes": int(v[1]), "streams": v[2] == 1}
+
     def load_shards(self, shards=None, rowptr=None, col=None, val=None, y=None):
         if shards is not None:
             rowptr, col, val, y = shards.rowptr, shards.col, shards.val, shards.y

@@ -1454,6 +1454,15 @@ asap_status asap_shard_block_bytes(asap_ctx* c, int64_t round, uint64_t* bytes) 
   return ASAP_OK;
 }
 
+asap_status asap_debug_shard_layout(asap_ctx* c, int32_t* out) {
+  if (!c || !out) return fail(c, ASAP_ERR_ARG, "NULL argument");
+  if (!c->nb || c->loss == ASAP_LOSS_SOFTMAX) return fail(c, ASAP_ERR_ARG, "no CSR shards loaded");
+  out[0] = c->entries ? 2 : 1;
+  out[1] = !c->entries ? 12 : c->row_shift > 16 ? 8 : 10;
+  out[2] = c->stream_slabs ? 1 : 0;
+  return ASAP_OK;
+}
+
 asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const int32_t* const* col,
                              const float* const* val, const float* const* y, const int64_t* n_rows) {
   if (!c || !rowptr || !col || !val || !y || !n_rows) return fail(c, ASAP_ERR_ARG, "NULL argument");

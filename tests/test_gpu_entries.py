@@ -2,8 +2,7 @@
 slabs: products exported by the reduce, row sums, updates from the rows' r
 inside the reduce) against the oracle, round by round (1e-5 normwise per
 worker), at the edges of its row passes, runs and regions, and on both sides
-of the rule that chooses it.  Which layout a context uses shows in the bytes of
-a minibatch block: 8 or 10 an entry (plus padding) against 16."""
+of the rule that chooses it."""
 import numpy as np
 import pytest
 
@@ -14,9 +13,8 @@ from parity import sparse_round_matching
 pytestmark = pytest.mark.gpu
 
 
-def _uses_entries(ctx, sh, B):
-    E = sum(int(sh.rowptr[i][B]) for i in range(sh.N))
-    return ctx.shard_block_bytes(0) < 13 * E + 6 * sh.N * B + 512
+def _uses_entries(ctx):
+    return ctx.debug_shard_layout()["entries"]
 
 
 def _make(sh, N, k, kind, loss, B, lr, l2=0.0, tau=1, residency="device", sync="bsp", regen=False):
@@ -65,8 +63,7 @@ def test_rows_and_graphs(B, N, k, kind):
     sh = inputs.sparse_custom(seed=B, N=N, d=d, rows=3 * B, lengths=lengths)
     W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
     with _make(sh, N, k, kind, "logistic", B, 0.5, regen=kind == "random_regular") as ctx:
-        if N * B >= 93:                                # enough entries to tell by
-            assert _uses_entries(ctx, sh, B)
+        assert _uses_entries(ctx)
         sched = rounds.graph_schedule(kind, N, k, graph_seed=7, regenerate=kind == "random_regular")
         _check(ctx, sh, 4, B, "logistic", 0.5, sched, W0=W0)
 
@@ -79,7 +76,7 @@ def test_local_steps_l2_and_residency(residency, sync):
     sched = rounds.graph_schedule("random_regular", N, 3, graph_seed=7, regenerate=True)
     with _make(sh, N, 3, "random_regular", "hinge", B, 0.4, l2=0.02, tau=tau, residency=residency, sync=sync,
                regen=True) as ctx:
-        assert _uses_entries(ctx, sh, B)
+        assert _uses_entries(ctx)
         _check(ctx, sh, 3, B, "hinge", 0.4, sched, l2=0.02, tau=tau)
 
 
@@ -102,7 +99,7 @@ def test_runs_up_to_the_rule(hot_rows, entries):
                 u = np.unique(np.concatenate([u, rng.integers(1, d, 1).astype(np.int32)]))
             sh.col[i][a:e] = u
     with _make(sh, N, 2, "root", "logistic", B, 0.5) as ctx:
-        assert _uses_entries(ctx, sh, B) == entries
+        assert _uses_entries(ctx) == entries
         _check(ctx, sh, 4, B, "logistic", 0.5, rounds.graph_schedule("root", N, 2))
 
 
@@ -115,7 +112,7 @@ def test_regions_up_to_the_rule(per_row, entries):
     sh = inputs.sparse_custom(seed=per_row, N=N, d=1024, rows=2 * B, lengths=ln)
     sh.d = d
     with _make(sh, N, 1, "ring", "logistic", B, 0.5) as ctx:
-        assert _uses_entries(ctx, sh, B) == entries
+        assert _uses_entries(ctx) == entries
         _check(ctx, sh, 3, B, "logistic", 0.5, rounds.graph_schedule("ring", N, 1))
 
 
@@ -129,7 +126,7 @@ def test_empty_minibatches_and_two_runs_bit_identical():
     outs = []
     for mode in ("bsp", "bsp", "notify_ack"):
         with _make(sh, N, 1, "ring", "logistic", B, 0.5, sync=mode) as ctx:
-            assert _uses_entries(ctx, sh, B)
+            assert _uses_entries(ctx)
             ctx.round(7)
             outs.append((ctx.read_params()[0], ctx.read_metrics(0, 7)))
     for W, (lm, cm) in outs[1:]:
@@ -154,6 +151,7 @@ def test_local_steps_streamed_and_touched(kind, k, residency, max_len, streams):
     rng = np.random.default_rng(3)
     W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
     with _make(sh, N, k, kind, "logistic", B, lr, l2=l2, tau=tau, residency=residency) as ctx:
+        assert ctx.debug_shard_layout()["streams"] == streams
         before = ctx.kernel_launches()
         _check(ctx, sh, 2, B, "logistic", lr, rounds.graph_schedule(kind, N, k, graph_seed=7), l2=l2, tau=tau, W0=W0)
         # one gather at the start; per round tau steps, tau - 1 updates (and gathers, unless streamed), a reduce
@@ -168,8 +166,7 @@ def test_row_and_place_in_the_code(B, row_len, packed):
     sh = inputs.sparse_custom(seed=B, N=N, d=d, rows=2 * B, lengths=[np.full(2 * B, row_len)] * N)
     W0 = (0.1 * np.random.default_rng(2).standard_normal((N, d))).astype(np.float32)
     with _make(sh, N, 1, "complete", "logistic", B, 0.5, tau=2) as ctx:
-        E = N * B * row_len
-        assert (ctx.shard_block_bytes(0) < 9.9 * E + 6 * N * B + 4096) == packed, ctx.shard_block_bytes(0) / E
+        assert ctx.debug_shard_layout()["entry_bytes"] == (8 if packed else 10)
         _check(ctx, sh, 2, B, "logistic", 0.5, rounds.graph_schedule("complete", N, 1), tau=2, W0=W0)
 
 
@@ -202,7 +199,7 @@ def test_missing_notify_and_the_rounds_after_it(N, d, max_len, sync):
     outs = []
     for stall in (False, True):
         with _make(sh, N, 1, "ring", "logistic", B, 0.4, sync=sync) as ctx:
-            assert _uses_entries(ctx, sh, B)
+            assert _uses_entries(ctx)
             ctx.write_params(W0, 0)
             if stall:
                 for _ in range(3):
@@ -218,3 +215,26 @@ def test_missing_notify_and_the_rounds_after_it(N, d, max_len, sync):
             outs.append((ctx.read_params()[0], ctx.read_metrics(0, 3)))
     assert np.array_equal(outs[0][0], outs[1][0])
     assert np.array_equal(outs[0][1][0], outs[1][1][0]) and np.array_equal(outs[0][1][1], outs[1][1][1])
+
+
+# Without streaming, the update and the products of the next step walk the slabs, a CTA each while one wave of CTAs
+# covers them (1,216 on a GB300), else a warp each: 489 and 1,368 slabs of 1,024 columns; the first slab's region
+# takes several passes of a warp, its runs are of up to 14 rows; the last slab is ragged.
+@pytest.mark.parametrize("residency", ["device", "host"])
+@pytest.mark.parametrize("d", [500001, 1400001])
+def test_updates_walk_the_slabs_one_by_one(d, residency):
+    N, B, tau, lr, l2 = 8, 32, 3, 0.4, 0.02
+    sh = inputs.sparse_custom(seed=11, N=N, d=d, rows=7 * B, lengths=[np.full(7 * B, 30)] * N)
+    rng = np.random.default_rng(4)
+    for i in range(N):
+        sh.col[i][sh.rowptr[i][1:] - 1] = np.where(rng.random(7 * B) < 0.3, d - 1, sh.col[i][sh.rowptr[i][1:] - 1])
+        sh.col[i][sh.rowptr[i][:-1]] = rng.integers(0, 8, 7 * B)          # eight columns, about four rows each
+        sh.col[i][sh.rowptr[i][:-1] + 1] = rng.integers(8, 1000, 7 * B)
+    W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
+    with _make(sh, N, 1, "ring", "logistic", B, lr, l2=l2, tau=tau, residency=residency) as ctx:
+        layout = ctx.debug_shard_layout()
+        assert layout["entries"] and not layout["streams"]
+        before = ctx.kernel_launches()
+        _check(ctx, sh, 2, B, "logistic", lr, rounds.graph_schedule("ring", N, 1, graph_seed=7), l2=l2, tau=tau, W0=W0)
+        # a gather at the start; per round tau steps, tau - 1 updates and gathers, a reduce
+        assert ctx.kernel_launches() - before == 1 + 2 * (3 * tau - 1)

@@ -15,14 +15,16 @@ pytestmark = pytest.mark.gpu
 # d = 3,000 and 1,300,000 at N = 8: 94 slabs of 32 columns (one CTA each) and
 # 1,270 of 1,024 (more than one wave of CTAs, so a warp per slab unless a region
 # is long); the wide slabs' first region holds about 8 x cols distinct (worker,
-# column) pairs: a few (one partial pass of a warp), 1,017, and 2,128.
+# column) pairs: a few (one partial pass of a warp), about 1,000, and 2,100.
+# Column 0 is in every row that is not empty, so that the shards are laid out as
+# column lists at every size.
 @pytest.mark.parametrize("d", [3000, 1300000])
 @pytest.mark.parametrize("cols", [3, 128, 300])
 def test_slab_walks_match_oracle(d, cols):
     from paper_1612_08608_gb300 import Context
     N, B, T, tau = 8, 64, 2, 2
     rng = np.random.default_rng(cols)
-    sh = inputs.sparse_custom(seed=cols, N=N, d=cols, rows=4 * B, max_len=min(cols, 20))
+    sh = inputs.sparse_custom(seed=cols, N=N, d=cols, rows=4 * B, max_len=min(cols, 20), hot_col=0)
     for i in range(N):      # one column near the end, so that the last slab has a region of its own
         last = sh.rowptr[i][1:][np.diff(sh.rowptr[i]) > 0] - 1
         sh.col[i][last[rng.random(last.shape[0]) < 0.3]] = d - 1
@@ -33,6 +35,7 @@ def test_slab_walks_match_oracle(d, cols):
         ctx.set_graph("ring")
         ctx.set_schedule(local_steps=tau)
         ctx.load_shards(sh)
+        assert not ctx.debug_shard_layout()["entries"]
         W_t, _ = ctx.read_params()
         for t in range(T):
             ctx.round(1)
