@@ -199,10 +199,11 @@ def make_shards(rows, seed):
     return inputs.dense_softmax(seed=seed, N=w["N"], d=w["d"], C=w["C"], rows=rows)
 
 
-def kernel_work(sh):
+def kernel_work(sh, layout=None):
     """Algorithmic work of one launch of each kernel kind: (unit, amount, bound)
     or (unit, amount, bound, flops) when a memory-bound kernel also runs a
-    GEMM.  Sparse byte counts use the mean minibatch over a sample of batches."""
+    GEMM.  Sparse byte counts use the mean minibatch over a sample of batches and
+    the layout the context chose for the shards (Context.debug_shard_layout)."""
     import numpy as np
     w = WORKLOAD
     N, B, d = w["N"], w["B"], w["d"]
@@ -227,15 +228,19 @@ def kernel_work(sh):
         nnz += rp[-1] - rp[0]
         touched += np.unique(sh.col[i][rp[0]:rp[-1]]).shape[0]
     nnz, touched = nnz * N / samples, touched * N / samples
-    if w["name"] == "sparse_logistic_hashed":
+    if layout["entries"]:
         # entry layout: the local step adds up one product per entry and reads
         # a label and a length and writes r per row
         out["local_step"] = ("GB/s", 4.0 * nnz + 10.0 * N * B, "hbm")
         out["reduce"] = ("GB/s", 8.0 * N * ld, "hbm")
-        # local steps before the round's last: code, value and r per entry, w read and written per column, and for
-        # the next step's entries code, value, place and w read and a product written
-        out["apply"] = ("GB/s", 30.0 * nnz + 8.0 * touched, "hbm")
-        out["gather"] = ("GB/s", 18.0 * nnz, "hbm")
+        # the products of a step: code, value and place of an entry read (8 or 10 B), w of a column, a product written
+        gather = (layout["entry_bytes"] + 4.0) * nnz
+        # the update of a local step before the round's last: code and value of an entry, r of a row, w of a column
+        # read and written
+        update = 8.0 * nnz + 4.0 * N * B + 4.0 * touched
+        out["gather"] = ("GB/s", gather + 4.0 * touched, "hbm")
+        # streamed, it reads all of W once, for itself and for the next step's products
+        out["apply"] = ("GB/s", update + (gather + 4.0 * N * ld if layout["streams"] else 4.0 * touched), "hbm")
         return out
     # list layout: the fused local step reads every entry once (list position,
     # value, row, segment slot: 12 B), the w value and writes the column sum
@@ -604,7 +609,7 @@ def run_asap(args):
     assert np.isfinite(last_loss[0]) and np.isfinite(last_cons[0])
 
     pk = peaks_all()
-    work = kernel_work(sh)
+    work = kernel_work(sh, None if dense else ctx.debug_shard_layout())
     kernels = {}
     for name, wk in work.items():
         unit, amount, bound = wk[:3]

@@ -127,7 +127,7 @@ class Context:
         before a round's last stream all of W}."""
         v = np.empty(3, dtype=np.int32)
         self._c(self._lib.asap_debug_shard_layout(self._h, _ptr(v)))
-        return {"entries": v[0] == 2, "entry_bytes": int(v[1]), "streams": v[2] == 1}
+        return {"entries": bool(v[0] == 2), "entry_bytes": int(v[1]), "streams": bool(v[2] == 1)}
 
     def load_shards(self, shards=None, rowptr=None, col=None, val=None, y=None):
         if shards is not None:

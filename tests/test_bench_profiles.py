@@ -49,3 +49,23 @@ def test_committed_summaries_match_the_committed_kernels():
         assert os.path.exists(os.path.join(bench.ROOT, "paper_1612_08608_gb300", "csrc", source))
         traffic = bench.traffic_per_launch(workload, kernel)
         assert traffic is not None and traffic > 0, (summary, source)
+
+
+def test_kernel_bytes_follow_the_layout_not_the_workload(monkeypatch):
+    # 2 workers x 8 rows of 5 entries in distinct columns, in 100 (128 stored) columns
+    import numpy as np
+    from paper_1612_08608_gb300 import inputs
+    N, B, d = 2, 8, 100
+    sh = inputs.sparse_custom(seed=0, N=N, d=d, rows=B, lengths=[np.full(B, 5)] * N)
+    for i in range(N):
+        sh.col[i][:] = np.arange(40)
+    monkeypatch.setattr(bench, "WORKLOAD", dict(name="sparse_logistic_hashed", N=N, B=B, d=d, loss="logistic"))
+    E = N * B * 5                                          # entries, and columns touched
+    bytes_of = lambda **kw: {k: v[1] for k, v in bench.kernel_work(sh, kw).items()}
+    lists = bytes_of(entries=False, entry_bytes=12, streams=False)
+    assert lists == {"local_step": 20 * E + 4 * N * B, "reduce": 8 * N * 128, "apply": 16 * E, "gather": 12 * E}
+    touched = bytes_of(entries=True, entry_bytes=10, streams=False)
+    assert touched == {"local_step": 4 * E + 10 * N * B, "reduce": 8 * N * 128, "gather": 18 * E,
+                       "apply": 16 * E + 4 * N * B}
+    streamed = bytes_of(entries=True, entry_bytes=8, streams=True)
+    assert streamed["apply"] == (8 + 4 + 8 + 4) * E + 4 * N * B + 4 * N * 128
