@@ -349,6 +349,20 @@ asap_status asap_debug_batch_image(int N, int64_t d, int batch, int slab_cols, i
                                    const float* const* y, unsigned char* image, int64_t cap, int64_t* image_bytes,
                                    int64_t* desc_out, int64_t* list_out);
 
+/* The same for the entry layout (evenly spread columns): out (9 int64) receives
+ * the byte offsets of the labels (float [N][B]), the entries of each row
+ * (uint16 [N][B]), the slab offsets (int32 [n_slabs + 1]), and per entry its
+ * code (uint32), value (float) and place in its row (uint16; -1: in the code),
+ * then the bit at which a code's row begins, the entries of the largest slab
+ * region and of the longest run of one (worker, column).  A code is row <<
+ * row_bit | place << 16 (if it is there) | 0x8000 if the entry before has the
+ * same worker and column | 0x4000 if the next one has | worker * slab_cols +
+ * column in the slab; padding is 0xffffffff.  ASAP_ERR_ARG too for a run of more
+ * than 32 entries and for N * slab_cols of 16384 or more. */
+asap_status asap_debug_entry_image(int N, int64_t d, int batch, int slab_cols, int t, const int64_t* const* rowptr,
+                                   const int32_t* const* col, const float* const* val, const float* const* y,
+                                   unsigned char* image, int64_t cap, int64_t* image_bytes, int64_t* out);
+
 /* For tests and measurements: how the loaded CSR shards are laid out.
  * out[0]: 1 column lists, 2 entries by column slab; out[1]: bytes of an entry
  * (lists 12 and the list itself; entries 8 or 10); out[2]: 1 if the local steps

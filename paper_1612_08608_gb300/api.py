@@ -47,20 +47,25 @@ def build_graph(kind: str, N: int, k: int, graph_seed: int = 0, rnd: int = 0) ->
     return out
 
 
+def _shard_arrays(shards, batch: int, t: int):
+    """The pointer arrays of a shard set that holds minibatch t, and what keeps them alive."""
+    rp = [np.ascontiguousarray(a, dtype=np.int64) for a in shards.rowptr]
+    cl = [np.ascontiguousarray(a, dtype=np.int32) for a in shards.col]
+    vl = [np.ascontiguousarray(a, dtype=np.float32) for a in shards.val]
+    yl = [np.ascontiguousarray(a, dtype=np.float32) for a in shards.y]
+    if t < 0 or any((t + 1) * batch > a.shape[0] - 1 for a in rp):
+        raise ValueError("minibatch %d of %d rows is past the end of a shard" % (t, batch))
+    return tuple(_ptr_array(a) for a in (rp, cl, vl, yl)), (rp, cl, vl, yl)
+
+
 def debug_batch_image(shards, batch: int, slab_cols: int, t: int, ctas_per_worker: int = 1):
     """The image asap_load_shards builds for minibatch t (host only, for
     tests): (image bytes uint8, desc [N, 8] int64, (list byte offset, slab
     offsets byte offset, list length))."""
     lib = load_library()
-    rp = [np.ascontiguousarray(a, dtype=np.int64) for a in shards.rowptr]
-    cl = [np.ascontiguousarray(a, dtype=np.int32) for a in shards.col]
-    vl = [np.ascontiguousarray(a, dtype=np.float32) for a in shards.val]
-    yl = [np.ascontiguousarray(a, dtype=np.float32) for a in shards.y]
-    N = len(rp)
-    if t < 0 or any((t + 1) * batch > a.shape[0] - 1 for a in rp):
-        raise ValueError("minibatch %d of %d rows is past the end of a shard" % (t, batch))
-    args = (N, shards.d, batch, slab_cols, ctas_per_worker, t, _ptr_array(rp), _ptr_array(cl), _ptr_array(vl),
-            _ptr_array(yl))
+    ptrs, keep = _shard_arrays(shards, batch, t)
+    N = len(keep[0])
+    args = (N, shards.d, batch, slab_cols, ctas_per_worker, t, *ptrs)
     size = C.c_int64()
     desc = np.empty((N, 8), dtype=np.int64)
     lst = np.empty(3, dtype=np.int64)
@@ -71,6 +76,24 @@ def debug_batch_image(shards, batch: int, slab_cols: int, t: int, ctas_per_worke
     _check(lib, None, lib.asap_debug_batch_image(*args, _ptr(img), img.shape[0], C.byref(size), _ptr(desc),
                                                  _ptr(lst)))
     return img, desc, (int(lst[0]), int(lst[1]), int(lst[2]))
+
+
+def debug_entry_image(shards, batch: int, slab_cols: int, t: int):
+    """The entry layout asap_load_shards builds for minibatch t of evenly spread columns (host only, for tests):
+    (image bytes uint8, {byte offsets of y, len, soff, code, val, place (-1: in the code); row_shift, max_region,
+    max_run})."""
+    lib = load_library()
+    ptrs, keep = _shard_arrays(shards, batch, t)
+    args = (len(keep[0]), shards.d, batch, slab_cols, t, *ptrs)
+    size = C.c_int64()
+    out = np.empty(9, dtype=np.int64)
+    st = lib.asap_debug_entry_image(*args, None, 0, C.byref(size), _ptr(out))
+    if st != 1:                       # anything but "buffer too small" is a real error
+        _check(lib, None, st)
+    img = np.empty(size.value, dtype=np.uint8)
+    _check(lib, None, lib.asap_debug_entry_image(*args, _ptr(img), img.shape[0], C.byref(size), _ptr(out)))
+    names = ("y", "len", "soff", "code", "val", "place", "row_shift", "max_region", "max_run")
+    return img, {n: int(v) for n, v in zip(names, out)}
 
 
 class Context:

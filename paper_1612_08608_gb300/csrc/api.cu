@@ -731,6 +731,14 @@ struct EntryImage {
   const char* err = nullptr;
 };
 
+// EntryList::row_shift: row and place share 16 bits of the code where both fit.
+int entry_row_shift(int64_t max_len, int B) {
+  int place_bits = 1, row_bits = 0;
+  while ((1ll << place_bits) < max_len) ++place_bits;
+  while ((1 << row_bits) < B) ++row_bits;
+  return place_bits + row_bits <= 16 && place_bits < 16 ? 16 + place_bits : 16;
+}
+
 // Entries per slab and worker of minibatch t, counted into cnt[slab * N + i];
 // false with *err set for a column id outside [0, d).
 bool count_entries(int N, int B, int64_t d, int lS, int t, const int64_t* const* rowptr, const int32_t* const* col,
@@ -947,11 +955,7 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
     }
   }
   std::vector<EntryImage> built(nb);
-  // Row and place share 16 bits of the code where both fit.
-  int place_bits = 1, row_bits = 0;
-  while ((1ll << place_bits) < max_len) ++place_bits;
-  while ((1 << row_bits) < B) ++row_bits;
-  c->row_shift = place_bits + row_bits <= 16 && place_bits < 16 ? 16 + place_bits : 16;
+  c->row_shift = entry_row_shift(max_len, B);
   for_batches(nb, [&](int t) {
     build_entry_image(N, B, c->d, c->S, c->n_slabs, c->row_shift, t, rowptr, col, val, y, built[t]);
   });
@@ -1120,6 +1124,38 @@ asap_status asap_debug_batch_image(int N, int64_t d, int batch, int slab_cols, i
   list_out[0] = static_cast<int64_t>(bt.list_off);
   list_out[1] = static_cast<int64_t>(bt.soff_off);
   list_out[2] = bt.list_len;
+  return ASAP_OK;
+}
+
+asap_status asap_debug_entry_image(int N, int64_t d, int batch, int slab_cols, int t, const int64_t* const* rowptr,
+                                   const int32_t* const* col, const float* const* val, const float* const* y,
+                                   unsigned char* image, int64_t cap, int64_t* image_bytes, int64_t* out) {
+  if (N < 1 || N > kMaxWorkers || d < 1 || batch < 1 || batch > 65535 || t < 0 || !rowptr || !col || !val || !y ||
+      !image_bytes || !out)
+    return fail(nullptr, ASAP_ERR_ARG, "bad arguments to asap_debug_entry_image");
+  if (slab_cols < 8 || slab_cols > 1024 || (slab_cols & (slab_cols - 1)) ||
+      static_cast<int64_t>(N) * slab_cols > kEntryOff)
+    return fail(nullptr, ASAP_ERR_ARG, "slab_cols must be a power of two in [8, 1024], N * slab_cols < 16384");
+  int64_t max_len = 0;
+  for (int i = 0; i < N; ++i)
+    for (int64_t r = static_cast<int64_t>(t) * batch; r < static_cast<int64_t>(t + 1) * batch; ++r)
+      max_len = std::max(max_len, rowptr[i][r + 1] - rowptr[i][r]);
+  if (max_len > 65535) return fail(nullptr, ASAP_ERR_ARG, "a row is too long for the entry layout");
+  const int64_t ld = (d + 63) / 64 * 64;
+  const int row_shift = entry_row_shift(max_len, batch);
+  EntryImage im;
+  build_entry_image(N, batch, d, slab_cols, (ld + slab_cols - 1) / slab_cols, row_shift, t, rowptr, col, val, y, im);
+  if (im.err) return fail(nullptr, ASAP_ERR_ARG, im.err);
+  if (im.max_run > kEntryRun) return fail(nullptr, ASAP_ERR_ARG, "a column has too many entries for the entry layout");
+  *image_bytes = static_cast<int64_t>(im.img.size());
+  if (!image || cap < static_cast<int64_t>(im.img.size())) return fail(nullptr, ASAP_ERR_ARG, "image buffer too small");
+  std::memcpy(image, im.img.data(), im.img.size());
+  const int64_t v[9] = {static_cast<int64_t>(im.off.y),    static_cast<int64_t>(im.off.len),
+                        static_cast<int64_t>(im.off.soff), static_cast<int64_t>(im.off.code),
+                        static_cast<int64_t>(im.off.val),  row_shift > 16 ? -1 : static_cast<int64_t>(im.off.place),
+                        row_shift,                         im.max_region,
+                        im.max_run};
+  std::memcpy(out, v, sizeof v);
   return ASAP_OK;
 }
 
