@@ -321,8 +321,8 @@ struct MixSmem {
   int* nbr;
   float* wgt;
   F2* scratch;       // two pairs per warp
-  int* flags;        // [0]: fail, [1]: last, [2]: failed CTAs of the launch (last CTA), [3]: slabs whose NOTIFY
-                     // the producer has seen (gated reduces on the entry layout)
+  int* flags;        // [0]: fail, [1]: last, [2]: failed CTAs of the launch (last CTA), [3]: slabs whose workers'
+                     // NOTIFY the producer has seen (gated reduces on the entry layout)
   unsigned* seen;    // [32]: bitmap of workers whose NOTIFY this CTA has seen (gated reduces)
 };
 
@@ -718,7 +718,12 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
             if (acquired && lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
           }
         }
-        if (ENTRIES && gated && it < n_my && lane == 0) st_release_cta(sm.flags + 3, it + 1);
+        // The updater warps may look up r for the slabs passed, and for all of them
+        // once every worker has been seen.  (Only ever the slabs passed, the early
+        // look-up mostly missed its turn: N = 64, d = 2^20, 110 entries a row 150
+        // us a NOTIFY_ACK round, now 123; 150 entries a row 170, now 155.)
+        if (ENTRIES && gated && it < n_my && lane == 0)
+          st_release_cta(sm.flags + 3, n_seen == a.N ? 0x7fffffff : it + 1);
         if (it < n_my && lane == 0) {
           const long long slab = blockIdx.x + it * stride;
           unsigned char* base = sm.stage0 + st * sm.stage_bytes;
