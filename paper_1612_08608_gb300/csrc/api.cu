@@ -1035,18 +1035,26 @@ void fill_entry_args(const asap_ctx* c, MixArgs* a, const unsigned char* bt, int
 }
 
 // Consumer warps of a local-step CTA: four, or more while a CTA has more than
-// one tile of its worker's largest minibatch to walk, the grid's CTAs still fit
-// on the device at once, and partial margins fit shared memory.
+// one tile of its worker's largest minibatch to walk, partial margins fit shared
+// memory, and the workers' clusters still fit on the device at once.  The driver
+// says how many do: a cluster's CTAs share a GPC, so that sixteen clusters of
+// eight do not fit 152 SMs at one CTA per SM (N = 16, d = 200,000, B = 1024, 40
+// entries a row, column lists, us a BSP round: four warps 47.7, eight, two CTAs
+// per SM, 36.4, twelve, one, in two waves 45.3).
 int local_step_warps(const asap_ctx* c, int max_nnz) {
   int warps = 4;
   if (c->B > kRSmemRows) return warps;
-  const int64_t ctas = static_cast<int64_t>(c->sharded ? c->own_n : c->N) * c->step_q;
+  const int workers = c->sharded ? c->own_n : c->N;
   const int64_t share = (static_cast<int64_t>(max_nnz) + c->step_q - 1) / c->step_q + kSlotSegment;
   while (warps < 12 && share > static_cast<int64_t>(warps) * kSlotSegment) {
     const int next = warps + 4;
-    const size_t smem = local_step_smem_bytes(c->B, c->step_stages, next);
-    const int64_t per_sm = std::min<int64_t>(next == 8 ? 3 : 2, (227 << 10) / static_cast<int64_t>(smem + 1024));
-    if (per_sm < 1 || ctas > per_sm * c->sm_count) break;
+    int clusters = 0;
+    if (local_step_clusters(c->loss, next, c->step_q, local_step_smem_bytes(c->B, c->step_stages, next), &clusters) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      break;
+    }
+    if (clusters < workers) break;
     warps = next;
   }
   return warps;

@@ -248,6 +248,8 @@ asap_status build_graph_host(asap_graph_kind kind, int N, int k, uint64_t seed, 
 cudaError_t launch_local_step(const LocalStepArgs& a, int loss, int warps, size_t smem, cudaStream_t s);
 size_t local_step_smem_bytes(int B, int stages, int warps);
 cudaError_t local_step_configure(int loss, int warps);
+// Clusters of Q local-step CTAs that the device holds at once (0: none).
+cudaError_t local_step_clusters(int loss, int warps, int Q, size_t smem, int* clusters);
 cudaError_t launch_apply_update(float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,
                                 int S, int max_region, const float* gsum, float scale, int sm_count, cudaStream_t s);
 cudaError_t launch_gather_wv(const float* W, int64_t ld, const uint32_t* list, const int* slab_off, long long n_slabs,

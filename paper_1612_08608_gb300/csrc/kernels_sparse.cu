@@ -812,6 +812,25 @@ cudaError_t local_step_configure(int loss, int warps) {
   });
 }
 
+cudaError_t local_step_clusters(int loss, int warps, int Q, size_t smem, int* clusters) {
+  *clusters = 0;
+  if (smem > (227u << 10)) return cudaSuccess;
+  cudaError_t e = local_step_configure(loss, warps);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(Q);
+  cfg.blockDim = dim3(local_step_threads(warps));
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = Q;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return with_kernel(loss, warps, [&](auto kernel) { return cudaOccupancyMaxActiveClusters(clusters, kernel, &cfg); });
+}
+
 cudaError_t launch_local_step(const LocalStepArgs& a, int loss, int warps, size_t smem, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.N * a.Q);

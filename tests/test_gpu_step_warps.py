@@ -16,8 +16,19 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("row_len", [1, 60, 64, 65, 100, 150, 171, 240, 257, 300, 500])
 @pytest.mark.parametrize("loss", ["hinge", "logistic"])
 def test_step_warps_match_oracle(row_len, loss):
+    _check(4, 96, row_len, loss)
+
+
+# many rows: shared memory leaves an SM two CTAs of eight warps, one of twelve, or one of eight; sixteen workers'
+# clusters do not all fit at one CTA per SM
+@pytest.mark.parametrize("N,B", [(16, 1024), (8, 2000), (16, 2048), (16, 2049)])
+def test_step_warps_with_many_rows(N, B):
+    _check(N, B, 40, "logistic")
+
+
+def _check(N, B, row_len, loss):
     from paper_1612_08608_gb300 import Context
-    N, d, B = 4, 2000, 96
+    d = 2000
     sh = inputs.sparse_custom(seed=row_len, N=N, d=d, rows=2 * B, hot_col=11,      # runs of 96: the list layout
                               lengths=[np.full(2 * B, row_len)] * N)
     sched = rounds.graph_schedule("ring", N, 1)
