@@ -147,8 +147,8 @@ asap_status asap_set_stream(asap_ctx* ctx, void* cuda_stream);
 asap_status asap_set_shard_residency(asap_ctx* ctx, asap_residency residency);
 
 /* Bytes of the minibatch block that round `round` reads (all workers: the
- * labels and the entries with their index, about 10 bytes an entry where
- * columns are spread evenly, 16 where they are skewed).  With HOST residency
+ * labels and the entries with their index, 8 or 10 bytes an entry where
+ * columns are spread evenly, about 16 where they are skewed).  With HOST residency
  * this is what one round copies to the GPU.  Host only. */
 asap_status asap_shard_block_bytes(asap_ctx* ctx, int64_t round, uint64_t* bytes);
 

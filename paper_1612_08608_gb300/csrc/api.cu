@@ -391,8 +391,11 @@ asap_status configure_mix_launch(asap_ctx* c, int mode) {
   };
   // The reduce alone asks for about 96 KB at a time: enough to stream at full
   // rate, while more only queues in the memory system (N = 128, d = 10^7: 0.98 of
-  // HBM with three 32 KB slabs in flight, 0.91 with four); in rows of 128 bytes
-  // for 128 KB (N = 256, d = 10^6, k = 4: 0.84 with four, 0.81 with three).
+  // HBM with three 32 KB slabs in flight, 0.91 with four).  Rows of at most 128
+  // bytes gain from 128 KB where rows are narrow or neighbours many (96 KB and 128
+  // KB, us: N = 512, d = 500,000, k = 2 462 and 441; N = 256, d = 10^6, k = 6 431
+  // and 391), and lose a little elsewhere (N = 256, d = 10^6, k = 4 374 and 372, k =
+  // 2 366 and 379, k = 1 370 and 387; N = 300, d = 300,000, k = 4 168 and 172).
   int want = 4;
   if (mode == kMixPlain) {
     const size_t slab = mix_stage_bytes(c->S, c->rows_pad, 0, mode);
@@ -984,10 +987,14 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   c->entries = true;
   // A local step before a round's last: stream every slab once, for its update
   // and the next step's products, or touch the entries' parameters one by one,
-  // twice.  Streaming pays from about one parameter in 24 touched (N = 64, d =
-  // 2^20, one in 20: 106 us against 75 + 57; N = 20, d = 200,000, one in 17: 16.0
-  // against 10.2 + 8.7; N = 16, d = 10^6, one in 83: 22.6 against 11.2 + 9.6; N =
-  // 70, d = 230,000, one in 230: 33 against 8 + 8) and two slabs' worth of them.
+  // twice.  With one parameter in 24 touched streaming pays at every size (a
+  // round of four local steps, touched and streamed, us: N = 16, d = 200,000 60.8
+  // and 47.0; N = 16, d = 10^6 141 and 113; N = 24, d = 10^6 185 and 174; N = 64,
+  // d = 2^20 486 and 427; N = 100, d = 10^6 718 and 610).  With fewer it depends
+  // on the size: they break even at one in 28 for W of 96 MB, in 44 for 268 MB, in
+  // 48 for 400 MB, in 64 for 64 MB, which L2 holds, and at 13 MB streaming still
+  // pays at one in 128; the line lies where no size loses.  (Fewer than 16,384
+  // parameters, two slabs, are touched.)
   const int64_t params = static_cast<int64_t>(N) * c->ld;
   c->stream_slabs = 24 * max_nnz >= params && params >= 16384;
   if (c->stream_slabs) CU(entry_step_configure(), "configuring the local update kernel");

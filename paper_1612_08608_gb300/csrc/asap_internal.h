@@ -128,12 +128,17 @@ constexpr uint32_t kEntryNext = 0x8000u;      // so has the entry before (set in
 
 // It is used when every slab region of every minibatch holds at most
 // kEntryRegion entries and no column of a worker's minibatch more than
-// kEntryRun: both bound the chain of the reduce's updater warps, which look
-// up an r per entry (480 entries in one pass), and a region's 10 bytes an
-// entry in every stage and 12 in the entry ring must leave the reduce
-// three shared-memory stages or more; a run must fit the 32 entries a warp holds.  Above, the list layout's column sums, formed
-// outside the reduce, are the better split.  The table of products is
-// rectangular, kEntryWaste bounds what padding to the longest row may cost.
+// kEntryRun.  A region bounds the chain of the reduce's updater warps, which
+// look up an r per entry (480 entries in one pass), and takes 10 bytes an entry
+// in every stage and 12 in the entry ring: up to 704 entries leave three stages
+// of 32 KB slabs, two must fit.  With longer regions (allowed up to 1,300 in a
+// copy; us a round, lists and entries, BSP): N = 64, d = 2^20, 660 entries on
+// average 168 and 162, 800 181 and 195; N = 4, d = 3,000, 817 17.5 and 19.8; N =
+// 256, d = 10^5, 921 89.9 and 92.4; but N = 32, d = 500,000, 838 73.4 and 55.7; N
+// = 16, d = 10^6, 838 68.3 and 56.6: one line for all sizes lies where no size
+// loses.  A run must fit the 32 entries a warp holds.  The table of products is
+// rectangular, kEntryWaste bounds what padding to the longest row may cost (at
+// 7.5 times, N = 32, d = 500,000, rows of 2 and 16, 36.7 us against 44.1 with lists).
 constexpr int kEntryRegion = 704;
 constexpr int kEntryRun = 32;
 constexpr int kEntryWaste = 8;

@@ -18,9 +18,10 @@
 // the local step of hashed logistic regression (N = 64, d = 2^20, B = 512, 100
 // entries a row) went from 47 to 11.5 us and the reduce from 106 to 128 us (150
 // to 132 us a round), and a minibatch takes 8 or 10 instead of 16 bytes an entry
-// (250 to 140 us a round with host-resident shards, which the copy bounds).
-// entries and columns with short runs (kEntryRegion, kEntryRun); skewed
-// columns stay with the list layout.
+// (250 to 140 us a round with host-resident shards, which the copy bounds).  The
+// layout is for minibatches whose slabs all hold few entries and whose columns
+// have short runs (kEntryRegion, kEntryRun); skewed columns stay with the list
+// layout.
 #include <cuda_runtime.h>
 
 #include <cstdint>

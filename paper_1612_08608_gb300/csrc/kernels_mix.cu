@@ -37,9 +37,9 @@
 //
 // Protocol (Section 4, NOTIFY-ACK): before it writes anything each CTA waits,
 // with a time limit, until ready[j] == round+1 for every worker j and
-// consumed[j] >= round (a gated reduce: before it reads).  The last CTA to finish (ticket) reduces the metric
-// partials in a fixed order and ACKs: consumed[j] = round+1,
-// stamp_next[j] = round+1.
+// consumed[j] >= round (a gated reduce: before it reads).  The last CTA to
+// finish (ticket) reduces the metric partials in a fixed order and ACKs:
+// consumed[j] = round+1, stamp_next[j] = round+1.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -62,10 +62,11 @@ constexpr unsigned long long kTmaWaitNs = 2000000000ull;   // 2 s: a TMA load ne
 // ends.  Two groups overlap two chains, and with half the threads a thread
 // has twice the rows, hence loads, in flight (N = 256, d = 10^6, k = 4: 414 ->
 // 363 us a reduce).  On the entry layout, where the stages' turnaround is the
-// bound, the shorter life of a slab in one group is worth more (hashed
-// workload: 141 us against 147 with two groups).  The number of stages is a multiple of the
-// groups, so that a stage always belongs to the same group (its warps wait for
-// every phase of the stage's barriers, which parities need).
+// bound, the shorter life of a slab in one group is worth more (hashed workload,
+// N = 64, d = 2^20, k = 4: 127 us against 160 with two groups; no other shape
+// was tried).  The number of stages is a multiple of the groups, so that a stage
+// always belongs to the same group (its warps wait for every phase of the
+// stage's barriers, which parities need).
 constexpr int mix_groups(int mode) { return mode == kMixEntries ? 1 : 2; }
 // Threads of a group: at least the 256 column quads of the widest slab.
 constexpr int mix_group_threads(int mode) { return kMixComputeWarps * 32 / mix_groups(mode); }
@@ -380,9 +381,9 @@ __device__ __forceinline__ MixSmem carve(unsigned char* raw, const MixArgs& a, i
 // 64, d = 2^20, ~400 entries a slab, 1.6 us a slab streamed): codes and r looked
 // up in the landed slab 167 us a reduce; r early, runs read in a loop 144; so,
 // 140 us then, 128 us now that the producer issues a slab before it adds up the
-// last one's column sums.  In a gated reduce r is read only after the NOTIFY of its worker:
-// early for slabs the producer has passed (sm.flags[3]), else in the landed
-// slab.
+// last one's column sums.  In a gated reduce r is read only after the NOTIFY of
+// its worker: early for slabs the producer has passed, and for all once it has
+// seen every worker (sm.flags[3]), else in the landed slab.
 // STORE: each updated value also goes to the stored parameters (a.step_w).
 template <bool STORE>
 __device__ __forceinline__ void update_entries(const MixSmem& sm, const MixArgs& a, int n_slabs, bool gated, int lS,

@@ -53,10 +53,11 @@ constexpr int kNoAllocMaxDevices = 64;
 
 // [0, 256): ticket counters; [256, 256 + 8 * kNoAllocMaxSlabs): double
 // partials, one per CTA.  (The largest ld that a call takes is 32,768 slabs of at
-// most 16 KB: the partials were one per slab when it was set.)  Calls take kSlots slots of both in turn.  A call's last CTA
-// leaves its own ticket at zero, and clears the one half the slots away: calls
-// that overlapped against the rules (their stream order is the caller's
-// business) cannot spoil more than the calls right after them.
+// most 16 KB: the partials were one per slab when it was set.)  Calls take
+// kSlots slots of both in turn.  A call's last CTA leaves its own ticket at zero,
+// and clears the one half the slots away: calls that overlapped against the
+// rules (their stream order is the caller's business) cannot spoil more than the
+// calls right after them.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 constexpr int kSlots = 32;
