@@ -1792,6 +1792,7 @@ asap_status asap_local_step(asap_ctx* c) {
       a.skip_worker = skip;
       a.mscale = s_scale;
       a.notify = last ? 1 : 0;
+      a.late_trigger = last && c->stream_slabs && c->tau > 1 && c->sync_mode != kSyncBsp ? 1 : 0;
       time_begin(c, ASAP_KERNEL_LOCAL_STEP);
       CU(launch_row_step(a, c->loss, n_step, c->stream), "launching the local-step kernel");
       time_end(c);

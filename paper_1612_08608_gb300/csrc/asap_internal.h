@@ -162,6 +162,7 @@ struct RowStepArgs {
   int skip_worker;
   float mscale;
   int notify;
+  int late_trigger;            // let the next kernel in only once the one before is complete
 };
 
 // Arguments of the stochastic reduce.

@@ -70,8 +70,10 @@ __global__ void __launch_bounds__(kThreads) k_row_step(const RowStepArgs a) {
   const int b_end = min((q + 1) * a.rows, a.B);
   // The stochastic reduce that follows is a programmatic dependent; this
   // grid is one of the previous round's reduce.  Labels and row lengths are
-  // static batch data, read before that reduce is waited for.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // static batch data, read before that reduce is waited for.  A gated reduce
+  // does not wait for the grids before it: one that follows a streamed update
+  // of W is let in only when that grid's writes are known to be there.
+  if (!a.late_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   float lsum = 0.f;
   bool waited = false;
   for (int b0 = q * a.rows; b0 < b_end; b0 += kRowsAtOnce) {
@@ -83,6 +85,7 @@ __global__ void __launch_bounds__(kThreads) k_row_step(const RowStepArgs a) {
     if (!waited) {
       asm volatile("griddepcontrol.wait;" ::: "memory");
       waited = true;
+      if (a.late_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     const float* p = a.prod + row * a.row_stride;
     float m = 0.f;

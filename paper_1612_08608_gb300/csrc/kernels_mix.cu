@@ -602,6 +602,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) k_mix(const __grid_constant__ 
   if (gated) {
     check_flags(tid, kMixThreads);
     __syncthreads();
+    // W is there by the ACKs; the copies read it through the async proxy.
+    if (warp == kProducerWarp) asm volatile("fence.proxy.async.global;" ::: "memory");
   }
   bool failed = gated && sm.flags[0] != 0;
   bool quiet = false;                    // a flag was missing: pass the slabs on, write nothing

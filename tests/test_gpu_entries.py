@@ -170,12 +170,20 @@ def test_row_and_place_in_the_code(B, row_len, packed):
         _check(ctx, sh, 2, B, "logistic", 0.5, rounds.graph_schedule("complete", N, 1), tau=2, W0=W0)
 
 
-@pytest.mark.parametrize("B", [2, 24])
-def test_notify_ack_after_streamed_local_steps_equals_bsp(B):
+@pytest.mark.parametrize("B,halves", [(2, False), (24, False), (24, True)])
+def test_notify_ack_after_streamed_local_steps_equals_bsp(B, halves):
     # a gated reduce starts while the round's last local step runs, and reads parameters that the step before has
-    # updated by streaming the slabs
+    # updated by streaming the slabs; `halves`: a round's steps touch one half of the columns each, so that the reduce
+    # has no worker to wait for in the slabs that the streamed update has written
     N, d = 21, 30011 if B == 24 else 2003
     sh = inputs.sparse_custom(seed=4, N=N, d=d, rows=6 * B, max_len=300)
+    if halves:
+        half = d // 2
+        for i in range(N):
+            for r in range(6 * B):
+                a, e = sh.rowptr[i][r:r + 2]
+                c = np.random.default_rng(1000 * i + r).choice(half, e - a, replace=False)
+                sh.col[i][a:e] = np.sort(c) + (half if (r // B) % 2 else 0)
     outs = []
     for sync in ("bsp", "notify_ack"):
         with _make(sh, N, 2, "root", "logistic", B, 0.4, l2=0.02, tau=2, sync=sync) as ctx:
