@@ -947,6 +947,19 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   const int64_t table = static_cast<int64_t>(N) * B * stride;
   if (max_len > 65535 || table > kEntryWaste * max_nnz + 65536 || table >= (1ll << 31)) return ASAP_OK;
   if (max_nnz > static_cast<int64_t>(kEntryRegion) * c->n_slabs) return ASAP_OK;
+  // Few entries in slabs of many workers: the entry layout's reduce, one compute
+  // group, mixes narrow slabs slower than the list layout's two, and what it saves
+  // in the local step is little.  Speed of entries over lists, BSP and NOTIFY_ACK: N =
+  // 300, d = 500,000, one entry a slab 0.68 and 0.68, 92 0.72 and 0.74; N = 256, d =
+  // 10^6, 10 entries 0.90 and 0.84, 42 0.96 and 0.99, 157 1.09 and 1.12; N = 512, d =
+  // 128,000, 10 entries 0.67 and 0.79, 200 0.76 and 0.99, 400 0.95 and 1.09; N = 100,
+  // d = 512,000, 10 0.83 and 0.79, 50 0.87 and 0.85, 200 1.00 and 1.01.  While L2
+  // holds most of W and of the next W, up to about 80 MB each, 65 to 256 workers lose
+  // less (0.8 to 1.0) and gain between local steps (up to 1.2; from there on 0.95 to
+  // 1.08); 64 or fewer lose only in NOTIFY_ACK with next to no entries.
+  const int64_t w_bytes = 4 * static_cast<int64_t>(N) * c->ld;
+  if (N > 64 && (N > 256 || w_bytes > (80ll << 20)) && 5 * max_nnz < 2 * static_cast<int64_t>(N) * c->n_slabs)
+    return ASAP_OK;
   {
     std::vector<int32_t> cnt(static_cast<size_t>(c->n_slabs) * N, 0);
     const char* err = nullptr;

@@ -246,3 +246,16 @@ def test_updates_walk_the_slabs_one_by_one(d, residency):
         _check(ctx, sh, 2, B, "logistic", lr, rounds.graph_schedule("ring", N, 1, graph_seed=7), l2=l2, tau=tau, W0=W0)
         # a gather at the start; per round tau steps, tau - 1 updates and gathers, a reduce
         assert ctx.kernel_launches() - before == 1 + 2 * (3 * tau - 1)
+
+
+# With many workers and few entries a slab (less than two for five workers) the column lists are taken, from 257
+# workers at any size, from 65 where W is more than 80 MB: either side of each line
+@pytest.mark.parametrize("N,d,B,row_len,entries", [(300, 3000, 16, 4, False), (300, 3000, 16, 5, True),
+                                                   (256, 3000, 8, 2, True), (65, 330000, 16, 150, True),
+                                                   (65, 330000, 16, 100, False), (65, 320000, 16, 100, True),
+                                                   (64, 340000, 8, 2, True)])
+def test_few_entries_of_many_workers(N, d, B, row_len, entries):
+    sh = inputs.sparse_custom(seed=N, N=N, d=d, rows=2 * B, lengths=[np.full(2 * B, row_len)] * N)
+    with _make(sh, N, 1, "ring", "logistic", B, 0.4, tau=2) as ctx:
+        assert _uses_entries(ctx) == entries
+        _check(ctx, sh, 1, B, "logistic", 0.4, rounds.graph_schedule("ring", N, 1), tau=2)
