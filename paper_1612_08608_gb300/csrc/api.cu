@@ -731,6 +731,7 @@ struct EntryImage {
   std::vector<unsigned char> img;
   asap_ctx::EntryOffsets off{};
   int max_region = 0, max_run = 0;
+  int max_hot = 0;             // most entries that runs of kHotRun or more hold in one slab
   const char* err = nullptr;
 };
 
@@ -816,6 +817,7 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int ro
   for (long long s = 0; s < n_slabs; ++s) {
     const size_t start = code.size();
     soff[s] = static_cast<int32_t>(start);
+    int hot = 0;
     for (int i = 0; i < N; ++i) {
       const int32_t p1 = at[static_cast<size_t>(s) * N + i];
       std::stable_sort(items.begin() + p0, items.begin() + p1,
@@ -824,6 +826,7 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int ro
         for (q = p + 1; q < p1 && ((items[q].code ^ items[p].code) & kEntryOff) == 0u;) ++q;
         im.max_run = std::max(im.max_run, q - p);
         if (q - p > kEntryRun) return;
+        if (q - p >= kHotRun) hot += q - p;
         const size_t at32 = (code.size() - start) & 31u;
         if (at32 + static_cast<size_t>(q - p) > 32) pad_to(code.size() + 32 - at32);
         for (int32_t j = p; j < q; ++j) {
@@ -836,6 +839,7 @@ void build_entry_image(int N, int B, int64_t d, int S, long long n_slabs, int ro
     }
     pad_to(start + (code.size() - start + 7) / 8 * 8);
     im.max_region = std::max(im.max_region, static_cast<int>(code.size() - start));
+    im.max_hot = std::max(im.max_hot, hot);
     if (code.size() >= (1ull << 31)) {
       im.err = "column list of a minibatch too long";
       return;
@@ -975,12 +979,23 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   for_batches(nb, [&](int t) {
     build_entry_image(N, B, c->d, c->S, c->n_slabs, c->row_shift, t, rowptr, col, val, y, built[t]);
   });
-  int max_region = 0;
+  int max_region = 0, max_run = 0, max_hot = 0;
   for (const EntryImage& im : built) {
     if (im.err) return fail(c, ASAP_ERR_ARG, im.err);
     if (im.max_region > kEntryRegion || im.max_run > kEntryRun) return ASAP_OK;
     max_region = std::max(max_region, im.max_region);
+    max_run = std::max(max_run, im.max_run);
+    max_hot = std::max(max_hot, im.max_hot);
   }
+  // Hot columns: a run is added up one entry after the other, and the slab that
+  // holds many long ones paces the launch, where a column list holds one item a
+  // worker.  Speed of entries over lists by the entries of the hot column times its
+  // run, BSP (two local steps): 2,048 1.02 to 1.14, 4,096 1.0 to 1.1, 6,144 0.91 to
+  // 1.08, 8,192 0.91 to 0.95, 10,240 0.81 to 0.93, 16,384 0.75 to 0.80.  Where a warp
+  // walks the slab of an update, 1,024 0.97 (1.0), 1,536 0.92 (0.87), 2,560 0.85 to
+  // 0.92 (0.77), 4,096 0.90 (0.71), 10,240 0.82 (0.42), 16,384 0.77 (0.36).
+  const int64_t hot_work = static_cast<int64_t>(max_hot) * max_run;
+  if (hot_work > (slab_per_cta(c->n_slabs, max_region, c->sm_count) ? 6000 : 1500)) return ASAP_OK;
   if (mix_smem_bytes(N, std::min(c->k + 1, kMaxKp1Sparse), c->S, c->rows_pad, 2, max_region, kMixEntries,
                      2 + kEntryAhead) >
       (220u << 10))

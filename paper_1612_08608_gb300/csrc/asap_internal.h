@@ -142,6 +142,7 @@ constexpr uint32_t kEntryNext = 0x8000u;      // so has the entry before (set in
 constexpr int kEntryRegion = 704;
 constexpr int kEntryRun = 32;
 constexpr int kEntryWaste = 8;
+constexpr int kHotRun = 4;               // a run from which a column counts as hot (load_entries)
 constexpr int kEntryAhead = 2;           // slabs by which the reduce's entry ring runs ahead of its slabs
 constexpr int kRowStepRows = 32;         // rows a local-step CTA works on at once
 

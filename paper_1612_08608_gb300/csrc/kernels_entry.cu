@@ -20,8 +20,8 @@
 // to 132 us a round), and a minibatch takes 8 or 10 instead of 16 bytes an entry
 // (250 to 140 us a round with host-resident shards, which the copy bounds).  The
 // layout is for minibatches whose slabs all hold few entries and whose columns
-// have short runs (kEntryRegion, kEntryRun); skewed columns stay with the list
-// layout.
+// have short runs (kEntryRegion, kEntryRun, load_entries); skewed columns stay
+// with the list layout.
 #include <cuda_runtime.h>
 
 #include <cstdint>

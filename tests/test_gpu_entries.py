@@ -227,7 +227,7 @@ def test_missing_notify_and_the_rounds_after_it(N, d, max_len, sync):
 
 # Without streaming, the update and the products of the next step walk the slabs, a CTA each while one wave of CTAs
 # covers them (1,216 on a GB300), else a warp each: 489 and 1,368 slabs of 1,024 columns; the first slab's region
-# takes several passes of a warp, its runs are of up to 14 rows; the last slab is ragged.
+# takes several passes of a warp, the last, ragged one has runs of up to 14 rows.
 @pytest.mark.parametrize("residency", ["device", "host"])
 @pytest.mark.parametrize("d", [500001, 1400001])
 def test_updates_walk_the_slabs_one_by_one(d, residency):
@@ -236,8 +236,8 @@ def test_updates_walk_the_slabs_one_by_one(d, residency):
     rng = np.random.default_rng(4)
     for i in range(N):
         sh.col[i][sh.rowptr[i][1:] - 1] = np.where(rng.random(7 * B) < 0.3, d - 1, sh.col[i][sh.rowptr[i][1:] - 1])
-        sh.col[i][sh.rowptr[i][:-1]] = rng.integers(0, 8, 7 * B)          # eight columns, about four rows each
-        sh.col[i][sh.rowptr[i][:-1] + 1] = rng.integers(8, 1000, 7 * B)
+        sh.col[i][sh.rowptr[i][:-1]] = rng.integers(0, 24, 7 * B)         # 24 columns, one or two rows each
+        sh.col[i][sh.rowptr[i][:-1] + 1] = rng.integers(24, 1000, 7 * B)
     W0 = (0.1 * rng.standard_normal((N, d))).astype(np.float32)
     with _make(sh, N, 1, "ring", "logistic", B, lr, l2=l2, tau=tau, residency=residency) as ctx:
         layout = ctx.debug_shard_layout()
@@ -259,3 +259,19 @@ def test_few_entries_of_many_workers(N, d, B, row_len, entries):
     with _make(sh, N, 1, "ring", "logistic", B, 0.4, tau=2) as ctx:
         assert _uses_entries(ctx) == entries
         _check(ctx, sh, 1, B, "logistic", 0.4, rounds.graph_schedule("ring", N, 1), tau=2)
+
+
+# A hot column: the entries of a slab's long runs times the longest run, at most 6,000 (1,500 where there are more slabs
+# than one wave of CTAs walks), else the column lists
+@pytest.mark.parametrize("N,d,hot_rows,entries", [(5, 4000, 32, True), (6, 4000, 32, False), (22, 30000, 16, True),
+                                                  (24, 30000, 16, False), (5, 1400000, 16, True),
+                                                  (6, 1400000, 16, False), (24, 1400000, 3, True)])
+def test_hot_columns(N, d, hot_rows, entries):
+    B = 64
+    sh = inputs.sparse_custom(seed=N, N=N, d=d, rows=2 * B, lengths=[np.full(2 * B, 6)] * N)
+    for i in range(N):
+        first = sh.rowptr[i][:-1]
+        sh.col[i][first] = np.where(np.arange(2 * B) % B < hot_rows, 0, np.maximum(sh.col[i][first], 1))
+    with _make(sh, N, 1, "ring", "logistic", B, 0.4, tau=2) as ctx:
+        assert _uses_entries(ctx) == entries
+        _check(ctx, sh, 2, B, "logistic", 0.4, rounds.graph_schedule("ring", N, 1), tau=2)
