@@ -312,11 +312,16 @@ asap_status setup_mix(asap_ctx* c) {
   c->box_rows = ((N + c->n_boxes - 1) / c->n_boxes + 3) / 4 * 4;
   c->rows_pad = c->n_boxes * c->box_rows;
   // Slab: S columns of all rows, about 32 KB (8 <= S <= 1024, a power of 2);
-  // narrower, down to 128-byte rows, while that leaves SMs without two slabs:
-  // a small problem is one slab's latency, and its hottest slab's list.
+  // narrower, down to 128-byte rows, while half the SMs have none.  A small problem
+  // is one slab's latency; but every CTA costs its ticket and partial sums, and more
+  // than one slab each cost CTAs a second turn (N = 8, d = 10^4, k = 4, a row of
+  // reduces: 10 slabs 9.2 us, 79 7.5, 157 8.4, 313 9.4; d = 60,000: 59 slabs 9.3, 118
+  // 8.5, 235 8.8, 469 9.9; fused, N = 12, d = 30,000, hinge, 5 entries a row: 59 slabs
+  // 18.9, 118 19.4, 235 22.1, 469 24.1).  Long column lists call for narrower slabs
+  // (asap_load_shards).
   int S = 1024;
   while (S > 8 && static_cast<size_t>(c->rows_pad) * S * 4 > 32768) S >>= 1;
-  while (S > 32 && (c->ld + S - 1) / S < 2LL * c->sm_count) S >>= 1;
+  while (S > 32 && (c->ld + S - 1) / S < c->sm_count / 2) S >>= 1;
   int maxS = 8;
   while (static_cast<int64_t>(maxS) * 2 <= c->ld && maxS < 1024) maxS <<= 1;
   c->S = std::min(std::min(S, maxS), c->s_cap);
@@ -927,13 +932,23 @@ asap_status upload_blocks(asap_ctx* c, int nb, Img&& img) {
   return ASAP_OK;
 }
 
+// Whether slabs may be halved to shorten their lists: up to two slabs per SM, which
+// keep one in flight for each compute group.
+bool may_narrow(const asap_ctx* c) { return c->S > 32 && c->n_slabs < 2LL * c->sm_count; }
+
+asap_status narrow_slabs(asap_ctx* c) {
+  c->s_cap = c->S / 2;
+  return setup_mix(c);
+}
+
 // Builds and uploads the entry layout if the shards allow it (kEntryRegion,
-// kEntryRun, kEntryWaste); c->entries says whether it did.  c->nb is left to
-// the caller.
+// kEntryRun, kEntryWaste); c->entries says whether it did, *narrower whether it
+// might with narrower slabs.  c->nb is left to the caller.
 asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, const int32_t* const* col,
-                         const float* const* val, const float* const* y) {
+                         const float* const* val, const float* const* y, bool* narrower) {
   const int N = c->N, B = c->B;
   const int lS = __builtin_ctz(static_cast<unsigned>(c->S));
+  *narrower = false;
   // Longest row, most entries of a minibatch, and the longest slab region of
   // the first one, before anything is built.
   int64_t max_len = 0, max_nnz = 0;
@@ -950,7 +965,10 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   const int64_t stride = std::max<int64_t>(4, (max_len + 3) / 4 * 4);
   const int64_t table = static_cast<int64_t>(N) * B * stride;
   if (max_len > 65535 || table > kEntryWaste * max_nnz + 65536 || table >= (1ll << 31)) return ASAP_OK;
-  if (max_nnz > static_cast<int64_t>(kEntryRegion) * c->n_slabs) return ASAP_OK;
+  if (max_nnz > static_cast<int64_t>(kEntryRegion) * c->n_slabs) {
+    *narrower = true;
+    return ASAP_OK;
+  }
   // Few entries in slabs of many workers: the entry layout's reduce, one compute
   // group, mixes narrow slabs slower than the list layout's two, and what it saves
   // in the local step is little.  Speed of entries over lists, BSP and NOTIFY_ACK: N =
@@ -971,7 +989,10 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
     for (long long s = 0; s < c->n_slabs; ++s) {
       int64_t n = 0;
       for (int i = 0; i < N; ++i) n += cnt[static_cast<size_t>(s) * N + i];
-      if (n > kEntryRegion) return ASAP_OK;
+      if (n > kEntryRegion) {
+        *narrower = true;
+        return ASAP_OK;
+      }
     }
   }
   std::vector<EntryImage> built(nb);
@@ -982,10 +1003,14 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   int max_region = 0, max_run = 0, max_hot = 0;
   for (const EntryImage& im : built) {
     if (im.err) return fail(c, ASAP_ERR_ARG, im.err);
-    if (im.max_region > kEntryRegion || im.max_run > kEntryRun) return ASAP_OK;
+    if (im.max_run > kEntryRun) return ASAP_OK;
     max_region = std::max(max_region, im.max_region);
     max_run = std::max(max_run, im.max_run);
     max_hot = std::max(max_hot, im.max_hot);
+  }
+  if (max_region > kEntryRegion) {
+    *narrower = true;
+    return ASAP_OK;
   }
   // Hot columns: a run is added up one entry after the other, and the slab that
   // holds many long ones paces the launch, where a column list holds one item a
@@ -1026,6 +1051,39 @@ asap_status load_entries(asap_ctx* c, int nb, const int64_t* const* rowptr, cons
   const int64_t params = static_cast<int64_t>(N) * c->ld;
   c->stream_slabs = 24 * max_nnz >= params && params >= 16384;
   if (c->stream_slabs) CU(entry_step_configure(), "configuring the local update kernel");
+  return ASAP_OK;
+}
+
+// Column lists: slabs are narrowed while the longest list of the first minibatch
+// holds more than 1,500 items, distinct (worker, column) pairs.  RCV1-shaped, N =
+// 16, d = 47,236: 4,096 items at 256 columns, 2,048 at 128: a round 26.3 -> 25.2 us,
+// with two local steps 53.1 -> 48.1; N = 16, d = 30,000, 480,000 entries: 59 slabs
+// of 6,000 29.2, 118 of 3,000 26.7, 235 of 1,500 26.5, 469 28.3; N = 12, d = 100,000,
+// 360,000 entries, 196 slabs of 1,600 26.0 (two steps 50.9), 391 25.4 (47.9).
+asap_status narrow_for_lists(asap_ctx* c, const int64_t* const* rowptr, const int32_t* const* col) {
+  if (!may_narrow(c)) return ASAP_OK;
+  std::vector<int32_t> items(c->d, 0);   // workers with an entry in each column (few: d < 311,296)
+  std::vector<int> last(c->d, -1);
+  for (int i = 0; i < c->N; ++i) {
+    if (!rowptr[i]) continue;
+    for (int64_t e = rowptr[i][0]; e < rowptr[i][c->B]; ++e) {
+      const int32_t cc = col[i][e];
+      if (cc < 0 || cc >= c->d) return fail(c, ASAP_ERR_ARG, "column id out of range [0, d)");
+      items[cc] += last[cc] != i;
+      last[cc] = i;
+    }
+  }
+  while (may_narrow(c)) {
+    int64_t longest = 0;
+    for (int64_t c0 = 0; c0 < c->d; c0 += c->S) {
+      int64_t n = 0;
+      for (int64_t q = c0; q < std::min<int64_t>(c0 + c->S, c->d); ++q) n += items[q];
+      longest = std::max(longest, n);
+    }
+    if (longest <= 1500) break;
+    asap_status s = narrow_slabs(c);
+    if (s != ASAP_OK) return s;
+  }
   return ASAP_OK;
 }
 
@@ -1576,14 +1634,23 @@ asap_status asap_load_shards(asap_ctx* c, const int64_t* const* rowptr, const in
   c->s_cap = 1024;
   s0 = setup_mix(c);
   if (s0 != ASAP_OK) return s0;
-  s0 = load_entries(c, nb, rp_use.data(), col, val, y);
-  if (s0 != ASAP_OK) return s0;
+  for (bool narrower = true; narrower && !c->entries;) {
+    s0 = load_entries(c, nb, rp_use.data(), col, val, y, &narrower);
+    if (s0 != ASAP_OK) return s0;
+    narrower = narrower && may_narrow(c);
+    if (narrower && (s0 = narrow_slabs(c)) != ASAP_OK) return s0;
+  }
   c->wv_step = -1;
   c->configured_key = -1;
   if (c->entries) {
     c->nb = nb;
     return ASAP_OK;
   }
+  c->s_cap = 1024;
+  s0 = setup_mix(c);
+  if (s0 != ASAP_OK) return s0;
+  s0 = narrow_for_lists(c, rp_use.data(), col);
+  if (s0 != ASAP_OK) return s0;
   const int Q = c->step_q;
   // Build every minibatch's image; narrow the slabs and rebuild while a
   // slab's column list is too long for the fused reduce's shared memory.

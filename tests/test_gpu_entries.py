@@ -275,3 +275,16 @@ def test_hot_columns(N, d, hot_rows, entries):
     with _make(sh, N, 1, "ring", "logistic", B, 0.4, tau=2) as ctx:
         assert _uses_entries(ctx) == entries
         _check(ctx, sh, 2, B, "logistic", 0.4, rounds.graph_schedule("ring", N, 1), tau=2)
+
+
+# Slab widths of small problems: entries in slabs as wide as half the SMs allow; entries that fit 704 a region only in
+# narrower ones; column lists narrowed for their length, in two steps
+@pytest.mark.parametrize("N,d,B,row_len,hot,entries", [(12, 30000, 32, 10, False, True), (5, 100000, 64, 250, False, True),
+                                                       (16, 30000, 64, 300, True, False), (2, 9000, 40, 20, True, False)])
+def test_slab_widths_of_small_problems(N, d, B, row_len, hot, entries):
+    sh = inputs.sparse_custom(seed=B, N=N, d=d, rows=3 * B, lengths=[np.full(3 * B, row_len)] * N,
+                              **({"hot_col": 7} if hot else {}))
+    W0 = (0.1 * np.random.default_rng(5).standard_normal((N, d))).astype(np.float32)
+    with _make(sh, N, 1, "ring", "logistic", B, 0.3, l2=0.01, tau=2) as ctx:
+        assert _uses_entries(ctx) == entries
+        _check(ctx, sh, 2, B, "logistic", 0.3, rounds.graph_schedule("ring", N, 1), l2=0.01, tau=2, W0=W0)
